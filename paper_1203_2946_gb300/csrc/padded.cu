@@ -27,6 +27,7 @@
 
 #include "common.cuh"
 #include "scan.cuh"
+#include "stage.cuh"
 
 namespace cmrs {
 namespace {
@@ -65,79 +66,139 @@ __device__ __forceinline__ int row_span(int sa, int sb, int height, uint32_t mas
   return lane < height ? end - start : 0;
 }
 
-// Runs the plan of strip s and writes its passes from out0 on, at most
-// `limit` of them.  Returns false if the plan does not fit (a pass
-// overflowing, or more passes than `limit`), which a valid unsorted strip
-// never does; the writes stay inside the strip's limit either way.
-template <typename S, bool kSplit>
-__device__ bool pad_strip_fill(int sa, int sb, int height, int bits, int slots, long long limit,
-                               const uint32_t *__restrict__ packed, const S *__restrict__ vh,
-                               const S *__restrict__ vl, long long out0, uint32_t *__restrict__ pk_out,
-                               S *__restrict__ vo_h, S *__restrict__ vo_l) {
+// One pass of the plan in its general form, for the passes k_pad_fill's short
+// form does not cover: `left` items per row, C passes left (this one
+// included).  Writes the pass at out (32 items) and takes it off left and
+// next; returns false, with nothing written, if the pass would overflow
+// (never for a valid unsorted strip).
+template <typename S, bool kSplit, int kM>
+__device__ __forceinline__ bool pad_pass(int &left, int &next, int C, int height,
+                                         const uint32_t *__restrict__ cp, const S *__restrict__ vh,
+                                         const S *__restrict__ vl, uint32_t *__restrict__ pk_out,
+                                         S *__restrict__ vo_h, S *__restrict__ vo_l) {
   const int lane = threadIdx.x & 31;
-  const uint32_t mask = (1u << bits) - 1;
-  int next;
-  int left = row_span(sa, sb, height, mask, packed, lane, &next);
-  if (left < 0) left = 0;  // a corrupt strip: what is left unwritten is reported below
-  long long passes = 0;
-  for (;;) {
-    const int total = (int)__reduce_add_sync(kFull, (unsigned)left);
-    if (total == 0) break;
-    if (passes == limit) return false;
-    const int longest = (int)__reduce_max_sync(kFull, (unsigned)left);
-    const int C = max((total + 31) / 32, (longest + slots - 1) / slots);
-    int take = max(0, left - slots * (C - 1));
-    int room = 32 - (int)__reduce_add_sync(kFull, (unsigned)take);
-    if (room < 0) return false;
-    // free room: rows with most items left first, lower row on ties
-    const int want = min(left, slots) - take;
-    const int wanted = (int)__reduce_add_sync(kFull, (unsigned)max(want, 0));
-    int extra;
-    if (wanted <= room) {
-      extra = max(want, 0);  // every row gets what it wants
-    } else {
-      // before = the want of the rows ranked ahead (more items left, or as
-      // many and a lower row), one distinct count of items left at a time,
-      // largest first, until the free room is given out
-      const int lv = want > 0 ? left - take : 0;  // >= 1 for a row that wants
-      unsigned rem = __ballot_sync(kFull, want > 0);
-      int before = room, done = 0;
-      while (rem && done < room) {
-        const int v = (int)__reduce_max_sync(kFull, (rem >> lane) & 1u ? (unsigned)lv : 0u);
-        const unsigned g = __ballot_sync(kFull, ((rem >> lane) & 1u) && lv == v);
-        const int wg = (g >> lane) & 1u ? want : 0;
-        const int below = warp_excl_scan(wg, lane);  // want of the group's lower rows
-        if ((g >> lane) & 1u) before = done + below;
-        done += (int)__reduce_add_sync(kFull, (unsigned)wg);
-        rem &= ~g;
-      }
-      extra = want > 0 ? max(0, min(want, room - before)) : 0;
+  int take = max(0, left - kM * (C - 1));
+  int room = 32 - (int)__reduce_add_sync(kFull, (unsigned)take);
+  if (room < 0 || __any_sync(kFull, take > kM)) return false;
+  // free room: rows with most items left first, lower row on ties
+  const int want = min(left, kM) - take;
+  const int wanted = (int)__reduce_add_sync(kFull, (unsigned)max(want, 0));
+  int extra;
+  if (wanted <= room) {
+    extra = max(want, 0);  // every row gets what it wants
+  } else {
+    // before = the want of the rows ranked ahead (more items left, or as
+    // many and a lower row), one distinct count of items left at a time,
+    // largest first, until the free room is given out
+    const int lv = want > 0 ? left - take : 0;  // >= 1 for a row that wants
+    unsigned rem = __ballot_sync(kFull, want > 0);
+    int before = room, done = 0;
+    while (rem && done < room) {
+      const int v = (int)__reduce_max_sync(kFull, (rem >> lane) & 1u ? (unsigned)lv : 0u);
+      const unsigned g = __ballot_sync(kFull, ((rem >> lane) & 1u) && lv == v);
+      const int wg = (g >> lane) & 1u ? want : 0;
+      const int below = warp_excl_scan(wg, lane);  // want of the group's lower rows
+      if ((g >> lane) & 1u) before = done + below;
+      done += (int)__reduce_add_sync(kFull, (unsigned)wg);
+      rem &= ~g;
     }
-    take += extra;
-    room -= (int)__reduce_add_sync(kFull, (unsigned)extra);
-    // zero items: rows 0 upwards, each topped up to `slots`
-    const int zcap = lane < height ? slots - take : 0;
-    const int zero = max(0, min(zcap, room - warp_excl_scan(zcap, lane)));
-    const int len = take + zero;
-    const int off = warp_excl_scan(len, lane);
-    const long long base = out0 + passes * 32 + off;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {  // slots <= 8 items of a row per pass
-      if (j < take) {
-        pk_out[base + j] = packed[next + j];
-        vo_h[base + j] = vh[next + j];
-        if (kSplit) vo_l[base + j] = vl[next + j];
-      } else if (j < len) {
-        pk_out[base + j] = (uint32_t)lane;  // column 0, this row
-        vo_h[base + j] = S(0);
-        if (kSplit) vo_l[base + j] = S(0);
-      }
-    }
-    next += take;
-    left -= take;
-    ++passes;
+    extra = want > 0 ? max(0, min(want, room - before)) : 0;
   }
-  return passes == limit;
+  take += extra;
+  room -= (int)__reduce_add_sync(kFull, (unsigned)extra);
+  // zero items: rows 0 upwards, each topped up to M
+  const int zcap = lane < height ? kM - take : 0;
+  const int zero = max(0, min(zcap, room - warp_excl_scan(zcap, lane)));
+  const int len = take + zero;
+  const int off = warp_excl_scan(len, lane);
+#pragma unroll
+  for (int j = 0; j < kM; ++j) {
+    if (j < take) {
+      pk_out[off + j] = cp[next + j];
+      vo_h[off + j] = vh[next + j];
+      if (kSplit) vo_l[off + j] = vl[next + j];
+    } else if (j < len) {
+      pk_out[off + j] = (uint32_t)lane;  // column 0, this row
+      vo_h[off + j] = S(0);
+      if (kSplit) vo_l[off + j] = S(0);
+    }
+  }
+  next += take;
+  left -= take;
+  return true;
+}
+
+// Runs the plan of one strip and writes its `limit` passes from out0 on.  The
+// strip's items are cp[next..], lane r's row starting at `next` with `left`
+// items; map: this warp's 2 x 32 words of shared memory.
+//
+// The passes left are limit - p throughout (the plan takes exactly the
+// minimum, see the top of the file), so a pass needs neither the total nor
+// the longest row.  With t the items left such that rows above t all go and
+// rows at t go lowest first until 32 / M rows do, a pass with t >= M is
+// exactly those 32 / M rows, M items each, and no zero item: every chosen row
+// holds M items, and a forced row (left > M (C - 1)) ranks at M (C - 1), so
+// it goes in full whenever t lies below that, or no row is forced at all.  t
+// only falls from pass to pass, so it is found by stepping down from the last
+// pass's, a vote a step.  Lane j then reads item j % M of the (j / M)-th
+// chosen row, whose next item is passed through `map`, and the pass leaves by
+// one 32-word store per array.  On rows of 4..60 items (height 32, M = 2)
+// 94% of the passes take this form; 98 instructions a pass on average against
+// 430 when every pass ran the general form, and with the staged reads
+// k_pad_fill takes 316 us instead of 1,149 on 2,097,152 such rows (67M FP32
+// entries; reading and writing them once is 163 us).  What is left is bound
+// by the votes' latency at 20 warps per SM (the stage's shared memory).
+template <typename S, bool kSplit, int kM>
+__device__ __forceinline__ void pad_strip_fill(int left, int next, int height, long long limit, uint32_t *map,
+                                               const uint32_t *__restrict__ cp, const S *__restrict__ vh,
+                                               const S *__restrict__ vl, long long out0,
+                                               uint32_t *__restrict__ pk_out, S *__restrict__ vo_h,
+                                               S *__restrict__ vo_l) {
+  constexpr int K = 32 / kM;  // rows of a full pass
+  const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1;
+  uint32_t *po = pk_out + out0;
+  S *ho = vo_h + out0, *lo = kSplit ? vo_l + out0 : nullptr;
+  if (limit <= 0) return;
+  int t = (int)__reduce_max_sync(kFull, (unsigned)left);
+  po += lane;
+  ho += lane;
+  lo += kSplit ? lane : 0;
+  // passes left after this one (below 2^31 / 32).  The last pass never takes
+  // the short form: every item left is forced then.
+  for (int D = (int)limit - 1; D > 0; --D, po += 32, ho += 32, lo += kSplit ? 32 : 0) {
+    unsigned gt = __ballot_sync(kFull, left > t), ge = __ballot_sync(kFull, left >= t);
+    if (__popc(ge) < K) {
+      gt = ge;
+      ge = __ballot_sync(kFull, left >= --t);  // the next lower count, usually
+      while (__popc(ge) < K) {                 // ends: at t = 0 every lane votes
+        gt = ge;
+        t = (int)__reduce_max_sync(kFull, left < t ? (unsigned)left : 0u);
+        ge = __ballot_sync(kFull, left >= t);
+      }
+    }
+    if (t >= kM && (t < kM * D || !__any_sync(kFull, left > kM * D))) {
+      const bool sel = left > t || (left == t && __popc(ge & ~gt & lt) < K - __popc(gt));
+      const unsigned sm = __ballot_sync(kFull, sel);
+      uint32_t *mp = map + ((D & 1) << 5);  // alternate halves: one warp barrier a pass
+      if (sel) {
+        mp[__popc(sm & lt)] = (uint32_t)next;
+        next += kM;
+        left -= kM;
+      }
+      __syncwarp();
+      const int src = (int)mp[lane / kM] + (lane & (kM - 1));
+      *po = cp[src];
+      *ho = vh[src];
+      if (kSplit) *lo = vl[src];
+    } else {
+      __syncwarp();
+      if (!pad_pass<S, kSplit, kM>(left, next, D + 1, height, cp, vh, vl, po - lane, ho - lane,
+                                   kSplit ? lo - lane : nullptr))
+        return;
+    }
+  }
+  pad_pass<S, kSplit, kM>(left, next, 1, height, cp, vh, vl, po - lane, ho - lane, kSplit ? lo - lane : nullptr);
 }
 
 // Passes of each strip: max(ceil(T / 32), ceil(L / M)), 0 for an empty strip.
@@ -170,13 +231,12 @@ __global__ void __launch_bounds__(kPadWarps * 32) k_pad_count(int strips, int he
 // each lane copies its own row, kPadFillU passes' loads in flight.
 constexpr int kPadFillU = 8;
 template <typename S, bool kSplit>
-__device__ bool pad_strip_fill_m1(int sa, int sb, int bits, long long limit, const uint32_t *__restrict__ packed,
-                                  const S *__restrict__ vh, const S *__restrict__ vl, long long out0,
-                                  uint32_t *__restrict__ pk_out, S *__restrict__ vo_h, S *__restrict__ vo_l) {
+__device__ __forceinline__ void pad_strip_fill_m1(int left, int next, long long limit,
+                                                  const uint32_t *__restrict__ cp, const S *__restrict__ vh,
+                                                  const S *__restrict__ vl, long long out0,
+                                                  uint32_t *__restrict__ pk_out, S *__restrict__ vo_h,
+                                                  S *__restrict__ vo_l) {
   const int lane = threadIdx.x & 31;
-  int next;
-  int left = row_span(sa, sb, 32, (1u << bits) - 1, packed, lane, &next);
-  if (left < 0) left = 0;
   for (long long p = 0; p < limit; p += kPadFillU) {
     uint32_t c[kPadFillU];
     S h[kPadFillU], l[kPadFillU];
@@ -186,7 +246,7 @@ __device__ bool pad_strip_fill_m1(int sa, int sb, int bits, long long limit, con
       h[u] = S(0);
       l[u] = S(0);
       if (p + u < left) {
-        c[u] = packed[next + p + u];
+        c[u] = cp[next + p + u];
         h[u] = vh[next + p + u];
         if (kSplit) l[u] = vl[next + p + u];
       }
@@ -200,27 +260,89 @@ __device__ bool pad_strip_fill_m1(int sa, int sb, int bits, long long limit, con
         if (kSplit) vo_l[o] = l[u];
       }
   }
-  return __all_sync(kFull, left <= limit);
 }
 
-template <typename S, bool kSplit>
-__global__ void __launch_bounds__(kPadWarps * 32, 4) k_pad_fill(int strips, int height, int bits, int slots,
-                                                            const int32_t *__restrict__ sp,
-                                                            const uint32_t *__restrict__ packed,
-                                                            const S *__restrict__ vh, const S *__restrict__ vl,
-                                                            const int32_t *__restrict__ sp_out,
-                                                            uint32_t *__restrict__ pk_out, S *__restrict__ vo_h,
-                                                            S *__restrict__ vo_l) {
-  const int nw = gridDim.x * kPadWarps;
-  for (int s = blockIdx.x * kPadWarps + (threadIdx.x >> 5); s < strips; s += nw) {
+// Strip [sa, sb) whose item k is at cp[k - base].
+template <typename S, bool kSplit, int kM>
+__device__ __forceinline__ void pad_strip(int sa, int sb, int base, int height, int bits, long long limit,
+                                          uint32_t *map, const uint32_t *__restrict__ cp, const S *__restrict__ vh,
+                                          const S *__restrict__ vl, long long out0, uint32_t *__restrict__ pk_out,
+                                          S *__restrict__ vo_h, S *__restrict__ vo_l) {
+  int next;
+  int left = row_span(sa - base, sb - base, height, (1u << bits) - 1, cp, threadIdx.x & 31, &next);
+  if (left < 0) left = 0;  // a corrupt strip, which the layout pass reports
+  if constexpr (kM == 1)
+    pad_strip_fill_m1<S, kSplit>(left, next, limit, cp, vh, vl, out0, pk_out, vo_h, vo_l);
+  else
+    pad_strip_fill<S, kSplit, kM>(left, next, height, limit, map, cp, vh, vl, out0, pk_out, vo_h, vo_l);
+}
+
+// One strip per warp.  The strip's items are copied into the warp's own
+// shared-memory stage by one bulk copy per stream (the plan then reads them M
+// at a time from 32 / M rows, which from global memory touches as many lines
+// per load); a strip longer than the stage is read from global memory.  The
+// stage also serves the row-start searches.  Should a copy's bounded wait
+// give up, the warp reads this and its later strips from global memory, so
+// the result does not depend on it, and waits (bounded) once more before it
+// leaves.
+#ifndef CMRS_FILL_WARPS
+#define CMRS_FILL_WARPS 4
+#endif
+constexpr int kFillWarps = CMRS_FILL_WARPS;
+constexpr int kFillCap = 2048;  // most items per stage
+template <int DT, int kM>
+__global__ void __launch_bounds__(kFillWarps * 32) k_pad_fill(int strips, int height, int bits, int cap, int nnz,
+                                                             const int32_t *__restrict__ sp,
+                                                             const uint32_t *__restrict__ packed,
+                                                             const typename Form<DT>::Stored *__restrict__ vh,
+                                                             const typename Form<DT>::Stored *__restrict__ vl,
+                                                             const int32_t *__restrict__ sp_out,
+                                                             uint32_t *__restrict__ pk_out,
+                                                             typename Form<DT>::Stored *__restrict__ vo_h,
+                                                             typename Form<DT>::Stored *__restrict__ vo_l) {
+  typedef typename Form<DT>::Stored S;
+  constexpr bool kSplit = DT == CMRS_BF16X2;
+  extern __shared__ __align__(128) char smem[];
+  __shared__ uint64_t bars[kFillWarps];
+  __shared__ StageInfo info[kFillWarps];
+  __shared__ uint32_t maps[kFillWarps][64];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  char *stg = smem + (size_t)w * (cap ? Stage<DT>::bytes(cap) : 0);
+  if (lane == 0) {
+    mbar_init(&bars[w], 1);
+    fence_barrier_init();
+  }
+  __syncwarp();
+  uint64_t pol = 0;
+  if (lane == 0) pol = policy_evict_first();
+  uint32_t phase = 0;
+  bool stages = cap > 0;
+  const int nw = gridDim.x * kFillWarps;
+  for (int s = blockIdx.x * kFillWarps + w; s < strips; s += nw) {
+    const int sa = sp[s], sb = sp[s + 1];
+    bool staged = stages && sb > sa && sb - sa <= cap;
+    if (staged && lane == 0) issue_stage<DT>(sa, sb, nnz, packed, vh, vl, stg, cap, &bars[w], pol, &info[w]);
     const long long o0 = sp_out[s], o1 = sp_out[s + 1];
     const long long limit = o1 > o0 ? (o1 - o0) / 32 : 0;
-    if (slots == 1)
-      pad_strip_fill_m1<S, kSplit>(sp[s], sp[s + 1], bits, limit, packed, vh, vl, o0, pk_out, vo_h, vo_l);
-    else
-      pad_strip_fill<S, kSplit>(sp[s], sp[s + 1], height, bits, slots, limit, packed, vh, vl, o0, pk_out, vo_h,
-                                vo_l);
+    if (staged) {
+      if (__all_sync(kFull, mbar_wait_bounded(&bars[w], phase))) {
+        phase ^= 1;
+      } else {
+        staged = stages = false;
+      }
+    }
+    // compiled twice, so that the staged walk's reads are shared-memory loads
+    if (staged) {
+      const char *sh = stg + Stage<DT>::colp_bytes(cap);
+      pad_strip<S, kSplit, kM>(sa, sb, (int)info[w].a8, height, bits, limit, maps[w],
+                               reinterpret_cast<const uint32_t *>(stg), reinterpret_cast<const S *>(sh),
+                               reinterpret_cast<const S *>(sh + Stage<DT>::val_bytes(cap)), o0, pk_out, vo_h, vo_l);
+    } else {
+      pad_strip<S, kSplit, kM>(sa, sb, 0, height, bits, limit, maps[w], packed, vh, vl, o0, pk_out, vo_h, vo_l);
+    }
+    __syncwarp();  // every lane is done with the stage before the next copy lands in it
   }
+  if (cap > 0 && !stages) mbar_wait_bounded(&bars[w], phase);  // the late copy lands before the warp leaves
 }
 
 size_t pad_ws_bytes(int strips) { return 256 + scan_ws_bytes(strips); }
@@ -253,18 +375,42 @@ int pad_grid(int strips) {
   return (int)std::min<long long>(ceil_div(strips, kPadWarps), (long long)sms * 8);
 }
 
-template <typename S, bool kSplit>
-int launch_fill(const cmrs_matrix *A, int slots, const int32_t *sp_out, int nnz_padded, uint32_t *pk_out,
-                void *val_out, cudaStream_t st) {
+template <int DT, int kM>
+int launch_fill_m(const cmrs_matrix *A, const int32_t *sp_out, int nnz_padded, uint32_t *pk_out, void *val_out,
+                  cudaStream_t st) {
+  typedef typename Form<DT>::Stored S;
+  constexpr bool kSplit = DT == CMRS_BF16X2;
   const S *vh = reinterpret_cast<const S *>(A->val);
   const S *vl = kSplit ? vh + cmrs_pad8(A->nnz) : nullptr;
   S *oh = reinterpret_cast<S *>(val_out);
   S *ol = kSplit ? oh + cmrs_pad8(nnz_padded) : nullptr;
-  k_pad_fill<S, kSplit><<<pad_grid(A->strips), kPadWarps * 32, 0, st>>>(A->strips, A->height, A->bits, slots,
-                                                                        A->strip_ptr, A->col_packed, vh, vl, sp_out,
-                                                                        pk_out, oh, ol);
+  // stage: 1.25x an average strip, so that most strips fit and short ones
+  // leave shared memory for more warps; none where the arrays' alignment does
+  // not allow bulk copies
+  const bool aligned = ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) == 0;
+  const long long avg = A->nnz / A->strips;
+  const int cap = aligned ? (int)std::min<long long>(kFillCap, (avg + avg / 4) / 32 * 32 + 64) : 0;
+  const size_t smem = cap ? (size_t)kFillWarps * Stage<DT>::bytes(cap) : 0;
+  const size_t smem_max = (size_t)kFillWarps * Stage<DT>::bytes(kFillCap);
+  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_pad_fill<DT, kM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+  int per_sm = 0;
+  CMRS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pad_fill<DT, kM>, kFillWarps * 32, smem));
+  const int grid = (int)std::min<long long>(ceil_div(A->strips, kFillWarps), (long long)std::max(1, per_sm) * sm_count());
+  k_pad_fill<DT, kM><<<grid, kFillWarps * 32, smem, st>>>(A->strips, A->height, A->bits, cap, A->nnz, A->strip_ptr,
+                                                          A->col_packed, vh, vl, sp_out, pk_out, oh, ol);
   CMRS_LAUNCH_CHECK();
   return CMRS_OK;
+}
+
+template <int DT>
+int launch_fill(const cmrs_matrix *A, int slots, const int32_t *sp_out, int nnz_padded, uint32_t *pk_out,
+                void *val_out, cudaStream_t st) {
+  switch (slots) {
+    case 1: return launch_fill_m<DT, 1>(A, sp_out, nnz_padded, pk_out, val_out, st);
+    case 2: return launch_fill_m<DT, 2>(A, sp_out, nnz_padded, pk_out, val_out, st);
+    case 4: return launch_fill_m<DT, 4>(A, sp_out, nnz_padded, pk_out, val_out, st);
+    default: return launch_fill_m<DT, 8>(A, sp_out, nnz_padded, pk_out, val_out, st);
+  }
 }
 
 }  // namespace
@@ -327,10 +473,10 @@ extern "C" int cmrs_pad_fill(const cmrs_matrix *A, int slots, const int32_t *str
   cudaStream_t st = as_stream(stream);
   if (A->strips > 0 && nnz_padded > 0) {
     switch (A->dtype) {
-      case CMRS_F64: rc = launch_fill<double, false>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
-      case CMRS_F32: rc = launch_fill<float, false>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
-      case CMRS_BF16: rc = launch_fill<uint16_t, false>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
-      default: rc = launch_fill<uint16_t, true>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
+      case CMRS_F64: rc = launch_fill<CMRS_F64>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
+      case CMRS_F32: rc = launch_fill<CMRS_F32>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
+      case CMRS_BF16: rc = launch_fill<CMRS_BF16>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
+      default: rc = launch_fill<CMRS_BF16X2>(A, slots, strip_ptr_padded, nnz_padded, col_packed_out, val_out, st); break;
     }
     if (rc) return rc;
   }
