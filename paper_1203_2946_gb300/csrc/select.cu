@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "stage.cuh"
 
 namespace cmrs {
 namespace {
@@ -25,48 +26,175 @@ struct FeatAcc {
   // modified CMRS items at (32, 1), (32, 2), (16, 8); entries in rows of
   // >= 32, 512, 8192; sum of squares and max of 32-row strip entry counts
   unsigned long long pad[3], elong[3], s32_sq, s32_max;
+  unsigned long long done;  // blocks finished
 };
 
 __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
-  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+// Features.  A warp takes 32 consecutive rows at a time, lane r row r: its
+// bounds, its length statistics and its entries.  The rows' column indices are
+// one contiguous range, which one bulk copy brings into the warp's
+// shared-memory stage; each lane then walks its own row there, |col - row| and
+// min / max in registers, no shuffle per entry (the furthest column of a row
+// is its min or its max).  A range longer than the stage (or an array that is
+// not 16-byte aligned) is read from global memory: a lane per row for rows of
+// up to kFeatShort entries, the whole warp for longer ones.  The strips of
+// every height h = 2^e <= 32 are aligned groups of h lanes, so a shuffle tree
+// over the rows' min and max gives each strip's column spread in the same
+// pass, and one over the row lengths each 32- and 16-row strip's entry count
+// and longest row (the modified CMRS pass counts).  A group with an invalid
+// RowPtr range is skipped.  The last block to finish computes the features, so
+// there is no second launch.  16M entries in rows of 20..60: 41 us for all 32
+// features; with one entry of the contiguous range per lane (an entry then
+// finds its row by a five-step shuffle search and joins its row's min / max in
+// a five-step scan: 69M warp instructions, here 17M) and a second kernel for
+// the features, 153 us.  Reading the columns once is 10 us; what is left is
+// each group's copy round trip and the walk's shared-memory reads.
+constexpr int kFeatU = 4;        // loads in flight per lane
+constexpr int kFeatShort = 64;   // unstaged rows up to this length: a lane each
+constexpr int kFeatCap = 2048;   // most entries per stage
+constexpr int kFeatThreads = 256;
+
+// Entries first, first + step, ... of a row of len entries at c[0..]: whole
+// batches of kFeatU without a guard, then one at a time.
+__device__ __forceinline__ void feat_entries(const int32_t *__restrict__ c, unsigned first, unsigned step, unsigned len,
+                                             int row, int &lo, int &hi, unsigned long long &sd, unsigned &near) {
+  auto one = [&](int v) {
+    // |v - row| of any two ints fits 32 unsigned bits
+    const unsigned ad = (unsigned)max(v, row) - (unsigned)min(v, row);
+    sd += ad;
+    near += ad <= 64u;
+    lo = min(lo, v);
+    hi = max(hi, v);
+  };
+  unsigned k = first;
+  for (; k + step * (kFeatU - 1) < len; k += step * kFeatU) {
+    int v[kFeatU];
+#pragma unroll
+    for (int u = 0; u < kFeatU; ++u) v[u] = c[k + step * u];
+#pragma unroll
+    for (int u = 0; u < kFeatU; ++u) one(v[u]);
+  }
+  for (; k < len; k += step) one(c[k]);
 }
 
-// Row length statistics, |col - row| statistics and each row's min/max
-// column (for the strip spreads).  A warp takes 32 consecutive rows at a
-// time: lane r holds row r's bounds and length statistics; the rows' entries
-// are one contiguous range, read in coalesced batches of 32 (kFeatU in
-// flight per lane); an entry finds its row among the 32 row starts by a
-// five-step shuffle search, adds its |col - row| to sums over all entries,
-// and a segmented shuffle scan over the batch gives each row's min and max,
-// which the row's lane carries over batches.  The strips of every height
-// h = 2^e <= 32 are aligned groups of h lanes, so a shuffle tree over the
-// rows' min and max gives each strip's column spread in the same pass, and
-// one over the row lengths each 32- and 16-row strip's entry count and
-// longest row (the modified CMRS pass counts).  A group with an invalid
-// RowPtr range is skipped.
-constexpr int kFeatU = 4;
-__global__ void k_feat_rows(int rows, int nnz, const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
-                            FeatAcc *acc) {
-  __shared__ unsigned long long s[23], s_spread[6], s_ne[6];
-  if (threadIdx.x < 23) s[threadIdx.x] = 0;
-  if (threadIdx.x < 6) {
-    s_spread[threadIdx.x] = 0;
-    s_ne[threadIdx.x] = 0;
+// The features from the integer sums, with the same operations, in the same
+// order, as their definition (no contraction into FMAs); thread t computes
+// feature t.  Every division, root and logarithm is written once and shared by
+// the features that need it: a branch per feature runs them one after another
+// (20 us for the 32 features; FP64 issues one warp instruction in 16 cycles).
+__device__ __forceinline__ void feat_final(int t, int rows, int nnz, const volatile FeatAcc *acc, double *f) {
+  const double n = (double)rows, z = (double)nnz;
+  const double ns = (double)((rows + 31) / 32);
+  // mean row length; mean entries of a 32-row strip
+  const double mean = __ddiv_rn(z, t >= 30 ? ns : n);
+  const double mean1 = mean > 1.0 ? mean : 1.0;
+  unsigned long long num = 0;
+  double den = 1.0;  // dividing by 1 is exact
+  bool plus1 = false, lg = false;
+  if (t == 3) {
+    num = acc->sum_l2;
+    den = n;
+  } else if (t == 4) {
+    num = acc->max_l;
+    plus1 = lg = true;
+  } else if (t == 5) {
+    num = acc->empty;
+    den = n;
+  } else if (t >= 6 && t < 14) {
+    num = acc->bins[t - 6];
+    den = n;
+  } else if (t == 14) {
+    if (nnz > 0) {
+      num = acc->sum_d;
+      den = z;
+    }
+    plus1 = lg = true;
+  } else if (t == 15) {
+    num = acc->max_d;
+    plus1 = lg = true;
+  } else if (t == 16) {
+    if (nnz > 0) {
+      num = acc->near;
+      den = z;
+    }
+  } else if (t == 17) {
+    if (rows > 1) {
+      num = acc->same;
+      den = (double)(rows - 1);
+    }
+  } else if (t >= 18 && t < 24) {
+    const unsigned long long ne = acc->nonempty[t - 18];
+    if (ne > 0) {
+      num = acc->spread[t - 18];
+      den = (double)ne;
+    }
+    plus1 = lg = true;
+  } else if (t >= 24 && t < 27) {
+    num = nnz > 0 ? acc->pad[t - 24] : 1ull;  // log2(1) = 0 for an empty matrix
+    den = nnz > 0 ? z : 1.0;
+    lg = true;
+  } else if (t >= 27 && t < 30) {
+    if (nnz > 0) {
+      num = acc->elong[t - 27];
+      den = z;
+    }
+  } else if (t == 30) {
+    num = acc->s32_sq;
+    den = ns;
+  } else if (t == 31) {
+    num = acc->s32_max;
+    den = mean1;
+    plus1 = lg = true;
+  }
+  double q = __ddiv_rn((double)num, den);
+  if (t == 3 || t == 30) {  // spread of the lengths over their mean
+    double var = __dsub_rn(q, __dmul_rn(mean, mean));
+    if (var < 0.0) var = 0.0;
+    q = __ddiv_rn(sqrt(var), mean1);
+  }
+  if (t == 0) q = n;
+  if (t == 1) q = z > 1.0 ? z : 1.0;
+  if (t == 2) q = mean;
+  if (t == 2) plus1 = true;
+  if (plus1) q = __dadd_rn(1.0, q);
+  if (lg || t < 3) q = log2(q);
+  f[t] = q;
+}
+
+__global__ void __launch_bounds__(kFeatThreads, 4) k_feat_rows(int rows, int nnz, int cap,
+                                                               const int32_t *__restrict__ rp,
+                                                               const int32_t *__restrict__ ci, FeatAcc *acc,
+                                                               double *__restrict__ feat) {
+  extern __shared__ __align__(128) char smem[];
+  __shared__ uint64_t bars[kFeatThreads / 32];
+  __shared__ unsigned long long s[35];
+  __shared__ unsigned s_bins[9];  // rows by length: [2^q, 2^(q+1)) for q < 7, [128, ..), empty
+  __shared__ bool s_last;
+  for (int i = threadIdx.x; i < 35; i += kFeatThreads) s[i] = 0;
+  if (threadIdx.x < 9) s_bins[threadIdx.x] = 0;
+  const int w = threadIdx.x >> 5;
+  int32_t *stg = reinterpret_cast<int32_t *>(smem) + (size_t)w * (cap + 8);
+  if ((threadIdx.x & 31) == 0) {
+    mbar_init(&bars[w], 1);
+    fence_barrier_init();
   }
   __syncthreads();
+  uint64_t pol = 0;
+  if ((threadIdx.x & 31) == 0) pol = policy_evict_first();
+  uint32_t phase = 0;
+  bool stages = cap > 0;
   const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+  const long long nw = ((long long)gridDim.x * kFeatThreads) >> 5;
   const long long groups = ((long long)rows + 31) / 32;
-  unsigned long long l2 = 0, mxl = 0, empty = 0, same = 0, near = 0, sd = 0, mxd = 0;
-  unsigned long long bins[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  unsigned long long pad1 = 0, pad2 = 0, pad8 = 0, e32 = 0, e512 = 0, e8192 = 0, ssq = 0, smx = 0;
-  for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < groups; g += nw) {
+  unsigned long long l2 = 0, sd = 0, e32 = 0, e512 = 0, e8192 = 0, pad1 = 0, pad2 = 0, pad8 = 0, ssq = 0;
+  unsigned long long spread[6] = {0, 0, 0, 0, 0, 0};
+  unsigned mxl = 0, mxd = 0, smx = 0, same = 0, near = 0;  // counts of rows or entries: below 2^31
+  unsigned nonempty = 0;                                   // lane e: strips of height 2^e with entries
+  for (long long g = ((long long)blockIdx.x * kFeatThreads + threadIdx.x) >> 5; g < groups; g += nw) {
     const long long r0 = g * 32, r = r0 + lane;
     const int nrows = (int)min(32LL, (long long)rows - r0);
     const int start = r < rows ? rp[r] : 0;
@@ -75,226 +203,126 @@ __global__ void k_feat_rows(int rows, int nnz, const int32_t *__restrict__ rp, c
     if (lane == 31 || r + 1 >= rows) end = last;
     const bool ok = lane >= nrows || (start >= 0 && end >= start && end <= nnz);
     if (!__all_sync(kAll, ok)) continue;
+    const int e0 = __shfl_sync(kAll, start, 0);
+    bool staged = stages && last > e0 && last - e0 <= cap;
+    if (staged && lane == 0) issue_words(e0, last, nnz, ci, stg, &bars[w], pol);
     // row lengths (lane r)
-    const int len = end - start;
+    const int len = lane < nrows ? end - start : 0;
     int lprev = __shfl_up_sync(kAll, len, 1);
     if (lane == 0) lprev = r0 > 0 ? start - rp[r0 - 1] : -1;
     if (lane < nrows) {
-      const unsigned long long l = (unsigned long long)len;
-      l2 += l * l;
-      mxl = max(mxl, l);
-      empty += l == 0;
-      if (r > 0 && len == lprev) same++;
-      if (l >= 1) {
-        int bb = 0;
-        while (bb < 7 && l >= (2ull << bb)) ++bb;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) bins[q] += q == bb;  // registers, not a local array
-      }
-      e32 += l >= 32 ? l : 0ull;
-      e512 += l >= 512 ? l : 0ull;
-      e8192 += l >= 8192 ? l : 0ull;
+      l2 += (unsigned long long)len * (unsigned)len;
+      mxl = max(mxl, (unsigned)len);
+      same += r > 0 && len == lprev;
+      atomicAdd(&s_bins[len > 0 ? min(7, 31 - __clz(len)) : 8], 1u);
+      e32 += len >= 32 ? len : 0;
+      e512 += len >= 512 ? len : 0;
+      e8192 += len >= 8192 ? len : 0;
     }
     // this group is strip g of height 32 and strips 2g, 2g+1 of height 16:
     // entries and longest row of each, by a shuffle tree over the lanes
     {
-      unsigned long long ns = lane < nrows ? (unsigned long long)len : 0ull, ms = ns;
+      unsigned ns = (unsigned)len, ms = ns;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        if (o == 16 && (lane & 15) == 0) {  // the 16-row strips, before their halves meet
-          const unsigned long long c = max((ns + 31) / 32, (ms + 7) / 8);
-          pad8 += 32 * c;
-        }
+        if (o == 16 && (lane & 15) == 0)  // the 16-row strips, before their halves meet
+          pad8 += 32ull * max((ns + 31) / 32, (ms + 7) / 8);
         ns += __shfl_xor_sync(kAll, ns, o);
         ms = max(ms, __shfl_xor_sync(kAll, ms, o));
       }
       if (lane == 0) {
-        pad1 += 32 * ms;
-        pad2 += 32 * max((ns + 31) / 32, (ms + 1) / 2);
-        ssq += ns * ns;
+        pad1 += 32ull * ms;
+        pad2 += 32ull * max((ns + 31) / 32, (ms + 1) / 2);
+        ssq += (unsigned long long)ns * ns;
         smx = max(smx, ns);
       }
     }
-    // entries
-    const int key = lane < nrows ? start : last;  // rows past the matrix sort last
-    const int e0 = __shfl_sync(kAll, start, 0);
-    int lo = INT32_MAX, hi = -1;  // row `lane`'s min and max column
-    for (int k0 = e0; k0 < last; k0 += 32 * kFeatU) {
-      int c[kFeatU];
-#pragma unroll
-      for (int u = 0; u < kFeatU; ++u) {
-        const int k = k0 + 32 * u + lane;
-        c[u] = k < last ? ci[k] : 0;
-      }
-#pragma unroll
-      for (int u = 0; u < kFeatU; ++u) {
-        const int kb = k0 + 32 * u;  // first entry of this batch
-        if (kb >= last) break;       // warp-uniform
-        const int k = kb + lane;
-        const bool valid = k < last;
-        int j = 0;  // row of entry k: the last of the group's rows starting at or before k
-#pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-          const int sj = __shfl_sync(kAll, key, j + step);
-          if (sj <= k) j += step;
-        }
-        if (valid) {
-          const long long d = (long long)c[u] - (r0 + j);
-          const unsigned long long ad = (unsigned long long)(d < 0 ? -d : d);
-          sd += ad;
-          mxd = max(mxd, ad);
-          near += ad <= 64 ? 1ull : 0ull;
-        }
-        // min / max over the lanes of the same row in this batch
-        const int seg = max(__shfl_sync(kAll, key, j), kb) - kb;  // first lane of row j in the batch
-        int vmin = valid ? c[u] : INT32_MAX, vmax = valid ? c[u] : -1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int tmin = __shfl_up_sync(kAll, vmin, o), tmax = __shfl_up_sync(kAll, vmax, o);
-          if (lane - o >= seg) {
-            vmin = min(vmin, tmin);
-            vmax = max(vmax, tmax);
-          }
-        }
-        // row `lane` takes the scan at its last entry in the batch
-        const int my_e = min(end, kb + 32) - kb - 1;
-        const bool mine = lane < nrows && max(start, kb) - kb <= my_e;
-        const int m1 = __shfl_sync(kAll, vmin, mine ? my_e : 0), m2 = __shfl_sync(kAll, vmax, mine ? my_e : 0);
-        if (mine) {
-          lo = min(lo, m1);
-          hi = max(hi, m2);
+    // entries: lo, hi become row `lane`'s min and max column
+    int lo = INT32_MAX, hi = -1;
+    if (staged) {
+      if (__all_sync(kAll, mbar_wait_bounded(&bars[w], phase))) phase ^= 1;
+      else staged = stages = false;  // read from global memory from here on; the late copy is waited for below
+    }
+    if (staged) {
+      feat_entries(stg + (start - (e0 & ~3)), 0, 1, (unsigned)len, (int)r, lo, hi, sd, near);
+      __syncwarp();  // every lane is done with the stage before the next copy lands in it
+    } else {
+      if (len <= kFeatShort) feat_entries(ci + start, 0, 1, (unsigned)len, (int)r, lo, hi, sd, near);
+      for (unsigned m = __ballot_sync(kAll, len > kFeatShort); m; m &= m - 1) {
+        const int src = __ffs(m) - 1;
+        const int ks = __shfl_sync(kAll, start, src), kl = __shfl_sync(kAll, len, src);
+        int a = INT32_MAX, b = -1;
+        feat_entries(ci + ks, lane, 32, (unsigned)kl, (int)(r0 + src), a, b, sd, near);
+        a = __reduce_min_sync(kAll, a);
+        b = __reduce_max_sync(kAll, b);
+        if (lane == src) {
+          lo = a;
+          hi = b;
         }
       }
     }
+    if (len > 0)
+      mxd = max(mxd, max((unsigned)max(hi, (int)r) - (unsigned)min(hi, (int)r),
+                         (unsigned)max(lo, (int)r) - (unsigned)min(lo, (int)r)));
     // strip spreads: after step e each lane holds the min and max of its
     // aligned group of 2^e rows (rows past the matrix, and empty rows, are
     // neutral); the group's first lane counts the strip if it has entries
-    int slo = lane < nrows ? lo : INT32_MAX, shi = lane < nrows ? hi : -1;
 #pragma unroll
     for (int e = 0; e < 6; ++e) {
       if (e > 0) {
-        slo = min(slo, __shfl_xor_sync(kAll, slo, 1 << (e - 1)));
-        shi = max(shi, __shfl_xor_sync(kAll, shi, 1 << (e - 1)));
+        lo = min(lo, __shfl_xor_sync(kAll, lo, 1 << (e - 1)));
+        hi = max(hi, __shfl_xor_sync(kAll, hi, 1 << (e - 1)));
       }
-      const bool counted = (lane & ((1 << e) - 1)) == 0 && shi >= 0;
-      const unsigned long long sp = warp_sum(counted ? (unsigned long long)(shi - slo) : 0ull);
-      const unsigned long long ne = warp_sum(counted ? 1ull : 0ull);
-      if (lane == 0 && ne) {
-        atomicAdd(&s_spread[e], sp);
-        atomicAdd(&s_ne[e], ne);
-      }
+      const bool counted = (lane & ((1 << e) - 1)) == 0 && hi >= 0;
+      spread[e] += counted ? (unsigned)(hi - lo) : 0u;
+      const unsigned c = __popc(__ballot_sync(kAll, counted));
+      if (lane == e) nonempty += c;
     }
   }
-  l2 = warp_sum(l2);
-  mxl = warp_max(mxl);
-  empty = warp_sum(empty);
-  same = warp_sum(same);
-  near = warp_sum(near);
-  sd = warp_sum(sd);
-  mxd = warp_max(mxd);
-  for (int bb = 0; bb < 8; ++bb) bins[bb] = warp_sum(bins[bb]);
-  pad1 = warp_sum(pad1);
-  pad2 = warp_sum(pad2);
-  pad8 = warp_sum(pad8);
-  e32 = warp_sum(e32);
-  e512 = warp_sum(e512);
-  e8192 = warp_sum(e8192);
-  ssq = warp_sum(ssq);
-  smx = warp_max(smx);
-  if (lane == 0) {
-    atomicAdd(&s[0], l2);
-    atomicMax(&s[1], mxl);
-    atomicAdd(&s[2], empty);
-    atomicAdd(&s[3], same);
-    atomicAdd(&s[4], near);
-    atomicAdd(&s[5], sd);
-    atomicMax(&s[6], mxd);
-    for (int bb = 0; bb < 8; ++bb) atomicAdd(&s[7 + bb], bins[bb]);
-    atomicAdd(&s[15], pad1);
-    atomicAdd(&s[16], pad2);
-    atomicAdd(&s[17], pad8);
-    atomicAdd(&s[18], e32);
-    atomicAdd(&s[19], e512);
-    atomicAdd(&s[20], e8192);
-    atomicAdd(&s[21], ssq);
-    atomicMax(&s[22], smx);
+  if (cap > 0 && !stages) mbar_wait_bounded(&bars[w], phase);
+  // joined per warp, per block and over the blocks; the order does not matter
+  auto add = [&](int i, unsigned long long v) {
+    v = warp_sum(v);
+    if (lane == 0 && v) atomicAdd(&s[i], v);
+  };
+  auto top = [&](int i, unsigned v) {
+    v = __reduce_max_sync(kAll, v);
+    if (lane == 0) atomicMax(&s[i], (unsigned long long)v);
+  };
+  add(0, l2);
+  top(1, mxl);
+  add(3, same);
+  add(4, near);
+  add(5, sd);
+  top(6, mxd);
+#pragma unroll
+  for (int e = 0; e < 6; ++e) add(15 + e, spread[e]);
+  if (lane < 6) atomicAdd(&s[21 + lane], (unsigned long long)nonempty);
+  add(27, pad1);
+  add(28, pad2);
+  add(29, pad8);
+  add(30, e32);
+  add(31, e512);
+  add(32, e8192);
+  add(33, ssq);
+  top(34, smx);
+  __syncthreads();
+  if (threadIdx.x < 9) s[threadIdx.x < 8 ? 7 + threadIdx.x : 2] = s_bins[threadIdx.x];
+  __syncthreads();
+  // s[] is laid out as FeatAcc's sums are
+  unsigned long long *sums = reinterpret_cast<unsigned long long *>(acc);
+  if (threadIdx.x < 35) {
+    const unsigned long long v = s[threadIdx.x];
+    if (threadIdx.x == 1 || threadIdx.x == 6 || threadIdx.x == 34) atomicMax(&sums[threadIdx.x], v);
+    else if (v) atomicAdd(&sums[threadIdx.x], v);
+    __threadfence();
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    atomicAdd(&acc->sum_l2, s[0]);
-    atomicMax(&acc->max_l, s[1]);
-    atomicAdd(&acc->empty, s[2]);
-    atomicAdd(&acc->same, s[3]);
-    atomicAdd(&acc->near, s[4]);
-    atomicAdd(&acc->sum_d, s[5]);
-    atomicMax(&acc->max_d, s[6]);
-    for (int bb = 0; bb < 8; ++bb) atomicAdd(&acc->bins[bb], s[7 + bb]);
-    for (int q = 0; q < 3; ++q) {
-      atomicAdd(&acc->pad[q], s[15 + q]);
-      atomicAdd(&acc->elong[q], s[18 + q]);
-    }
-    atomicAdd(&acc->s32_sq, s[21]);
-    atomicMax(&acc->s32_max, s[22]);
-  }
-  if (threadIdx.x < 6) {
-    atomicAdd(&acc->spread[threadIdx.x], s_spread[threadIdx.x]);
-    atomicAdd(&acc->nonempty[threadIdx.x], s_ne[threadIdx.x]);
-  }
-}
-
-// The 32 features from the integer sums, with the same operations, in the
-// same order, as their definition (no contraction into FMAs); thread t
-// computes feature t.
-__global__ void k_feat_final(int rows, int nnz, const FeatAcc *acc, double *f) {
-  const int t = threadIdx.x;
-  if (blockIdx.x != 0 || t >= kNFeat) return;
-  const double n = (double)rows, z = (double)nnz;
-  const double mu = __ddiv_rn(z, n);
-  double v;
-  if (t == 0) {
-    v = log2(n);
-  } else if (t == 1) {
-    v = log2(z > 1.0 ? z : 1.0);
-  } else if (t == 2) {
-    v = log2(__dadd_rn(1.0, mu));
-  } else if (t == 3) {
-    double var = __dsub_rn(__ddiv_rn((double)acc->sum_l2, n), __dmul_rn(mu, mu));
-    if (var < 0.0) var = 0.0;
-    v = __ddiv_rn(sqrt(var), mu > 1.0 ? mu : 1.0);
-  } else if (t == 4) {
-    v = log2(__dadd_rn(1.0, (double)acc->max_l));
-  } else if (t == 5) {
-    v = __ddiv_rn((double)acc->empty, n);
-  } else if (t < 14) {
-    v = __ddiv_rn((double)acc->bins[t - 6], n);
-  } else if (t == 14) {
-    v = log2(__dadd_rn(1.0, nnz > 0 ? __ddiv_rn((double)acc->sum_d, z) : 0.0));
-  } else if (t == 15) {
-    v = log2(__dadd_rn(1.0, (double)acc->max_d));
-  } else if (t == 16) {
-    v = nnz > 0 ? __ddiv_rn((double)acc->near, z) : 0.0;
-  } else if (t == 17) {
-    v = rows > 1 ? __ddiv_rn((double)acc->same, (double)(rows - 1)) : 0.0;
-  } else if (t < 24) {
-    const double ne = (double)acc->nonempty[t - 18];
-    v = log2(__dadd_rn(1.0, ne > 0 ? __ddiv_rn((double)acc->spread[t - 18], ne) : 0.0));
-  } else if (t < 27) {
-    v = nnz > 0 ? log2(__ddiv_rn((double)acc->pad[t - 24], z)) : 0.0;
-  } else if (t < 30) {
-    v = nnz > 0 ? __ddiv_rn((double)acc->elong[t - 27], z) : 0.0;
-  } else {
-    const double ns = (double)((rows + 31) / 32);
-    const double sm = __ddiv_rn(z, ns);
-    const double sden = sm > 1.0 ? sm : 1.0;
-    if (t == 30) {
-      double var = __dsub_rn(__ddiv_rn((double)acc->s32_sq, ns), __dmul_rn(sm, sm));
-      if (var < 0.0) var = 0.0;
-      v = __ddiv_rn(sqrt(var), sden);
-    } else {
-      v = log2(__dadd_rn(1.0, __ddiv_rn((double)acc->s32_max, sden)));
-    }
-  }
-  f[t] = v;
+  if (threadIdx.x == 0) s_last = atomicAdd(&acc->done, 1ull) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (threadIdx.x < kNFeat) feat_final(threadIdx.x, rows, nnz, acc, feat);
 }
 
 // ------------------------------------------------------------------ MLP (FP32)
@@ -310,39 +338,229 @@ __global__ void k_dense_fwd(int B, int nin, int nout, const float *__restrict__ 
   if (H) H[t] = relu ? fmaxf(s, 0.f) : s;
 }
 
-// gO = (O - T) / (B * nout); loss = sum (O - T)^2 / (2 B nout), one block.
+// gO = (O - T) / (B * nout)
 __global__ void k_out_grad(int total, float scale, const float *__restrict__ O, const float *__restrict__ T,
-                           float *__restrict__ G, float *loss) {
-  __shared__ float part[256];
-  float s = 0.f;
-  for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    const float e = O[i] - T[i];
-    G[i] = e * scale;
-    s = fmaf(e, e, s);
-  }
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && loss) *loss = 0.5f * part[0] * scale;
+                           float *__restrict__ G) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < total) G[i] = (O[i] - T[i]) * scale;
 }
 
-// dW[j][i] = sum_n G[n][j] H[n][i]; db[j] = sum_n G[n][j] (thread per (j, i),
-// i == nin for the bias); sums run over n in order.
-__global__ void k_weight_grad(int B, int nin, int nout, const float *__restrict__ G, const float *__restrict__ H,
-                              float *__restrict__ dW, float *__restrict__ db) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nout * (nin + 1)) return;
-  const int j = t / (nin + 1), i = t - j * (nin + 1);
-  float s = 0.f;
-  if (i < nin) {
-    for (int n = 0; n < B; ++n) s = fmaf(G[n * nout + j], H[n * nin + i], s);
-    dW[j * nin + i] = s;
-  } else {
-    for (int n = 0; n < B; ++n) s += G[n * nout + j];
-    db[j] = s;
+// All three layers' weight gradients in one launch: dW[j][i] = sum_n G[n][j]
+// H[n][i], db[j] = sum_n G[n][j] (i == nin: H = 1), and the loss.  A block
+// takes a tile of 32 inputs i (a lane each) by kGradJ outputs j of one layer;
+// its warps take every kGradWarps-th sample, and their partial sums are added
+// in warp order, so the sums do not depend on the launch.  With a thread
+// walking the whole batch for one weight the three launches took 52 us at a
+// batch of 256 (a chain of 256 dependent loads and FMAs, 60 blocks).
+constexpr int kGradJ = 4, kGradWarps = 16;
+struct GradLayer {
+  int nin, nout;
+  const float *G, *H;
+  float *dW, *db;
+};
+struct GradArgs {
+  GradLayer l[3];
+  int tiles[3];  // blocks of each layer
+};
+__global__ void __launch_bounds__(kGradWarps * 32) k_weight_grads(int B, GradArgs ga, int nloss, float scale,
+                                                                  const float *O,
+                                                                  const float *T, float *loss) {
+  __shared__ float part[kGradWarps][kGradJ][32];
+  pdl_wait();
+  pdl_launch_dependents();
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int t = blockIdx.x, k = 0;
+  while (k < 3 && t >= ga.tiles[k]) t -= ga.tiles[k++];
+  if (k == 3) {  // the last block: loss = sum (O - T)^2 / (2 B nout), 256 partial sums joined by a tree
+    float *p = &part[0][0][0];
+    if (threadIdx.x < 256) {
+      float s = 0.f;
+      for (int i = threadIdx.x; i < nloss; i += 256) {
+        const float e = O[i] - T[i];
+        s = fmaf(e, e, s);
+      }
+      p[threadIdx.x] = s;
+    }
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+      if ((int)threadIdx.x < h) p[threadIdx.x] += p[threadIdx.x + h];
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) *loss = 0.5f * p[0] * scale;
+    return;
+  }
+  const GradLayer L = ga.l[k];
+  const int itiles = L.nin / 32 + 1;  // nin + 1 inputs, the bias's 1 last
+  const int i = (t % itiles) * 32 + lane, j0 = (t / itiles) * kGradJ;
+  float s[kGradJ] = {};
+#pragma unroll 8
+  for (int n = w; n < B; n += kGradWarps) {
+    const float h = i < L.nin ? L.H[(size_t)n * L.nin + i] : 1.f;
+#pragma unroll
+    for (int u = 0; u < kGradJ; ++u)
+      if (j0 + u < L.nout) s[u] = fmaf(L.G[(size_t)n * L.nout + j0 + u], h, s[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < kGradJ; ++u) part[w][u][lane] = s[u];
+  __syncthreads();
+  if (w < kGradJ && j0 + w < L.nout && i <= L.nin) {
+    float v = part[0][w][lane];
+    for (int q = 1; q < kGradWarps; ++q) v += part[q][w][lane];
+    if (i < L.nin) L.dW[(size_t)(j0 + w) * L.nin + i] = v;
+    else L.db[j0 + w] = v;
+  }
+}
+
+// These kernels start before the one ahead of them in the stream has ended and
+// wait for it first thing (pdl_wait); none of their inputs is declared
+// __restrict__, so that no read of it can be scheduled ahead of the wait.
+//
+// A block takes kMlpRows samples through all layers: the weights and the
+// samples' activations are in shared memory, so a layer costs a block barrier
+// instead of a launch and a trip through L2 (three launches, 15.7 us at a
+// batch of 256).  A weight row is padded to an odd length: the lanes of a warp
+// hold consecutive outputs j and read W[j][i] at the same i.  Every output is
+// bias + one FMA chain over i, as k_dense_fwd sums it.  A training step at a
+// batch of 256 (forward, backward, Adam): 98 us with ten launches, 39 us with
+// these four, of which the host's launches and calls are most.
+constexpr int kMlpRows = 4, kMlpThreads = 256;
+constexpr size_t kMlpSmem = 96 * 1024;  // larger networks: a launch per layer
+__host__ __device__ __forceinline__ int odd(int n) { return n | 1; }
+__host__ __device__ __forceinline__ size_t mlp_smem_floats(int nin, int nh, int nout) {
+  return (size_t)nh * odd(nin) + (size_t)nh * odd(nh) + (size_t)nout * odd(nh) + 2 * nh + nout +
+         (size_t)kMlpRows * (nin + 2 * nh);
+}
+bool mlp_fits(int nin, int nh, int nout) { return mlp_smem_floats(nin, nh, nout) * 4 <= kMlpSmem; }
+
+// `rows` rows of n floats into shared memory at a stride of ld floats, 4 bytes
+// per cp.async (the padded rows allow no wider copy): all of a thread's words
+// are in flight at once; mlp_copy_wait() before the block barrier.
+__device__ __forceinline__ void mlp_copy(const float *src, float *dst, int rows, int n, int ld) {
+  const int total = rows * n;
+  const int dj = kMlpThreads / n, di = kMlpThreads - dj * n;  // a step of kMlpThreads words, in rows and columns
+  int j = threadIdx.x / n, i = threadIdx.x - j * n;
+  for (int t = threadIdx.x; t < total; t += kMlpThreads) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + j * ld + i)), "l"(src + t) : "memory");
+    j += dj;
+    i += di;
+    if (i >= n) {
+      i -= n;
+      ++j;
+    }
+  }
+}
+__device__ __forceinline__ void mlp_copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// out(r, j, sum) for every sample r < R of the block and output j
+template <typename F>
+__device__ __forceinline__ void mlp_layer(int R, int nin, int nout, const float *W, const float *bias, const float *in,
+                                          F out) {
+  for (int t = threadIdx.x; t < R * nout; t += kMlpThreads) {
+    const int r = t / nout, j = t - r * nout;
+    const float *w = W + j * odd(nin), *x = in + r * nin;
+    float s = bias[j];
+#pragma unroll 8
+    for (int i = 0; i < nin; ++i) s = fmaf(w[i], x[i], s);
+    out(r, j, s);
+  }
+}
+// The whole network on R samples held in x (shared), O(r, j, value) the outputs; Z1, H1, Z2, H2 (global, the block's
+// first row) written when Z1 is not NULL.
+template <typename F>
+__device__ __forceinline__ void mlp_block(int R, int nin, int nh, int nout, const float *params,
+                                          float *smem, float *Z1, float *H1, float *Z2, float *H2, F O) {
+  float *W1 = smem, *W2 = W1 + nh * odd(nin), *W3 = W2 + nh * odd(nh), *b1 = W3 + nout * odd(nh), *b2 = b1 + nh,
+        *b3 = b2 + nh, *x = b3 + nout, *a1 = x + kMlpRows * nin, *a2 = a1 + kMlpRows * nh;
+  const float *p2 = params + nh * nin + nh, *p3 = p2 + nh * nh + nh;
+  mlp_copy(params, W1, nh, nin, odd(nin));
+  mlp_copy(p2, W2, nh, nh, odd(nh));
+  mlp_copy(p3, W3, nout, nh, odd(nh));
+  mlp_copy(params + nh * nin, b1, 1, nh, nh);
+  mlp_copy(p2 + nh * nh, b2, 1, nh, nh);
+  mlp_copy(p3 + nout * nh, b3, 1, nout, nout);
+  mlp_copy_wait();
+  __syncthreads();
+  mlp_layer(R, nin, nh, W1, b1, x, [&](int r, int j, float s) {
+    const float h = fmaxf(s, 0.f);
+    a1[r * nh + j] = h;
+    if (Z1) {
+      Z1[r * nh + j] = s;
+      H1[r * nh + j] = h;
+    }
+  });
+  __syncthreads();
+  mlp_layer(R, nh, nh, W2, b2, a1, [&](int r, int j, float s) {
+    const float h = fmaxf(s, 0.f);
+    a2[r * nh + j] = h;
+    if (Z1) {
+      Z2[r * nh + j] = s;
+      H2[r * nh + j] = h;
+    }
+  });
+  __syncthreads();
+  mlp_layer(R, nh, nout, W3, b3, a2, O);
+}
+__device__ __forceinline__ float *mlp_x(float *smem, int nin, int nh, int nout) {
+  return smem + nh * odd(nin) + nh * odd(nh) + nout * odd(nh) + 2 * nh + nout;
+}
+
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_fwd(int B, int nin, int nh, int nout, const float *X,
+                                                         const float *params, float *Z1, float *H1,
+                                                         float *Z2, float *H2, float *O) {
+  extern __shared__ float smem_f[];
+  pdl_wait();
+  pdl_launch_dependents();
+  const size_t n0 = (size_t)blockIdx.x * kMlpRows;
+  const int R = (int)min((size_t)kMlpRows, (size_t)B - n0);
+  float *x = mlp_x(smem_f, nin, nh, nout);
+  for (int t = threadIdx.x; t < R * nin; t += kMlpThreads) x[t] = X[n0 * nin + t];
+  const size_t at = n0 * nh;
+  mlp_block(R, nin, nh, nout, params, smem_f, Z1 + at, H1 + at, Z2 + at, H2 + at,
+            [&](int r, int j, float s) { O[(n0 + r) * nout + j] = s; });
+}
+
+// Backward through the samples: gO = (O - T) / (B nout), g2 = (Z2 > 0) W3^T gO,
+// g1 = (Z1 > 0) W2^T g2, kMlpRows samples per block, W2 and W3 in shared
+// memory.
+__host__ __device__ __forceinline__ size_t mlp_bwd_smem_floats(int nh, int nout) {
+  return (size_t)nh * nh + (size_t)nout * nh + (size_t)kMlpRows * (nout + nh);
+}
+__global__ void __launch_bounds__(kMlpThreads) k_mlp_bwd(int B, int nh, int nout, float scale, const float *O,
+                                                         const float *T, const float *W2, const float *W3,
+                                                         const float *Z1, const float *Z2, float *gO, float *g2,
+                                                         float *g1) {
+  extern __shared__ float smem_f[];
+  pdl_wait();
+  pdl_launch_dependents();
+  const size_t n0 = (size_t)blockIdx.x * kMlpRows;
+  const int R = (int)min((size_t)kMlpRows, (size_t)B - n0);
+  float *w2 = smem_f, *w3 = w2 + nh * nh, *so = w3 + nout * nh, *s2 = so + kMlpRows * nout;
+  mlp_copy(W3, w3, nout, nh, nh);
+  mlp_copy(W2, w2, nh, nh, nh);
+  for (int t = threadIdx.x; t < R * nout; t += kMlpThreads) {
+    const float g = (O[n0 * nout + t] - T[n0 * nout + t]) * scale;
+    so[t] = g;
+    gO[n0 * nout + t] = g;
+  }
+  mlp_copy_wait();
+  __syncthreads();
+  for (int t = threadIdx.x; t < R * nh; t += kMlpThreads) {
+    const int r = t / nh, i = t - r * nh;
+    const float z = Z2[n0 * nh + t];
+    float s = 0.f;
+#pragma unroll 8
+    for (int j = 0; j < nout; ++j) s = fmaf(w3[j * nh + i], so[r * nout + j], s);
+    s = z > 0.f ? s : 0.f;
+    s2[t] = s;
+    g2[n0 * nh + t] = s;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < R * nh; t += kMlpThreads) {
+    const int r = t / nh, i = t - r * nh;
+    const float z = Z1[n0 * nh + t];
+    float s = 0.f;
+#pragma unroll 8
+    for (int j = 0; j < nh; ++j) s = fmaf(w2[j * nh + i], s2[r * nh + j], s);
+    g1[n0 * nh + t] = z > 0.f ? s : 0.f;
   }
 }
 
@@ -358,8 +576,10 @@ __global__ void k_back_hidden(int B, int nin, int nout, const float *__restrict_
 }
 
 // Adam (Kingma and Ba 2015); c1 = 1 - beta1^t, c2 = 1 - beta2^t.
-__global__ void k_adam(int n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2) {
+__global__ void k_adam(int n, float *p, const float *g, float *m,
+                       float *v, float lr, float b1, float b2, float eps, float c1, float c2) {
+  pdl_wait();
+  pdl_launch_dependents();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float gi = g[i];
@@ -370,19 +590,26 @@ __global__ void k_adam(int n, float *__restrict__ p, const float *__restrict__ g
   p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-// x = (f - mean) * scale as FP32 network input; then the argmin of the
-// network's predicted cost over the choices.
-__global__ void k_normalize(int nf, const double *__restrict__ f, const float *__restrict__ mean,
-                            const float *__restrict__ scale, float *__restrict__ x) {
-  const int i = threadIdx.x;
-  if (i < nf) x[i] = ((float)f[i] - mean[i]) * scale[i];
-}
-
-__global__ void k_argmin(int n, const float *__restrict__ o, int *__restrict__ out) {
+// One matrix through the selector, one block: x = (f - mean) * scale as FP32
+// network input, the network, and the argmin of its predicted cost over the
+// choices (the first of equal costs).
+__global__ void __launch_bounds__(kMlpThreads) k_choose(int nin, int nh, int nout, const double *f,
+                                                        const float *mean,
+                                                        const float *scale,
+                                                        const float *params, int *out) {
+  extern __shared__ float smem_f[];
+  __shared__ float cost[CMRS_SEL_CHOICES];
+  float *x = mlp_x(smem_f, nin, nh, nout);
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = threadIdx.x; i < nin; i += kMlpThreads) x[i] = ((float)f[i] - mean[i]) * scale[i];
+  mlp_block(1, nin, nh, nout, params, smem_f, nullptr, nullptr, nullptr, nullptr,
+            [&](int, int j, float s) { cost[j] = s; });
+  __syncthreads();
   if (threadIdx.x != 0) return;
   int best = 0;
-  for (int i = 1; i < n; ++i)
-    if (o[i] < o[best]) best = i;
+  for (int i = 1; i < nout; ++i)
+    if (cost[i] < cost[best]) best = i;
   *out = best;
 }
 
@@ -419,10 +646,17 @@ extern "C" int cmrs_features(int rows, int nnz, const int32_t *row_ptr, const in
   FeatAcc *acc = reinterpret_cast<FeatAcc *>(ws);
   CMRS_CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(FeatAcc), st));
   const int sms = sm_count();
-  const int g = (int)std::min<long long>(ceil_div((long long)rows, 256), (long long)sms * 8);  // 8 warps x 32 rows
-  k_feat_rows<<<g, 256, 0, st>>>(rows, nnz, row_ptr, col_ind, acc);
-  CMRS_LAUNCH_CHECK();
-  k_feat_final<<<1, 32, 0, st>>>(rows, nnz, acc, feat);
+  // stage: 1.25x an average group's entries, so that most groups fit and short
+  // rows leave shared memory for more warps; none where bulk copies cannot go
+  const long long avg = 32LL * nnz / rows;
+  const int cap = (reinterpret_cast<uintptr_t>(col_ind) & 15) == 0 && nnz > 0
+                      ? (int)std::min<long long>(kFeatCap, (avg + avg / 4) / 32 * 32 + 64)
+                      : 0;
+  const size_t smem = cap ? (size_t)(kFeatThreads / 32) * (cap + 8) * 4 : 0;
+  const int g = (int)std::min<long long>(ceil_div((long long)rows, kFeatThreads), (long long)sms * 4);
+  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_feat_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)((kFeatThreads / 32) * (kFeatCap + 8) * 4)));
+  k_feat_rows<<<g, kFeatThreads, smem, st>>>(rows, nnz, cap, row_ptr, col_ind, acc, feat);
   CMRS_LAUNCH_CHECK();
   return CMRS_OK;
 }
@@ -442,6 +676,13 @@ extern "C" int cmrs_mlp_forward(int B, int nin, int nh, int nout, const float *X
               *b3 = W3 + (size_t)nout * nh;
   float *Z1 = acts, *H1 = Z1 + (size_t)B * nh, *Z2 = H1 + (size_t)B * nh, *H2 = Z2 + (size_t)B * nh,
         *O = H2 + (size_t)B * nh;
+  if (mlp_fits(nin, nh, nout)) {
+    const size_t smem = mlp_smem_floats(nin, nh, nout) * 4;
+    if (smem > 48 * 1024)
+      CMRS_CUDA_TRY(cudaFuncSetAttribute(k_mlp_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem));
+    return launch_pdl(k_mlp_fwd, (unsigned)ceil_div(B, kMlpRows), kMlpThreads, smem, st, B, nin, nh, nout, X, params, Z1,
+                      H1, Z2, H2, O);
+  }
   k_dense_fwd<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nin, nh, X, W1, b1, Z1, H1, 1);
   k_dense_fwd<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nh, nh, H1, W2, b2, Z2, H2, 1);
   k_dense_fwd<<<grid_for((long long)B * nout, 128), 128, 0, st>>>(B, nh, nout, H2, W3, b3, nullptr, O, 0);
@@ -465,14 +706,30 @@ extern "C" int cmrs_mlp_backward(int B, int nin, int nh, int nout, const float *
         *dW3 = db2 + nh, *db3 = dW3 + (size_t)nout * nh;
   float *gO = scratch, *g2 = gO + (size_t)B * nout, *g1 = g2 + (size_t)B * nh;
   const float scale = 1.0f / ((float)B * (float)nout);
-  k_out_grad<<<1, 256, 0, st>>>(B * nout, scale, O, T, gO, loss);
-  k_weight_grad<<<grid_for((long long)nout * (nh + 1), 128), 128, 0, st>>>(B, nh, nout, gO, H2, dW3, db3);
-  k_back_hidden<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nh, nout, gO, W3, Z2, g2);
-  k_weight_grad<<<grid_for((long long)nh * (nh + 1), 128), 128, 0, st>>>(B, nh, nh, g2, H1, dW2, db2);
-  k_back_hidden<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nh, nh, g2, W2, Z1, g1);
-  k_weight_grad<<<grid_for((long long)nh * (nin + 1), 128), 128, 0, st>>>(B, nin, nh, g1, X, dW1, db1);
-  CMRS_LAUNCH_CHECK();
-  return CMRS_OK;
+  const size_t smem = mlp_bwd_smem_floats(nh, nout) * 4;
+  if (smem <= kMlpSmem) {
+    if (smem > 48 * 1024)
+      CMRS_CUDA_TRY(cudaFuncSetAttribute(k_mlp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMlpSmem));
+    const int rc = launch_pdl(k_mlp_bwd, (unsigned)ceil_div(B, kMlpRows), kMlpThreads, smem, st, B, nh, nout, scale, O,
+                              T, W2, W3, Z1, Z2, gO, g2, g1);
+    if (rc) return rc;
+  } else {  // wide layers: a launch per layer
+    k_out_grad<<<grid_for((long long)B * nout, 256), 256, 0, st>>>(B * nout, scale, O, T, gO);
+    k_back_hidden<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nh, nout, gO, W3, Z2, g2);
+    k_back_hidden<<<grid_for((long long)B * nh, 128), 128, 0, st>>>(B, nh, nh, g2, W2, Z1, g1);
+    CMRS_LAUNCH_CHECK();
+  }
+  GradArgs ga;
+  ga.l[0] = GradLayer{nh, nout, gO, H2, dW3, db3};
+  ga.l[1] = GradLayer{nh, nh, g2, H1, dW2, db2};
+  ga.l[2] = GradLayer{nin, nh, g1, X, dW1, db1};
+  int blocks = 0;
+  for (int k = 0; k < 3; ++k) {
+    ga.tiles[k] = (ga.l[k].nin / 32 + 1) * (int)ceil_div(ga.l[k].nout, kGradJ);
+    blocks += ga.tiles[k];
+  }
+  return launch_pdl(k_weight_grads, (unsigned)(blocks + (loss ? 1 : 0)), kGradWarps * 32, 0, st, B, ga, B * nout, scale,
+                    O, T, loss);
 }
 
 extern "C" int cmrs_mlp_adam(int n, float *params, const float *grads, float *m, float *v, int step, float lr,
@@ -480,9 +737,8 @@ extern "C" int cmrs_mlp_adam(int n, float *params, const float *grads, float *m,
   CMRS_TRACE();
   if (n < 1 || !params || !grads || !m || !v || step < 1) return CMRS_ERR_ARG;
   const float c1 = 1.f - powf(beta1, (float)step), c2 = 1.f - powf(beta2, (float)step);
-  k_adam<<<grid_for(n, 256), 256, 0, as_stream(stream)>>>(n, params, grads, m, v, lr, beta1, beta2, eps, c1, c2);
-  CMRS_LAUNCH_CHECK();
-  return CMRS_OK;
+  return launch_pdl(k_adam, (unsigned)grid_for(n, 256), 256, 0, as_stream(stream), n, params, grads, m, v, lr, beta1,
+                    beta2, eps, c1, c2);
 }
 
 // ------------------------------------------------------------------ selection
@@ -491,7 +747,7 @@ extern "C" int cmrs_mlp_adam(int n, float *params, const float *grads, float *m,
 static size_t pad_cap(int rows, int nnz) { return 2 * (size_t)nnz + 32 * ((size_t)rows / 16 + 2); }
 
 static size_t select_ws(int rows, int cols, int nnz, int exhaustive) {
-  size_t b = features_ws(rows) + align256(kNFeat * 8) + align256(1024 * 4) + align256(64);
+  size_t b = features_ws(rows) + align256(kNFeat * 8) + align256(64);
   if (exhaustive) {
     const size_t strips = (size_t)rows + 1;
     b += align256(strips * 4) + align256((size_t)std::max(nnz, 1) * 4) * 3 + align256((size_t)std::max(cols, 1) * 4) +
@@ -612,8 +868,6 @@ extern "C" int cmrs_select_strip(int rows, int cols, int nnz, const int32_t *row
   size_t off = features_ws(rows);
   double *feat = reinterpret_cast<double *>(ws + off);
   off += align256(kNFeat * 8);
-  float *buf = reinterpret_cast<float *>(ws + off);
-  off += align256(1024 * 4);
   int *choice = reinterpret_cast<int *>(ws + off);
   off += align256(64);
   if (!exhaustive) {
@@ -622,13 +876,10 @@ extern "C" int cmrs_select_strip(int rows, int cols, int nnz, const int32_t *row
       return CMRS_ERR_ARG;
     int rc = cmrs_features(rows, nnz, row_ptr, col_ind, feat, workspace, features_ws(rows), stream);
     if (rc) return rc;
-    const int nh = model->nh, nout = model->nout;
-    float *x = buf, *acts = buf + 32;  // 4*nh + nout <= 4*64 + 21 floats fit in the 992 left
-    k_normalize<<<1, 32, 0, st>>>(kNFeat, feat, model->feat_mean, model->feat_scale, x);
-    rc = cmrs_mlp_forward(1, kNFeat, nh, nout, x, model->params, acts, stream);
+    const int nh = model->nh, nout = model->nout;  // nh <= 64: the network takes at most 34 KB of shared memory
+    rc = launch_pdl(k_choose, 1, kMlpThreads, mlp_smem_floats(kNFeat, nh, nout) * 4, st, kNFeat, nh, nout, feat,
+                    model->feat_mean, model->feat_scale, model->params, choice);
     if (rc) return rc;
-    k_argmin<<<1, 32, 0, st>>>(nout, acts + 4 * nh, choice);
-    CMRS_LAUNCH_CHECK();
     int c = 0;
     CMRS_CUDA_TRY(cudaMemcpyAsync(&c, choice, sizeof(int), cudaMemcpyDeviceToHost, st));
     CMRS_CUDA_TRY(cudaStreamSynchronize(st));

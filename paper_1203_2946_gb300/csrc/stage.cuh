@@ -55,4 +55,18 @@ __device__ void issue_stage(long long ea, long long eb, long long nnz, const uin
   }
 }
 
+// One thread: copy words [ea, eb) of one 16-byte aligned array of n 32-bit
+// words into dst (room for eb - ea + 8), word k at dst[k - (ea & ~3)].  As
+// issue_stage: the bulk copy covers the 4-word-aligned body, the words past the
+// array's last full group of four are loaded by this thread.
+__device__ __forceinline__ void issue_words(int ea, int eb, int n, const int32_t *src, int32_t *dst, uint64_t *bar,
+                                            uint64_t pol) {
+  const int a4 = ea & ~3, n4 = n & ~3;
+  const int e4 = max(a4, (int)min((long long)n4, ((long long)eb + 3) & ~3LL));
+  for (int k = e4; k < eb; ++k) dst[k - a4] = src[k];
+  fence_proxy_async();
+  mbar_arrive_expect_tx(bar, (uint32_t)(e4 - a4) * 4u);
+  if (e4 > a4) bulk_g2s(dst, src + a4, (uint32_t)(e4 - a4) * 4u, bar, pol);
+}
+
 }  // namespace cmrs
