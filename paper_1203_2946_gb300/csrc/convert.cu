@@ -20,42 +20,11 @@ struct StatusBlock {
   uint32_t pad[62];
 };
 
-// ---------------------------------------------------------------- validation
-// Section 2.3: RowPtr[0] = 0, RowPtr[rows] = nnz, row lengths >= 0.
-__global__ void k_validate_rowptr(int rows, int nnz, const int32_t *__restrict__ row_ptr, StatusBlock *st) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t bad = 0;
-  for (; i < rows; i += gridDim.x * blockDim.x) {
-    int32_t a = row_ptr[i], b = row_ptr[i + 1];
-    if (a < 0 || b < a || b > nnz) bad = 1;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && (row_ptr[0] != 0 || row_ptr[rows] != nnz)) bad = 1;
-  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&st->status, ST_BAD_ROWPTR);
-}
-
-// ---------------------------------------------------------------- StripPtr
-// Section 3: StripPtr[j] = RowPtr[j * height] for j < strips, StripPtr[strips]
-// = nnz.  Also records the longest strip.
-__global__ void k_strip_ptr(int rows, int nnz, int height, int strips, const int32_t *__restrict__ row_ptr,
-                            int32_t *__restrict__ strip_ptr, StatusBlock *st) {
-  int j = blockIdx.x * blockDim.x + threadIdx.x;
-  int len = 0;
-  if (j <= strips) {
-    int32_t v = j < strips ? row_ptr[(int64_t)j * height] : nnz;
-    strip_ptr[j] = v;
-    if (j < strips) {
-      int64_t e = std::min<int64_t>((int64_t)(j + 1) * height, rows);
-      len = row_ptr[e] - v;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(0xffffffffu, len, o));
-  if ((threadIdx.x & 31) == 0 && len > 0) atomicMax(&st->max_strip, len);
-}
-
 // ---------------------------------------------------------------- value forms
 // F32: IEEE round to nearest even.  BF16: round to nearest even of the FP32
 // value.  BF16X2: hi = BF16(v), lo = BF16(v - hi), the difference taken in
-// double.
+// double.  A float source skips the double: same bits, and no conversion on
+// the FP64 pipe.
 template <int DT>
 struct Encode;
 template <>
@@ -67,12 +36,21 @@ template <>
 struct Encode<CMRS_F32> {
   typedef float Out;
   __device__ static void put(double v, Out *hi, Out *, int64_t k) { hi[k] = __double2float_rn(v); }
+  // as through double and back: a signalling NaN comes out quiet, its other bits kept (no conversion: one on the
+  // FP64 pipe costs its issue slot even where no lane needs it)
+  __device__ static void put(float v, Out *hi, Out *, int64_t k) {
+    if (v != v) v = __uint_as_float(__float_as_uint(v) | 0x00400000u);
+    hi[k] = v;
+  }
 };
 template <>
 struct Encode<CMRS_BF16> {
   typedef uint16_t Out;
   __device__ static void put(double v, Out *hi, Out *, int64_t k) {
-    hi[k] = __bfloat16_as_ushort(__float2bfloat16_rn(__double2float_rn(v)));
+    put(__double2float_rn(v), hi, nullptr, k);
+  }
+  __device__ static void put(float v, Out *hi, Out *, int64_t k) {
+    hi[k] = __bfloat16_as_ushort(__float2bfloat16_rn(v));
   }
 };
 template <>
@@ -84,43 +62,78 @@ struct Encode<CMRS_BF16X2> {
     hi[k] = h;
     lo[k] = __bfloat16_as_ushort(__float2bfloat16_rn(__double2float_rn(rest)));
   }
+  // v - hi is a multiple of v's last place of at most 17 bits: FP32 holds it exactly
+  __device__ static void put(float v, Out *hi, Out *lo, int64_t k) {
+    const uint16_t h = __bfloat16_as_ushort(__float2bfloat16_rn(v));
+    hi[k] = h;
+    lo[k] = __bfloat16_as_ushort(__float2bfloat16_rn(__fsub_rn(v, bf16_bits_to_float(h))));
+  }
 };
 
 // ---------------------------------------------------------------- packing
-// Section 4: packed = (col << bits) | (row mod height).  A warp takes 32
-// consecutive rows at a time: their entries are one contiguous CRS range,
-// walked with coalesced loads, kPackU batches of 32 in flight per lane; an
-// entry finds its row among the 32 row starts (held one per lane) by a
-// five-step shuffle search.  A group of rows with an invalid RowPtr range is
-// skipped (the validation kernel has flagged it), so no access leaves the
-// arrays.
+// The whole unsorted conversion in one pass.  A warp takes 32 consecutive rows
+// at a time, row `lane`'s start in each lane.
+//   Section 2.3: RowPtr[0] = 0, RowPtr[rows] = nnz, row lengths >= 0.  A group
+// of rows with an invalid RowPtr range is flagged and skipped, so no access
+// leaves the arrays.
+//   Section 3: StripPtr[j] = RowPtr[j * height] for j < strips,
+// StripPtr[strips] = nnz; the longest strip is recorded.
+//   Section 4: packed = (col << bits) | (row mod height).  The rows' entries
+// are one contiguous CRS range, walked with coalesced loads, kPackU batches of
+// 32 in flight per lane.  The row of an entry is the number of row starts up
+// to it: the starts that fall into a batch are joined into one 32-bit mask, so
+// a batch costs one reduction and a bit count.  Where a group has empty rows
+// (equal starts) an entry finds its row among the 32 starts by a five-step
+// shuffle search instead.
+// Bound by HBM: 67M FP32 entries (1.07 GB) in 174 us; with the search for every
+// batch and a conversion through double for every value (the FP64 pipe 85%
+// busy) it took 267 us, and the checks and StripPtr were two more launches.
 constexpr int kPackU = 4;
 template <typename In, int DT>
-__global__ void k_pack(int rows, int cols, int nnz, int height, int bits, const int32_t *__restrict__ row_ptr,
-                       const int32_t *__restrict__ col_ind, const In *__restrict__ val_in,
-                       uint32_t *__restrict__ packed, typename Encode<DT>::Out *__restrict__ vhi,
-                       typename Encode<DT>::Out *__restrict__ vlo, StatusBlock *st) {
+__global__ void k_pack(int rows, int cols, int nnz, int height, int strips, int bits,
+                       const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col_ind,
+                       const In *__restrict__ val_in, int32_t *__restrict__ strip_ptr, uint32_t *__restrict__ packed,
+                       typename Encode<DT>::Out *__restrict__ vhi, typename Encode<DT>::Out *__restrict__ vlo,
+                       StatusBlock *st) {
+  const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const long long groups = ((long long)rows + 31) / 32;
   uint32_t bad = 0;
+  int longest = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    strip_ptr[strips] = nnz;
+    if (row_ptr[0] != 0 || row_ptr[rows] != nnz) bad = ST_BAD_ROWPTR;
+  }
   for (long long g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < groups; g += warps) {
     const long long r0 = g * 32;
     const long long r = r0 + lane;
     // row `lane` of the group: [start, end); rows past the matrix are empty
     const int32_t start = r < rows ? row_ptr[r] : 0;
     const int32_t last = row_ptr[min(r0 + 32, (long long)rows)];
-    int32_t end = __shfl_down_sync(0xffffffffu, start, 1);
+    int32_t end = __shfl_down_sync(kAll, start, 1);
     if (lane == 31 || r + 1 >= rows) end = last;
+    const unsigned sj = (unsigned)r / (unsigned)height;  // r < rows + 32 fits 32 unsigned bits
+    const int ris_r = (int)((unsigned)r - sj * (unsigned)height);
+    if (r < rows && ris_r == 0) {
+      strip_ptr[sj] = start;
+      longest = max(longest, row_ptr[min(r + height, (long long)rows)] - start);
+    }
     const bool ok = r >= rows || (start >= 0 && end >= start && end <= nnz);
-    if (!__all_sync(0xffffffffu, ok)) continue;
-    const int32_t e0 = __shfl_sync(0xffffffffu, start, 0);
+    if (!__all_sync(kAll, ok)) {
+      bad |= ST_BAD_ROWPTR;
+      continue;
+    }
+    const int32_t e0 = __shfl_sync(kAll, start, 0);
     const int32_t e1 = last;
     const int nrows = (int)min(32LL, rows - r0);
     const int32_t key = lane < nrows ? start : e1;  // empty tail rows sort last
-    const uint32_t ris_lane = (uint32_t)(r % height);
+    const uint32_t ris_lane = (uint32_t)ris_r;
+    const bool full = __all_sync(kAll, lane >= nrows || end > start);
+    int before = -1;  // rows started before the batch, minus one
     for (int32_t k0 = e0; k0 < e1; k0 += 32 * kPackU) {
       int32_t c[kPackU];
+      int j[kPackU];  // the row of the group holding the entry
       In v[kPackU];
 #pragma unroll
       for (int u = 0; u < kPackU; ++u) {
@@ -130,30 +143,49 @@ __global__ void k_pack(int rows, int cols, int nnz, int height, int bits, const 
           v[u] = val_in[k];
         }
       }
+      if (full) {
+#pragma unroll
+        for (int u = 0; u < kPackU; ++u) {
+          const int32_t kb = k0 + 32 * u;
+          const unsigned rel = (unsigned)(key - kb);
+          const unsigned starts = __reduce_or_sync(kAll, rel < 32u ? 1u << rel : 0u);
+          j[u] = before + __popc(starts << (31 - lane));  // of which at or before this lane's entry
+          before += __popc(starts);
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < kPackU; ++u) {
+          const int32_t k = k0 + 32 * u + lane;
+          j[u] = 0;  // the last of the group's rows starting at or before k
+#pragma unroll
+          for (int step = 16; step >= 1; step >>= 1) {
+            const int32_t s = __shfl_sync(kAll, key, j[u] + step);
+            if (s <= k) j[u] += step;
+          }
+        }
+      }
 #pragma unroll
       for (int u = 0; u < kPackU; ++u) {
         const int32_t k = k0 + 32 * u + lane;
-        // the row holding k: the last of the group's rows starting at or before k
-        int j = 0;
-#pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-          const int32_t sj = __shfl_sync(0xffffffffu, key, j + step);
-          if (sj <= k) j += step;
-        }
-        const uint32_t ris = __shfl_sync(0xffffffffu, ris_lane, j);
+        const uint32_t ris = __shfl_sync(kAll, ris_lane, j[u]);
         if (k < e1) {
           int32_t col = c[u];
-          if (col < 0 || col >= cols) {
-            bad = 1;
+          if ((uint32_t)col >= (uint32_t)cols) {
+            bad |= ST_BAD_COL;
             col = 0;
           }
           packed[k] = ((uint32_t)col << bits) | ris;
-          Encode<DT>::put((double)v[u], vhi, vlo, k);
+          Encode<DT>::put(v[u], vhi, vlo, k);
         }
       }
     }
   }
-  if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&st->status, ST_BAD_COL);
+  bad = __reduce_or_sync(kAll, bad);
+  longest = __reduce_max_sync(kAll, longest);
+  if (lane == 0) {
+    if (bad) atomicOr(&st->status, bad);
+    if (longest > 0) atomicMax(&st->max_strip, longest);
+  }
 }
 
 // ---------------------------------------------------------------- in-strip sort
@@ -580,20 +612,14 @@ int from_csr_impl(int rows, int cols, int nnz, int height, int bits, uint32_t fl
   const int strips = (int)ceil_div(rows, height);
   CMRS_CUDA_TRY(cudaMemsetAsync(sb, 0, sizeof(StatusBlock), st));
   const int sms = sm_count();
-  {
-    int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(rows, 256), sms * 8));
-    k_validate_rowptr<<<g, 256, 0, st>>>(rows, nnz, row_ptr, sb);
-    CMRS_LAUNCH_CHECK();
-  }
-  k_strip_ptr<<<(int)ceil_div(strips + 1, 256), 256, 0, st>>>(rows, nnz, height, strips, row_ptr, strip_ptr, sb);
-  CMRS_LAUNCH_CHECK();
   const bool sorted = (flags & CMRS_SORTED) != 0;
   uint32_t *pk = sorted ? reinterpret_cast<uint32_t *>(ws + L.ptmp) : packed;
   Out *vh = sorted ? reinterpret_cast<Out *>(ws + L.vtmp) : reinterpret_cast<Out *>(val_out);
   Out *vl = DT == CMRS_BF16X2 ? vh + cmrs_pad8(nnz) : nullptr;
-  if (rows > 0 && nnz > 0) {
-    int g = (int)std::min<int64_t>(ceil_div((int64_t)rows, 256), (int64_t)sms * 16);  // 8 warps x 32 rows
-    k_pack<In, DT><<<g, 256, 0, st>>>(rows, cols, nnz, height, bits, row_ptr, col_ind, val_in, pk, vh, vl, sb);
+  {
+    int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div((int64_t)rows, 256), (int64_t)sms * 16));  // 8 warps x 32 rows
+    k_pack<In, DT><<<g, 256, 0, st>>>(rows, cols, nnz, height, strips, bits, row_ptr, col_ind, val_in, strip_ptr, pk,
+                                      vh, vl, sb);
     CMRS_LAUNCH_CHECK();
   }
   if (sorted && nnz > 0 && strips > 0) {
