@@ -58,3 +58,79 @@ def test_row_of_each_entry(b, h, lengths):
     assert np.array_equal(M.col_packed.cpu().numpy()[:a.nnz].view(np.uint32), ref["packed"])
     assert np.array_equal(b.stored_values(M).cpu().numpy(), ref["val"])
     assert M.struct.max_strip_nnz == np.diff(ref["strip_ptr"]).max()
+
+
+def csr(lengths, cols, seed, ordered=True, repeats=False):
+    """Rows of the given lengths; columns increasing, or shuffled inside each row, or drawn with repeats."""
+    a = inputs.from_lengths(lengths, cols, seed=seed)
+    if ordered:
+        return a
+    rng = np.random.default_rng(seed)
+    ci = a.col_ind.copy()
+    for r in range(a.rows):
+        p, q = a.row_ptr[r], a.row_ptr[r + 1]
+        ci[p:q] = rng.integers(0, min(50, cols), q - p) if repeats else rng.permutation(ci[p:q])
+    return inputs.CSR(a.rows, a.cols, a.row_ptr, ci, a.val, a.name)
+
+
+SORT_CASES = {
+    "short": (lambda rng: rng.integers(0, 12, 501), 4000),  # warp strips, empty rows, a last strip cut short
+    "equal_columns": (lambda rng: np.full(320, 7), 9),      # nearly every column in every row: ties across rows
+    "full_rows": (lambda rng: np.full(96, 32), 32),         # dense strips: as many ties as rows
+    # a warp's buffer, a CTA's, the radix sort: strips either side of each bound at some height below
+    "bounds": (lambda rng: np.concatenate([np.full(64, 8), [256 - 8 * 7, 257, 1024, 1025, 6144, 6145, 9000], np.full(57, 8)]),
+               20000),
+    "long_mean": (lambda rng: rng.integers(100, 300, 160), 3000),  # CTA strips throughout at height 32
+}
+
+
+@pytest.mark.parametrize("h", [1, 2, 3, 6, 8, 16, 32])
+@pytest.mark.parametrize("case", sorted(SORT_CASES))
+@pytest.mark.parametrize("order", ["ordered", "shuffled", "repeats"])
+def test_sorted_strips(b, case, h, order):
+    make, cols = SORT_CASES[case]
+    a = csr(make(np.random.default_rng(3)), cols, 5, order == "ordered", order == "repeats")
+    rp, ci = dev(a)
+    M = b.cmrs_from_csr(rp, ci, torch.from_numpy(a.val).cuda(), a.cols, h, flags=b.CMRS_SORTED)
+    ref = orc.csr_to_cmrs(a.row_ptr, a.col_ind, a.val, a.cols, h, sorted_=True)
+    assert np.array_equal(M.strip_ptr.cpu().numpy(), ref["strip_ptr"])
+    assert np.array_equal(M.col_packed.cpu().numpy()[:a.nnz].view(np.uint32), ref["packed"])
+    assert np.array_equal(b.stored_values(M).cpu().numpy(), ref["val"])
+    assert M.struct.max_strip_nnz == np.diff(ref["strip_ptr"]).max()
+    rp2, ci2, v2 = b.cmrs_to_csr(M)
+    r3 = orc.cmrs_to_csr(a.rows, h, ref["strip_ptr"], ref["packed"], ref["val"])
+    assert np.array_equal(rp2.cpu().numpy(), r3["row_ptr"])
+    assert np.array_equal(ci2.cpu().numpy(), r3["col_ind"])
+    assert np.array_equal(v2.view(torch.float64).cpu().numpy()[:a.nnz], r3["val"])
+
+
+@pytest.mark.parametrize("src", [torch.float32, torch.float64])
+@pytest.mark.parametrize("dtype", [0, 1, 2, 3])
+def test_sorted_values_every_form(b, dtype, src):
+    a = csr(np.random.default_rng(1).integers(0, 90, 300), 900, 2)
+    rp, ci = dev(a)
+    va = torch.from_numpy(a.val).cuda().to(src)
+    plain = b.cmrs_from_csr(rp, ci, va, a.cols, 12, dtype=dtype)
+    M = b.cmrs_from_csr(rp, ci, va, a.cols, 12, flags=b.CMRS_SORTED, dtype=dtype)
+    order = torch.from_numpy(orc.csr_to_cmrs(a.row_ptr, a.col_ind, a.val, a.cols, 12, sorted_=True)["src"].astype(np.int64)).cuda()
+    v, w = b.stored_values(plain), b.stored_values(M)
+    for k in range(2 if dtype == 3 else 1):
+        assert torch.equal(v[k * a.nnz:(k + 1) * a.nnz][order], w[k * a.nnz:(k + 1) * a.nnz])
+
+
+@pytest.mark.parametrize("what", ["column", "negative", "row_ptr", "last"])
+def test_sorted_invalid_input_is_refused(b, what):
+    a = csr(np.random.default_rng(1).integers(1, 90, 3000), 900, 2)
+    rp, ci = a.row_ptr.copy(), a.col_ind.copy()
+    if what == "column":
+        ci[1234] = 900
+    elif what == "negative":
+        ci[5] = -1
+    elif what == "row_ptr":
+        rp[700] = rp[702]
+    else:
+        rp[-1] -= 1
+    with pytest.raises(b.CmrsError) as e:
+        b.cmrs_from_csr(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), torch.from_numpy(a.val).cuda(), 900, 8,
+                        flags=b.CMRS_SORTED)
+    assert e.value.code == 4
