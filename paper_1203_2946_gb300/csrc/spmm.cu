@@ -11,10 +11,25 @@
 // four rows at once.  Otherwise lane g accumulates column c0 + g (G =
 // min(32, next_pow2(k))).  Columns beyond the group are done in further
 // passes over the row; each column's sum is one FMA chain in entry order
-// either way.  Row bounds inside a strip come from binary
-// searches on RowInStrip (unsorted strips).  A warp takes 32 / G rows at a
-// time.  Work units (matrix, row range) are fetched by warps from a device
-// queue (one atomic per unit), which balances uneven matrices.
+// either way.  Work units (matrix, row range) are fetched by warps from a
+// device queue (one atomic per unit), which balances uneven matrices.
+//
+// What bounds it is the L1 data pipe: a warp's rows lie apart in the entry
+// streams, so a column word and a value read from global memory cost a line
+// each per row and entry, as much as the gather of X itself (78% busy, three
+// lines an entry).  So a warp copies the entries of up to 32 consecutive rows
+// -- one contiguous range -- into its own shared-memory stage with two bulk
+// copies and reads words and values there, where the lanes of a row share one
+// read.  Rows whose entries do not fit the stage, and matrices whose arrays
+// are not 16-byte aligned, are read from global memory.  Where one or two
+// lanes hold a row's columns, two lane groups share the row's entries (their
+// sums joined by a shuffle), which halves the stage a warp needs.  And the
+// warps of an SM work on neighbouring rows (see QueueHead), so that they find
+// X in L1.  32 banded matrices (119M entries, rows of 10..60, one launch), all
+// with k columns, before and after: k = 1 665 -> 244 us, k = 4 727 -> 371 us, k
+// = 8 714 -> 527 us, k = 32 1,467 -> 1,199 us (its gathers of whole lines wait
+// on L2: 7 CTAs of 4 warps keep more of them in flight than 5 or 6 with a
+// larger L1; 2, 3, 6 and 8 gathers in flight per lane are slower than 4).
 #include <algorithm>
 #include <chrono>
 #include <mutex>
@@ -22,25 +37,39 @@
 #include <vector>
 
 #include "common.cuh"
+#include "stage.cuh"
 
 namespace cmrs {
 namespace {
 
-constexpr int kSpmmThreads = 256;
-constexpr int kSpmmCH = 2;  // entries whose gathers are in flight together (8 raised registers to 64 and was slower)
-#ifndef CMRS_SPMM_CH4
-#define CMRS_SPMM_CH4 2  // 16-byte gathers in flight per lane (measured 6.45 ms per batch; 1: 6.72, 3: 7.06, 4: 7.07, 8: 7.73)
+#ifndef CMRS_SPMM_CAP
+#define CMRS_SPMM_CAP 704  // entries per warp's stage
 #endif
-constexpr int kSpmmCH4 = CMRS_SPMM_CH4;  // the same for the 16-byte gathers
 #ifndef CMRS_SPMM_MINB
-#define CMRS_SPMM_MINB 5  // resident CTAs per SM asked of the register allocator (48 registers)
+#define CMRS_SPMM_MINB 7  // resident CTAs per SM asked of the register allocator (72 registers)
 #endif
-#ifndef CMRS_SPMM_PREFETCH
-#define CMRS_SPMM_PREFETCH 1  // next batch's column words loaded during this batch's gathers
+#ifndef CMRS_SPMM_D
+#define CMRS_SPMM_D 4  // X gathers in flight per lane
 #endif
+#ifndef CMRS_SPMM_BLOCK
+#define CMRS_SPMM_BLOCK 64  // neighbouring units dealt to one SM together (8: k = 4, 8 products 12% slower)
+#endif
+#ifndef CMRS_SPMM_SPLIT
+#define CMRS_SPMM_SPLIT 2  // most lane groups per row (4 with a stage of 384: no faster, k = 8 slower)
+#endif
+#ifndef CMRS_SPMM_THREADS
+#define CMRS_SPMM_THREADS 128
+#endif
+constexpr int kSpmmThreads = CMRS_SPMM_THREADS;
+constexpr int kSpmmWarps = kSpmmThreads / 32;
+constexpr int kSpmmCap = CMRS_SPMM_CAP;
+constexpr int kSpmmD = CMRS_SPMM_D;
+constexpr size_t kSpmmSmem = kSpmmWarps * Stage<CMRS_F32>::bytes(kSpmmCap);
 
 struct Desc {
-  int32_t rows, height, bits, k, vec, pad;
+  int32_t rows, height, bits, k, vec, nnz;
+  int32_t stage;  // the arrays' alignment allows bulk copies
+  int32_t split;  // lanes groups sharing one row (1 or 2)
   const int32_t *sp;
   const uint32_t *packed;
   const float *val;
@@ -52,15 +81,27 @@ struct Unit {
   int32_t mat, row0, row1, pad;
 };
 
+// The queue: one share of the units per SM.  Units are dealt to the shares in
+// blocks of `block` consecutive ones, so that the warps of an SM work on
+// neighbouring rows of one matrix and find each other's rows of X in L1; a
+// warp takes the next unit of its own SM's share, and of another's when that
+// is used up.
+constexpr int kMaxShares = 1024;
 struct QueueHead {
-  unsigned int next;
-  unsigned int pad[63];
+  unsigned int taken[kMaxShares];  // units taken of each share
+};
+struct Shares {
+  int nunits, shares, block, len;  // len: units per share, the last blocks counted whole
+  __device__ __forceinline__ unsigned unit(int share, unsigned i) const {
+    return ((i / (unsigned)block) * (unsigned)shares + (unsigned)share) * (unsigned)block + i % (unsigned)block;
+  }
 };
 
-__device__ __forceinline__ int lb_ris_g(const uint32_t *__restrict__ cp, int lo, int hi, uint32_t r, uint32_t mask) {
+// First k in [lo, hi) whose RowInStrip is >= r, or hi; entry k is at cp[k - base].
+__device__ __forceinline__ int lb_ris_g(const uint32_t *cp, int base, int lo, int hi, uint32_t r, uint32_t mask) {
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if ((__ldg(cp + mid) & mask) < r) lo = mid + 1;
+    if ((cp[mid - base] & mask) < r) lo = mid + 1;
     else hi = mid;
   }
   return lo;
@@ -74,164 +115,228 @@ __host__ __device__ __forceinline__ int spmm_lanes(int k, int vec) {
   return G;
 }
 
-// Row bounds inside the strip (binary searches on RowInStrip).
-__device__ __forceinline__ void spmm_bounds(const Desc &d, int row, int &k0, int &k1) {
-  const uint32_t mask = (1u << d.bits) - 1;
-  const int s = row / d.height;
-  const uint32_t r = (uint32_t)(row - s * d.height);
-  const int sa = __ldg(d.sp + s), sb = __ldg(d.sp + s + 1);
-  k0 = sa;
-  k1 = sb;
-  if (d.height > 1) {
-    k0 = lb_ris_g(d.packed, sa, sb, r, mask);
-    k1 = lb_ris_g(d.packed, k0, sb, r + 1, mask);
+__device__ __forceinline__ void fma_to(float &acc, float v, float x) { acc = fmaf(v, x, acc); }
+__device__ __forceinline__ void fma_to(float4 &acc, float v, const float4 &x) {
+  acc.x = fmaf(v, x.x, acc.x);
+  acc.y = fmaf(v, x.y, acc.y);
+  acc.z = fmaf(v, x.z, acc.z);
+  acc.w = fmaf(v, x.w, acc.w);
+}
+
+__device__ __forceinline__ void join(float &acc, int lanes) { acc += __shfl_xor_sync(0xffffffffu, acc, lanes); }
+__device__ __forceinline__ void join(float4 &acc, int lanes) {
+  acc.x += __shfl_xor_sync(0xffffffffu, acc.x, lanes);
+  acc.y += __shfl_xor_sync(0xffffffffu, acc.y, lanes);
+  acc.z += __shfl_xor_sync(0xffffffffu, acc.z, lanes);
+  acc.w += __shfl_xor_sync(0xffffffffu, acc.w, lanes);
+}
+
+// One lane's part of one row: columns g, g + G, ... (of kv, in units of V) of
+// Y[row] from entries k0 + q, k0 + q + L, ... of [k0, k1), entry k at cp[k -
+// base], vp[k - base]; the L lanes' sums are joined by a shuffle tree.  All
+// lanes of the warp call (a lane without a row has k0 == k1 and row < 0).
+// Batches of kSpmmD entries have their X gathers in flight together; whole
+// batches go without guards, the last one with.
+template <typename V>
+__device__ __forceinline__ void spmm_row(const Desc &d, int row, int k0, int k1, int base, const uint32_t *cp,
+                                         const float *vp, int g, int G, int q, int L, int kv) {
+  const V *X = reinterpret_cast<const V *>(d.X);
+  V *Y = reinterpret_cast<V *>(d.Y);
+  for (int c0 = 0; c0 < kv; c0 += G) {  // warp-uniform
+    const int col = c0 + g;
+    V acc = {};
+    if (col < kv) {
+      const V *Xc = X + col;
+      int j = k0 - base + q;
+      const int end = k1 - base;
+      for (; j + L * (kSpmmD - 1) < end; j += L * kSpmmD) {
+        V xv[kSpmmD];
+#pragma unroll
+        for (int u = 0; u < kSpmmD; ++u) xv[u] = __ldg(Xc + (size_t)(cp[j + L * u] >> d.bits) * kv);
+#pragma unroll
+        for (int u = 0; u < kSpmmD; ++u) fma_to(acc, vp[j + L * u], xv[u]);
+      }
+      if (j < end) {
+        V xv[kSpmmD - 1];
+#pragma unroll
+        for (int u = 0; u < kSpmmD - 1; ++u)
+          if (j + L * u < end) xv[u] = __ldg(Xc + (size_t)(cp[j + L * u] >> d.bits) * kv);
+#pragma unroll
+        for (int u = 0; u < kSpmmD - 1; ++u)
+          if (j + L * u < end) fma_to(acc, vp[j + L * u], xv[u]);
+      }
+    }
+    for (int o = L >> 1; o > 0; o >>= 1) join(acc, o * G);  // the L lanes of a column are G apart
+    if (row >= 0 && q == 0 && col < kv) Y[(size_t)row * kv + col] = acc;
   }
 }
 
-// Rows [row0, row1) of matrix d, four columns per lane (d.vec).
-__device__ __forceinline__ void spmm_rows4(const Desc &d, int row0, int row1, int lane) {
-  const int kv = d.k >> 2;
-  const int G = spmm_lanes(d.k, 1);
-  const int per = 32 / G;
-  const int g = lane & (G - 1);
-  const int sub = lane / G;
-  const float4 *X4 = reinterpret_cast<const float4 *>(d.X);
-  float4 *Y4 = reinterpret_cast<float4 *>(d.Y);
-  for (int rb = row0; rb < row1; rb += per) {
-    const int row = rb + sub;
-    const bool active = row < row1;
-    int k0 = 0, k1 = 0;
-    if (active) spmm_bounds(d, row, k0, k1);
-    for (int c0 = 0; c0 < kv; c0 += G) {
-      const int col = c0 + g;
-      if (active && col < kv) {
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        // The column words and values of the next batch are loaded while this
-        // batch's X gathers are in flight: a gather waits for its column word,
-        // so without this every batch pays two memory round trips in a row.
-        uint32_t pn[kSpmmCH4];
-        float vn[kSpmmCH4];
-#pragma unroll
-        for (int u = 0; u < kSpmmCH4; ++u)
-          if (k0 + u < k1) {
-            pn[u] = __ldg(d.packed + k0 + u);
-            vn[u] = __ldg(d.val + k0 + u);
-          }
-        for (int j = k0; j < k1; j += kSpmmCH4) {
-          float4 xv[kSpmmCH4];
-          float vv[kSpmmCH4];
-#pragma unroll
-          for (int u = 0; u < kSpmmCH4; ++u) {
-            vv[u] = vn[u];
-            if (j + u < k1) xv[u] = __ldg(X4 + (size_t)(pn[u] >> d.bits) * kv + col);
-          }
-          if (CMRS_SPMM_PREFETCH) {
-#pragma unroll
-            for (int u = 0; u < kSpmmCH4; ++u)
-              if (j + kSpmmCH4 + u < k1) {
-                pn[u] = __ldg(d.packed + j + kSpmmCH4 + u);
-                vn[u] = __ldg(d.val + j + kSpmmCH4 + u);
-              }
-          }
-#pragma unroll
-          for (int u = 0; u < kSpmmCH4; ++u)
-            if (j + u < k1) {
-              acc.x = fmaf(vv[u], xv[u].x, acc.x);
-              acc.y = fmaf(vv[u], xv[u].y, acc.y);
-              acc.z = fmaf(vv[u], xv[u].z, acc.z);
-              acc.w = fmaf(vv[u], xv[u].w, acc.w);
-            }
-          if (!CMRS_SPMM_PREFETCH) {
-#pragma unroll
-            for (int u = 0; u < kSpmmCH4; ++u)
-              if (j + kSpmmCH4 + u < k1) {
-                pn[u] = __ldg(d.packed + j + kSpmmCH4 + u);
-                vn[u] = __ldg(d.val + j + kSpmmCH4 + u);
-              }
-          }
-        }
-        Y4[(size_t)row * kv + col] = acc;
-      }
-    }
-  }
-}
+// A warp's stage.  Should a copy's bounded wait give up, the warp reads its
+// rows from global memory from then on, so the result does not depend on it.
+struct WarpStage {
+  char *mem;
+  uint64_t *bar;
+  StageInfo *info;
+  uint64_t pol;
+  uint32_t phase;
+  bool ok;
+};
 
 // Rows [row0, row1) of matrix d, processed by one warp.
-__device__ __forceinline__ void spmm_rows(const Desc &d, int row0, int row1, int lane) {
-  if (d.vec) {
-    spmm_rows4(d, row0, row1, lane);
-    return;
-  }
-  const int k = d.k;
-  const int G = spmm_lanes(k, 0);
-  const int per = 32 / G;
-  const int g = lane & (G - 1);
-  const int sub = lane / G;
+__device__ __forceinline__ void spmm_rows(const Desc &d, int row0, int row1, WarpStage &st) {
+  const unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int kv = d.vec ? d.k >> 2 : d.k;
+  const int G = spmm_lanes(d.k, d.vec);
+  const int L = d.split, per = 32 / (G * L);  // rows worked at once
+  const int g = lane & (G - 1), q = (lane / G) & (L - 1), sub = lane / (G * L);
   const uint32_t mask = (1u << d.bits) - 1;
-  for (int rb = row0; rb < row1; rb += per) {
-    const int row = rb + sub;
+  for (int ra = row0; ra < row1;) {
+    // lane r: row ra + r, its strip's bounds
+    const int row = ra + lane;
     const bool active = row < row1;
-    int k0 = 0, k1 = 0;
+    int a = 0, b = 0;
+    uint32_t r = 0;
     if (active) {
-      const int s = row / d.height;
-      const uint32_t r = (uint32_t)(row - s * d.height);
-      const int sa = __ldg(d.sp + s), sb = __ldg(d.sp + s + 1);
-      k0 = sa;
-      k1 = sb;
-      if (d.height > 1) {
-        k0 = lb_ris_g(d.packed, sa, sb, r, mask);
-        k1 = lb_ris_g(d.packed, k0, sb, r + 1, mask);
+      const int s = d.height == 1 ? row : (int)((unsigned)row / (unsigned)d.height);
+      r = (uint32_t)(row - s * d.height);
+      a = __ldg(d.sp + s);
+      b = __ldg(d.sp + s + 1);
+    }
+    // the rows whose strips fit the stage together: whole groups of `per` rows, or all that are left
+    const int base = __shfl_sync(kAll, a, 0);
+    int nr = 0;
+    if (d.stage && st.ok) {
+      nr = __popc(__ballot_sync(kAll, active && b - base <= kSpmmCap));
+      if (ra + nr < row1 && nr >= per) nr = nr / per * per;
+      if (2 * nr < min(per, row1 - ra)) nr = 0;  // a stage of too few rows leaves lanes idle
+    }
+    const bool staged = nr > 0;
+    if (!staged) nr = min(per, row1 - ra);
+    const uint32_t *cp = d.packed;
+    int cbase = 0;
+    bool use = staged;
+    if (staged) {
+      const int eb = __shfl_sync(kAll, b, nr - 1);
+      if (lane == 0)
+        issue_stage<CMRS_F32>(base, eb, d.nnz, d.packed, d.val, nullptr, st.mem, kSpmmCap, st.bar, st.pol, st.info);
+      if (__all_sync(kAll, mbar_wait_bounded(st.bar, st.phase))) {
+        st.phase ^= 1;
+      } else {
+        st.ok = use = false;
       }
     }
-    for (int c0 = 0; c0 < k; c0 += G) {
-      const int col = c0 + g;
-      if (active && col < k) {
-        // kSpmmCH entries per batch: their column words, values and X gathers
-        // are all issued before the FMAs that use them
-        float acc = 0.f;
-        for (int j = k0; j < k1; j += kSpmmCH) {
-          float xv[kSpmmCH], vv[kSpmmCH];
-#pragma unroll
-          for (int u = 0; u < kSpmmCH; ++u) {
-            if (j + u < k1) {
-              const uint32_t p = __ldg(d.packed + j + u);
-              vv[u] = __ldg(d.val + j + u);
-              xv[u] = __ldg(d.X + (size_t)(p >> d.bits) * k + col);
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < kSpmmCH; ++u)
-            if (j + u < k1) acc = fmaf(vv[u], xv[u], acc);
-        }
-        d.Y[(size_t)row * k + col] = acc;
+    if (use) {
+      cp = reinterpret_cast<const uint32_t *>(st.mem);
+      cbase = (int)st.info->a8;
+    }
+    int k0 = a, k1 = b;
+    if (d.height > 1 && active && lane < nr) {
+      k0 = lb_ris_g(cp, cbase, a, b, r, mask);
+      k1 = lb_ris_g(cp, cbase, k0, b, r + 1, mask);
+    }
+    for (int g0 = 0; g0 < nr; g0 += per) {
+      const int src = g0 + sub;
+      int q0 = __shfl_sync(kAll, k0, src & 31), q1 = __shfl_sync(kAll, k1, src & 31);
+      const bool mine = src < nr;
+      if (!mine) q0 = q1 = cbase;
+      const int out = mine ? ra + src : -1;
+      // compiled for the stage and for global memory, so that the former's reads are shared-memory loads
+      if (use) {
+        const uint32_t *sc = reinterpret_cast<const uint32_t *>(st.mem);
+        const float *sv = reinterpret_cast<const float *>(st.mem + Stage<CMRS_F32>::colp_bytes(kSpmmCap));
+        if (d.vec) spmm_row<float4>(d, out, q0, q1, cbase, sc, sv, g, G, q, L, kv);
+        else spmm_row<float>(d, out, q0, q1, cbase, sc, sv, g, G, q, L, kv);
+      } else {
+        if (d.vec) spmm_row<float4>(d, out, q0, q1, 0, d.packed, d.val, g, G, q, L, kv);
+        else spmm_row<float>(d, out, q0, q1, 0, d.packed, d.val, g, G, q, L, kv);
       }
     }
+    __syncwarp();  // every lane is done with the stage before the next copy lands in it
+    ra += nr;
   }
+}
+
+__device__ __forceinline__ WarpStage warp_stage(char *smem, uint64_t *bars, StageInfo *info) {
+  const int w = threadIdx.x >> 5;
+  WarpStage st;
+  st.mem = smem + (size_t)w * Stage<CMRS_F32>::bytes(kSpmmCap);
+  st.bar = &bars[w];
+  st.info = &info[w];
+  if ((threadIdx.x & 31) == 0) {
+    mbar_init(st.bar, 1);
+    fence_barrier_init();
+  }
+  __syncwarp();
+  st.pol = policy_evict_first();
+  st.phase = 0;
+  st.ok = true;
+  return st;
+}
+// a copy whose wait gave up lands before the warp leaves
+__device__ __forceinline__ void warp_stage_end(WarpStage &st) {
+  if (!st.ok) mbar_wait_bounded(st.bar, st.phase);
 }
 
 __global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_queue(const Desc *__restrict__ descs,
-                                                             const Unit *__restrict__ units, int nunits,
-                                                             QueueHead *q) {
+                                                                            const Unit *__restrict__ units, Shares sh,
+                                                                            QueueHead *q) {
+  extern __shared__ __align__(128) char smem[];
+  __shared__ uint64_t bars[kSpmmWarps];
+  __shared__ StageInfo info[kSpmmWarps];
+  WarpStage st = warp_stage(smem, bars, info);
+  const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
+  unsigned smid;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+  const int own = (int)(smid % (unsigned)sh.shares);
+  int share = own;
   for (;;) {
-    unsigned int u = 0;
-    if (lane == 0) u = atomicAdd(&q->next, 1u);
-    u = __shfl_sync(0xffffffffu, u, 0);
-    if (u >= (unsigned)nunits) break;
+    unsigned i = 0;
+    if (lane == 0) i = atomicAdd(&q->taken[share], 1u);
+    i = __shfl_sync(kAll, i, 0);
+    if (i >= (unsigned)sh.len) {
+      // used up: the next share, from this SM's on, with units left
+      int found = -1;
+      for (int k0 = 0; k0 < sh.shares && found < 0; k0 += 32) {
+        const int k = k0 + lane;
+        int s = own + k;
+        if (s >= sh.shares) s -= sh.shares;
+        const bool left = k < sh.shares && *reinterpret_cast<volatile unsigned *>(&q->taken[s]) < (unsigned)sh.len;
+        const unsigned m = __ballot_sync(kAll, left);
+        if (m) found = __shfl_sync(kAll, s, __ffs(m) - 1);
+      }
+      if (found < 0) break;
+      share = found;
+      continue;
+    }
+    const unsigned u = sh.unit(share, i);
+    if (u >= (unsigned)sh.nunits) continue;  // a block past the end
     const Unit un = units[u];
     const Desc d = descs[un.mat];
-    spmm_rows(d, un.row0, un.row1, lane);
+    spmm_rows(d, un.row0, un.row1, st);
   }
+  warp_stage_end(st);
 }
 
 // One matrix, no queue: warp w takes rows [w*rpw, (w+1)*rpw).
 __global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_one(Desc d, int rows_per_warp) {
-  const int lane = threadIdx.x & 31;
+  extern __shared__ __align__(128) char smem[];
+  __shared__ uint64_t bars[kSpmmWarps];
+  __shared__ StageInfo info[kSpmmWarps];
   const long long w = ((long long)blockIdx.x * kSpmmThreads + threadIdx.x) >> 5;
   const long long r0 = w * rows_per_warp;
   if (r0 >= d.rows) return;
+  WarpStage st = warp_stage(smem, bars, info);
   const int r1 = (int)std::min<long long>(r0 + rows_per_warp, d.rows);
-  spmm_rows(d, (int)r0, r1, lane);
+  spmm_rows(d, (int)r0, r1, st);
+  warp_stage_end(st);
+}
+
+int spmm_smem_opt_in() {
+  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_spmm_queue, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpmmSmem));
+  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_spmm_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpmmSmem));
+  return CMRS_OK;
 }
 
 int check_item(const cmrs_matrix *A, int k, const float *X, float *Y) {
@@ -257,7 +362,14 @@ Desc make_desc(const cmrs_matrix *A, int k, const float *X, float *Y) {
   d.X = X;
   d.Y = Y;
   d.vec = (k % 4 == 0) && !((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Y)) & 15);
-  d.pad = 0;
+  d.nnz = A->nnz;
+  d.stage = ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) == 0;
+  // Lanes per row: with one lane a row, 32 rows at once would need a stage four
+  // times as large (fewer warps, less L1 for X); rows too short to feed the
+  // lanes keep fewer.
+  const double mu = A->rows > 0 ? (double)A->nnz / A->rows : 0.0;
+  d.split = 1;
+  while (d.split < CMRS_SPMM_SPLIT && spmm_lanes(k, d.vec) * d.split < CMRS_SPMM_SPLIT && mu >= 8.0 * d.split) d.split <<= 1;
   return d;
 }
 
@@ -283,6 +395,7 @@ struct cmrs_spmm_plan {
   Unit *d_units = nullptr;
   QueueHead *d_q = nullptr;
   int grid = 0;
+  Shares sh = {};
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -298,10 +411,16 @@ extern "C" int cmrs_spmm(const cmrs_matrix *A, int k, const float *X, float *Y, 
     return CMRS_OK;
   }
   const Desc d = make_desc(A, k, X, Y);
-  const int rpw = 32 / spmm_lanes(k, d.vec);
+  // rows per warp: up to 32 (one stage), fewer while the warps would not fill
+  // the SMs twice, whole groups of the rows a warp works at once
+  const int per = 32 / (spmm_lanes(k, d.vec) * d.split);
+  const long long resident = (long long)sm_count() * CMRS_SPMM_MINB * kSpmmWarps;
+  const int rpw = (int)std::max<long long>(per, std::min<long long>(32, A->rows / (2 * resident)) / per * per);
   const long long warps = ceil_div(A->rows, rpw);
   const int grid = (int)ceil_div(warps * 32, kSpmmThreads);
-  k_spmm_one<<<grid, kSpmmThreads, 0, st>>>(d, rpw);
+  const int arc = spmm_smem_opt_in();
+  if (arc) return arc;
+  k_spmm_one<<<grid, kSpmmThreads, kSpmmSmem, st>>>(d, rpw);
   CMRS_LAUNCH_CHECK();
   return CMRS_OK;
 }
@@ -330,6 +449,34 @@ static int build_units(int batch, const cmrs_matrix *const *A, const int32_t *k,
     return w(x) > w(y);
   });
   return CMRS_OK;
+}
+
+// Shares of a plan's units: blocks of up to CMRS_SPMM_BLOCK units, smaller ones
+// while a share would hold fewer than eight.
+static Shares make_shares(size_t nunits) {
+  Shares sh;
+  sh.nunits = (int)nunits;
+  sh.shares = std::max(1, std::min(sm_count(), kMaxShares));
+  sh.block = std::max(1, std::min(CMRS_SPMM_BLOCK, sh.nunits / (8 * sh.shares)));
+  sh.len = (int)ceil_div(ceil_div(sh.nunits, sh.block), sh.shares) * sh.block;
+  return sh;
+}
+
+// Units of wide products are dealt one by one instead: where a row of X fills
+// whole lines (four or more 16-byte lanes), neighbouring rows on one SM find
+// few of each other's lines in L1, and their misses wait for each other there
+// (k = 32: 1,298 us in blocks of 64, 1,212 us one by one; k = 4: 374 us in
+// blocks, 423 us one by one).  The units of every full round over the shares
+// are reordered so that the blocks deal them that way.
+static void deal_wide(const Shares &sh, const int32_t *k, std::vector<Unit> &units) {
+  const size_t round = (size_t)sh.shares * sh.block;
+  std::vector<Unit> tmp(round);
+  for (size_t r0 = 0; r0 + round <= units.size(); r0 += round) {
+    const int ka = k[units[r0].mat], kb = k[units[r0 + round - 1].mat];
+    if (spmm_lanes(ka, ka % 4 == 0) < 4 || spmm_lanes(kb, kb % 4 == 0) < 4) continue;
+    for (size_t i = 0; i < round; ++i) tmp[i % sh.shares * sh.block + i / sh.shares] = units[r0 + i];
+    std::copy(tmp.begin(), tmp.end(), units.begin() + r0);
+  }
 }
 
 extern "C" int cmrs_spmm_plan_workspace(int batch, const cmrs_matrix *const *A, const int32_t *k, int work_target,
@@ -361,6 +508,8 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
   if (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255)) return CMRS_ERR_WORKSPACE;
   std::vector<Unit> units;
   build_units(batch, A, k, work_target, units);
+  const Shares sh = make_shares(units.size());
+  deal_wide(sh, k, units);
   std::vector<Desc> descs(batch);
   for (int b = 0; b < batch; ++b) descs[b] = make_desc(A[b], k[b], X[b], Y[b]);
   cmrs_spmm_plan *p = new (std::nothrow) cmrs_spmm_plan();
@@ -368,6 +517,7 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
   char *ws = reinterpret_cast<char *>(workspace);
   p->batch = batch;
   p->nunits = (int)units.size();
+  p->sh = sh;
   p->work_target = work_target;
   p->d_q = reinterpret_cast<QueueHead *>(ws);
   p->d_desc = reinterpret_cast<Desc *>(ws + align256(sizeof(QueueHead)));
@@ -383,8 +533,12 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
     delete p;
     return set_cuda_error(e);
   }
+  if (const int arc = spmm_smem_opt_in()) {
+    delete p;
+    return arc;
+  }
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmm_queue, kSpmmThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmm_queue, kSpmmThreads, kSpmmSmem);
   p->grid = std::max(1, per_sm) * sm_count();
   if (use_graph) {
     // the graph holds the queue reset and the persistent launch; replaying it
@@ -393,8 +547,8 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int), cap);
-      k_spmm_queue<<<p->grid, kSpmmThreads, 0, cap>>>(p->d_desc, p->d_units, p->nunits, p->d_q);
+      cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int) * p->sh.shares, cap);
+      k_spmm_queue<<<p->grid, kSpmmThreads, kSpmmSmem, cap>>>(p->d_desc, p->d_units, p->sh, p->d_q);
       e = cudaStreamEndCapture(cap, &p->graph);
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&p->exec, p->graph, 0);
@@ -417,8 +571,8 @@ extern "C" int cmrs_spmm_batched(cmrs_spmm_plan *p, void *stream) {
   if (p->exec) {
     CMRS_CUDA_TRY(cudaGraphLaunch(p->exec, st));
   } else {
-    CMRS_CUDA_TRY(cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int), st));
-    k_spmm_queue<<<p->grid, kSpmmThreads, 0, st>>>(p->d_desc, p->d_units, p->nunits, p->d_q);
+    CMRS_CUDA_TRY(cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int) * p->sh.shares, st));
+    k_spmm_queue<<<p->grid, kSpmmThreads, kSpmmSmem, st>>>(p->d_desc, p->d_units, p->sh, p->d_q);
     CMRS_LAUNCH_CHECK();
   }
   return CMRS_OK;
