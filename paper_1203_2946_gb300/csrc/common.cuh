@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
+#include <type_traits>
 
 #include "../../include/cmrs.h"
 
@@ -217,6 +218,37 @@ struct Form<CMRS_BF16X2> {
     return bf16_bits_to_float(hi[k]) + bf16_bits_to_float(lo[k]);
   }
 };
+
+// One chunk of 32 entries of a strip, rows r (valid lanes), in strip order:
+// each entry's place among the entries of its row, counted on from `next`
+// (lane q: row q's next place), which moves past the chunk.  NB: bits of the
+// row number.  One vote per bit instead of a match instruction: the votes also
+// give row q's count to lane q.
+template <int NB>
+__device__ __forceinline__ int place_in_row(int r, bool valid, int &next) {
+  const unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  unsigned peers = __ballot_sync(kAll, valid), mine = peers;
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    const bool one = (r >> k) & 1;
+    const unsigned v = __ballot_sync(kAll, one);
+    peers &= v ^ (one ? 0u : ~0u);
+    mine &= v ^ ((lane >> k) & 1 ? 0u : ~0u);
+  }
+  const int at = __shfl_sync(kAll, next, r & 31) + __popc(peers & ((1u << lane) - 1));
+  next += __popc(mine);
+  return at;
+}
+// f(NB) for the bits of a row number below nrow (1..5), as a compile-time constant
+template <typename F>
+__device__ __forceinline__ void with_row_bits(int nrow, F f) {
+  if (nrow <= 2) f(std::integral_constant<int, 1>());
+  else if (nrow <= 4) f(std::integral_constant<int, 2>());
+  else if (nrow <= 8) f(std::integral_constant<int, 3>());
+  else if (nrow <= 16) f(std::integral_constant<int, 4>());
+  else f(std::integral_constant<int, 5>());
+}
 
 __device__ __forceinline__ double fma_acc(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fma_acc(float a, float b, float c) { return fmaf(a, b, c); }

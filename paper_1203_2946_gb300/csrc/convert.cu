@@ -242,37 +242,6 @@ __device__ __forceinline__ bool strip_rows(int s, int rows, int nnz, int height,
   return __all_sync(kAll, lane >= R.nrow || (R.start >= 0 && R.end >= R.start && R.end <= nnz));
 }
 
-// One chunk of 32 entries of a strip, rows r (valid lanes), in strip order:
-// each entry's place among the entries of its row, counted on from `next`
-// (lane q: row q's next place), which moves past the chunk.  NB: bits of the
-// row number.  One vote per bit instead of a match instruction: the votes also
-// give row q's count to lane q.
-template <int NB>
-__device__ __forceinline__ int place_in_row(int r, bool valid, int &next) {
-  const unsigned kAll = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  unsigned peers = __ballot_sync(kAll, valid), mine = peers;
-#pragma unroll
-  for (int k = 0; k < NB; ++k) {
-    const bool one = (r >> k) & 1;
-    const unsigned v = __ballot_sync(kAll, one);
-    peers &= v ^ (one ? 0u : ~0u);
-    mine &= v ^ ((lane >> k) & 1 ? 0u : ~0u);
-  }
-  const int at = __shfl_sync(kAll, next, r & 31) + __popc(peers & ((1u << lane) - 1));
-  next += __popc(mine);
-  return at;
-}
-// f(NB) for the bits of a row number below nrow (1..5), as a compile-time constant
-template <typename F>
-__device__ __forceinline__ void with_row_bits(int nrow, F f) {
-  if (nrow <= 2) f(std::integral_constant<int, 1>());
-  else if (nrow <= 4) f(std::integral_constant<int, 2>());
-  else if (nrow <= 8) f(std::integral_constant<int, 3>());
-  else if (nrow <= 16) f(std::integral_constant<int, 4>());
-  else f(std::integral_constant<int, 5>());
-}
-
 __device__ __forceinline__ uint32_t word_of(uint32_t v) { return v; }
 __device__ __forceinline__ uint32_t word_of(uint2 v) { return v.x; }
 __device__ __forceinline__ void make_entry(uint32_t word, uint32_t, uint32_t &v) { v = word; }

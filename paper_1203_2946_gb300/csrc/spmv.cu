@@ -451,19 +451,35 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_spmv_lane(int rows, int hei
   const long long units = ((long long)rows + R - 1) / R;
   const long long nw = (long long)gridDim.x * kLaneWarps;
   uint32_t phase = 0;
-  for (long long u = (long long)blockIdx.x * kLaneWarps + w; u < units; u += nw) {
-    const long long r0 = u * R;
-    const long long r1 = min(r0 + R, (long long)rows);
-    const int s0 = (int)(r0 / height), s1 = (int)((r1 - 1) / height) + 1;  // the unit's strips
-    const int ea = sp[s0], eb = sp[s1];
-    const bool staged = eb - ea <= cap;  // warp-uniform
-    if (staged && lane == 0) issue_stage<DT>(ea, eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
-    // this lane's row and its strip's bounds, loaded while the copy is in flight
-    const long long row = r0 + slot;
+  // Strip bounds of a unit: the unit's own (its first and last strip's) and of
+  // this lane's row's strip.  Loaded a unit ahead, so that a unit starts with
+  // its copy instead of a round trip for StripPtr.
+  struct Bounds {
+    int ea, eb, sa, sb;
+  };
+  auto bounds = [&](long long u) {
+    const long long r0 = u * R, r1 = min(r0 + R, (long long)rows), row = r0 + slot;
+    const int s0 = (int)((unsigned)r0 / (unsigned)height), s1 = (int)((unsigned)(r1 - 1) / (unsigned)height) + 1;
+    Bounds B;
+    B.ea = sp[s0];
+    B.eb = sp[s1];
+    const int s = row < rows ? (int)((unsigned)row / (unsigned)height) : s0;
+    B.sa = row < rows ? sp[s] : 0;
+    B.sb = row < rows ? sp[s + 1] : 0;
+    return B;
+  };
+  long long u = (long long)blockIdx.x * kLaneWarps + w;
+  Bounds next = {0, 0, 0, 0};
+  if (u < units) next = bounds(u);
+  for (; u < units; u += nw) {
+    const Bounds B = next;
+    const bool staged = B.eb - B.ea <= cap;  // warp-uniform
+    if (staged && lane == 0) issue_stage<DT>(B.ea, B.eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
+    if (u + nw < units) next = bounds(u + nw);
+    const long long row = u * R + slot;
     const bool active = row < rows;
-    const int s = active ? (int)(row / height) : s0;
-    const uint32_t rr = active ? (uint32_t)(row - (long long)s * height) : 0;
-    const int sa = active ? sp[s] : 0, sb = active ? sp[s + 1] : 0;
+    const uint32_t rr = active ? (uint32_t)row % (uint32_t)height : 0;
+    const int sa = B.sa, sb = B.sb;
     bool ok = true;
     if (staged) {
       ok = __all_sync(kAll, mbar_wait_bounded(&bars[w], phase));
@@ -512,6 +528,63 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_spmv_lane(int rows, int hei
 #define CMRS_STRIP_U 4
 #endif
 constexpr int kStripU = CMRS_STRIP_U;
+// One strip by one warp; buf: height * 32 sums of shared memory.
+template <int DT>
+__device__ __forceinline__ void strip_sums(int s, int rows, int height, int bits, const int32_t *__restrict__ sp,
+                                           const uint32_t *__restrict__ packed,
+                                           const typename Form<DT>::Stored *__restrict__ hi,
+                                           const typename Form<DT>::Stored *__restrict__ vl,
+                                           const typename Form<DT>::Acc *__restrict__ x,
+                                           typename Form<DT>::Acc *__restrict__ y,
+                                           const int32_t *__restrict__ row_map, typename Form<DT>::Acc *buf) {
+  typedef typename Form<DT>::Acc A;
+  const int lane = threadIdx.x & 31;
+  const uint32_t mask = (1u << bits) - 1;
+  for (int r = 0; r < height; ++r) buf[r * 32 + lane] = A(0);
+  const int a = sp[s], b = sp[s + 1];
+  for (int j0 = a; j0 < b; j0 += 32 * kStripU) {  // kStripU steps' loads in flight
+    uint32_t c[kStripU];
+    A v[kStripU], xv[kStripU];
+#pragma unroll
+    for (int u = 0; u < kStripU; ++u) {
+      const int j = j0 + 32 * u + lane;
+      if (j < b) {
+        c[u] = packed[j];
+        v[u] = Form<DT>::value(hi, vl, j);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kStripU; ++u)
+      if (j0 + 32 * u + lane < b) xv[u] = ld_x(x + (c[u] >> bits));
+#pragma unroll
+    for (int u = 0; u < kStripU; ++u) {
+      if (j0 + 32 * u + lane < b) {
+        const int r = (int)(c[u] & mask);
+        if (r < height) {
+          A *p = buf + r * 32 + lane;
+          *p = fma_acc(v[u], xv[u], *p);
+        }
+      }
+    }
+  }
+  __syncwarp();
+  for (int half = 16; half >= 1; half >>= 1) {
+    for (int idx = lane; idx < height * half; idx += 32) {
+      const int r = idx / half, l = idx - r * half;
+      buf[r * 32 + l] += buf[r * 32 + l + half];
+    }
+    __syncwarp();
+  }
+  if (lane < height) {
+    const long long row = (long long)s * height + lane;
+    if (row < rows) {
+      const long long t = row_map ? row_map[row] : row;
+      if (t >= 0 && t < rows) y[t] = buf[lane * 32];
+    }
+  }
+  __syncwarp();
+}
+
 template <int DT>
 __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int height, int bits, int strips,
                                                                   const int32_t *__restrict__ sp,
@@ -523,55 +596,217 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
                                                                   const int32_t *__restrict__ row_map) {
   typedef typename Form<DT>::Acc A;
   extern __shared__ __align__(128) char smem[];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int w = threadIdx.x >> 5;
   A *buf = reinterpret_cast<A *>(smem) + (size_t)w * height * 32;
-  const uint32_t mask = (1u << bits) - 1;
   const int nw = gridDim.x * kStripWarps;
-  const typename Form<DT>::Stored *vl = Stage<DT>::kSplit ? lo : hi;
-  for (int s = blockIdx.x * kStripWarps + w; s < strips; s += nw) {
-    for (int r = 0; r < height; ++r) buf[r * 32 + lane] = A(0);
-    const int a = sp[s], b = sp[s + 1];
-    for (int j0 = a; j0 < b; j0 += 32 * kStripU) {  // kStripU steps' loads in flight
-      uint32_t c[kStripU];
-      A v[kStripU], xv[kStripU];
-#pragma unroll
-      for (int u = 0; u < kStripU; ++u) {
-        const int j = j0 + 32 * u + lane;
-        if (j < b) {
-          c[u] = packed[j];
-          v[u] = Form<DT>::value(hi, vl, j);
-        }
+  for (int s = blockIdx.x * kStripWarps + w; s < strips; s += nw)
+    strip_sums<DT>(s, rows, height, bits, sp, packed, hi, Stage<DT>::kSplit ? lo : hi, x, y, row_map, buf);
+}
+
+// ============================================================== SORTED mapping
+// Column-sorted strips with short rows (the STRIP variant on CMRS_SORTED
+// matrices).  Algorithm 1's reduction costs 31 height adds per strip, and on
+// this GPU an FP64 warp instruction costs its issue slot whatever its active
+// lanes do: with rows of 27 entries the reduction and the steps' partly filled
+// multiply-adds are two thirds of the FP64 pipe's time (27-point 128^3, h = 4:
+// 353 us).  Here a warp takes R = 32 / L rows, or the whole strips below that,
+// stages their entries by one bulk copy, and finds each row's entries there
+// with integer work only; L lanes then walk each row in column order, one
+// multiply-add per entry and lane, the row's sum in a register (FP32 forms: four sums, joined at the end,
+// so that their chains stay as short as the paper's 32 partial sums of a
+// strip keep them).  x is gathered at the same place of consecutive rows.
+//   An entry's place among its row's entries is found and its index left in
+// list[place][row]; the lanes of a row take every L-th place.  Heights up to 8
+// (kPack): each strip is cut into P parts, a lane each, and every lane counts
+// its part's entries per row in one packed register (8 bits a row); a scan of
+// the packed counts over the strip's lanes gives each lane its first places,
+// and a second walk of its part hands them out -- about 16 instructions per
+// entry and lane, where a vote per bit of the row over 32 entries (larger
+// heights, place_in_row) takes about 40.
+//   A unit longer than its stage, or with a row longer than the list (or a
+// packed count), runs Algorithm 1 strip by strip.
+#ifndef CMRS_SORTED_WARPS
+#define CMRS_SORTED_WARPS 4
+#endif
+#ifndef CMRS_SORTED_CAP
+#define CMRS_SORTED_CAP 1024  // most entries per warp stage
+#endif
+#ifndef CMRS_SORTED_MU1
+#define CMRS_SORTED_MU1 14.0  // mean entries per row up to which a lane takes a row alone
+#endif
+#ifndef CMRS_SORTED_CH_F64
+#define CMRS_SORTED_CH_F64 7
+#endif
+#ifndef CMRS_SORTED_CTAS
+#define CMRS_SORTED_CTAS 0
+#endif
+#ifndef CMRS_SORTED_MINB
+#define CMRS_SORTED_MINB 6
+#endif
+constexpr int kSortedWarps = CMRS_SORTED_WARPS;
+// kPack: bytes of the packed counts, 4 (heights up to 4), 8 (up to 8), 0 (votes)
+template <int DT, int L, int kPack>
+__global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_sorted(int rows, int height, int bits, int strips, int cap,
+                                                                   int ml, int warp_bytes, int nnz,
+                                                                   const int32_t *__restrict__ sp,
+                                                                   const uint32_t *__restrict__ packed,
+                                                                   const typename Form<DT>::Stored *__restrict__ hi,
+                                                                   const typename Form<DT>::Stored *__restrict__ lo,
+                                                                   const typename Form<DT>::Acc *__restrict__ x,
+                                                                   typename Form<DT>::Acc *__restrict__ y,
+                                                                   const int32_t *__restrict__ row_map,
+                                                                   uint32_t *status) {
+  typedef typename Form<DT>::Stored S;
+  typedef typename Form<DT>::Acc A;
+  constexpr int CH = DT == CMRS_F64 ? CMRS_SORTED_CH_F64 : 8;
+  constexpr int kAcc = DT == CMRS_F64 ? 1 : 4;
+  constexpr int RS = 32 / L + 2;  // the list's row stride: an odd number of words
+  extern __shared__ __align__(128) char smem[];
+  __shared__ uint64_t bars[kSortedWarps];
+  __shared__ StageInfo info[kSortedWarps];
+  const unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  char *stg = smem + (size_t)w * warp_bytes;
+  uint16_t *list = reinterpret_cast<uint16_t *>(stg + Stage<DT>::bytes(cap));
+  const uint32_t mask = (1u << bits) - 1;
+  if (lane == 0) {
+    mbar_init(&bars[w], 1);
+    fence_barrier_init();
+  }
+  __syncwarp();
+  uint64_t pol = 0;
+  if (lane == 0) pol = policy_evict_first();
+  const int ns = 32 / L / height, R = ns * height;  // strips and rows per unit
+  const int q = lane & (L - 1), slot = lane / L;
+  const int units = (strips + ns - 1) / ns, nw = gridDim.x * kSortedWarps;
+  const uint32_t *cp = reinterpret_cast<const uint32_t *>(stg);
+  const S *vh = reinterpret_cast<const S *>(stg + Stage<DT>::colp_bytes(cap));
+  const S *vl = reinterpret_cast<const S *>(stg + Stage<DT>::colp_bytes(cap) + Stage<DT>::val_bytes(cap));
+  uint32_t phase = 0;
+  int u = blockIdx.x * kSortedWarps + w;
+  // the unit's strip bounds (ns <= 16: the height is at least 2), loaded a unit ahead
+  int nbound = u < units ? sp[min(u * ns + min(lane, ns), strips)] : 0;
+  for (; u < units; u += nw) {
+    const int s0 = u * ns, n_s = min(ns, strips - s0);
+    const int bound = nbound;
+    if (u + nw < units) nbound = sp[min((u + nw) * ns + min(lane, ns), strips)];
+    const int ea = __shfl_sync(kAll, bound, 0), eb = __shfl_sync(kAll, bound, n_s);
+    bool listed = eb - ea <= cap;  // warp-uniform
+    if (listed) {
+      if (lane == 0) issue_stage<DT>(ea, eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
+      if (!__all_sync(kAll, mbar_wait_bounded(&bars[w], phase))) {
+        if (lane == 0) atomicOr(status, ST_TIMEOUT);
+        break;
       }
+      phase ^= 1;
+      const int base = (int)info[w].a8;
+      int len = 0;  // of this lane's row
+      if constexpr (kPack > 0) {
+        typedef typename std::conditional<kPack == 4, uint32_t, unsigned long long>::type C;
+        const int P = 32 / ns;  // lanes per strip
+        const int j = lane / P, p = lane - j * P;
+        const int a = __shfl_sync(kAll, bound, min(j, n_s)) - base, b = __shfl_sync(kAll, bound, min(j + 1, n_s)) - base;
+        const int seg = ((b - a + P - 1) / P) | 1;  // odd: the lanes' reads hit all banks
+        const int a0 = min(b, a + p * seg), b0 = min(b, a0 + seg);
+        C count = 0;
+#pragma unroll 4
+        for (int i = a0; i < b0; ++i) {
+          const uint32_t r = cp[i] & mask;
+          if (r < (uint32_t)height) count += C(1) << (8 * r);
+        }
+        C incl = count;
+        for (int o = 1; o < P; o <<= 1) {
+          const C t = __shfl_up_sync(kAll, incl, o);
+          if (p >= o) incl += t;
+        }
+        const C total = __shfl_sync(kAll, incl, min(j * P + P - 1, 31));
+        // a count past 255 carries into the next row's and the sum comes out short
+        int sum = 0;
 #pragma unroll
-      for (int u = 0; u < kStripU; ++u)
-        if (j0 + 32 * u + lane < b) xv[u] = ld_x(x + (c[u] >> bits));
-#pragma unroll
-      for (int u = 0; u < kStripU; ++u) {
-        if (j0 + 32 * u + lane < b) {
-          const int r = (int)(c[u] & mask);
-          if (r < height) {
-            A *p = buf + r * 32 + lane;
-            *p = fma_acc(v[u], xv[u], *p);
+        for (int k = 0; k < kPack; ++k) sum += (int)(total >> (8 * k)) & 255;
+        listed = !__any_sync(kAll, sum != b - a);
+        C place = incl - count;
+#pragma unroll 4
+        for (int i = a0; i < b0; ++i) {
+          const uint32_t r = cp[i] & mask;
+          if (r < (uint32_t)height) {
+            const int at = (int)(place >> (8 * r)) & 255;
+            place += C(1) << (8 * r);
+            if (at < ml) list[at * RS + j * height + (int)r] = (uint16_t)i;
           }
         }
+        const int js = slot / height;  // this lane's row: strip js, row slot - js * height
+        const C t = __shfl_sync(kAll, total, min(js * P, 31));
+        if (js < n_s) len = (int)(t >> (8 * (slot - js * height))) & 255;
+      } else {
+        int rl = 0;  // of row `lane`
+        with_row_bits(height, [&](auto nb) {
+          for (int j = 0; j < n_s; ++j) {
+            const int a = __shfl_sync(kAll, bound, j) - base, b = __shfl_sync(kAll, bound, j + 1) - base;
+            int next = 0;
+            for (int i0 = a; i0 < b; i0 += 32) {
+              const int i = i0 + lane;
+              const uint32_t r = i < b ? cp[i] & mask : 0u;
+              const bool valid = i < b && r < (uint32_t)height;
+              const int at = place_in_row<decltype(nb)::value>((int)r, valid, next);
+              if (valid && at < ml) list[at * RS + j * height + (int)r] = (uint16_t)i;
+            }
+            const int t = __shfl_sync(kAll, next, (lane - j * height) & 31);
+            if (lane >= j * height && lane < (j + 1) * height) rl = t;
+          }
+        });
+        len = __shfl_sync(kAll, rl, slot);
+      }
+      listed = listed && !__any_sync(kAll, slot < R && len > ml);
+      if (listed) {
+        __syncwarp();
+        const long long row = (long long)s0 * height + slot;
+        const bool active = slot < R && row < rows;
+        const int n = active && len > q ? (len - q + L - 1) / L : 0;  // this lane's entries
+        const int nmax = __reduce_max_sync(kAll, n);
+        const uint16_t *l = list + slot + q * RS;
+        A acc[kAcc];
+#pragma unroll
+        for (int k = 0; k < kAcc; ++k) acc[k] = A(0);
+        // FP64: whole batches, then the last, shorter one entry by entry (see seg_dot)
+        const int nfull = DT == CMRS_F64 ? nmax - nmax % CH : nmax;
+        for (int j0 = 0; j0 < nfull; j0 += CH) {
+          int i[CH];
+          A xv[CH];
+#pragma unroll
+          for (int k = 0; k < CH; ++k)
+            if (j0 + k < n) {
+              i[k] = l[(j0 + k) * (L * RS)];
+              xv[k] = ld_x(x + (cp[i[k]] >> bits));
+            }
+#pragma unroll
+          for (int k = 0; k < CH; ++k)
+            if (j0 + k < nmax) {  // warp-uniform
+              if (j0 + k < n) acc[k % kAcc] = fma_acc(Form<DT>::value(vh, vl, i[k]), xv[k], acc[k % kAcc]);
+            }
+        }
+#pragma unroll 1
+        for (int j = nfull; j < nmax; ++j)
+          if (j < n) {
+            const int i = l[j * (L * RS)];
+            acc[0] = fma_acc(Form<DT>::value(vh, vl, i), ld_x(x + (cp[i] >> bits)), acc[0]);
+          }
+        if constexpr (kAcc == 4) acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+        for (int o = L / 2; o >= 1; o >>= 1) acc[0] += __shfl_down_sync(kAll, acc[0], o);
+        if (active && q == 0) {
+          const long long t = row_map ? row_map[row] : row;  // y position (row map of a reordered matrix)
+          if (t >= 0 && t < rows) y[t] = acc[0];
+        }
       }
     }
-    __syncwarp();
-    for (int half = 16; half >= 1; half >>= 1) {
-      for (int idx = lane; idx < height * half; idx += 32) {
-        const int r = idx / half, l = idx - r * half;
-        buf[r * 32 + l] += buf[r * 32 + l + half];
-      }
+    if (!listed) {
       __syncwarp();
+      for (int s = s0; s < s0 + n_s; ++s)
+        strip_sums<DT>(s, rows, height, bits, sp, packed, hi, Stage<DT>::kSplit ? lo : hi, x, y, row_map,
+                       reinterpret_cast<A *>(stg));
     }
-    if (lane < height) {
-      const long long row = (long long)s * height + lane;
-      if (row < rows) {
-        const long long t = row_map ? row_map[row] : row;
-        if (t >= 0 && t < rows) y[t] = buf[lane * 32];
-      }
-    }
-    __syncwarp();
+    __syncwarp();  // every lane is done with the stage before the next copy lands in it
   }
 }
 
@@ -1456,6 +1691,46 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
   return launch_pdl(k_merge_fixup<Acc>, (unsigned)ceil_div(ntiles, 256), 256, 0, st, ntiles, A->rows, recs, y);
 }
 
+// Lanes per row of the SORTED mapping, 0 where Algorithm 1 runs instead:
+// unsorted or padded strips, heights of 1 or too large for the lanes a row of
+// this mean length needs, arrays the bulk copies cannot read.
+template <int DT>
+int sorted_lanes(const cmrs_matrix *A) {
+  if (!(A->flags & CMRS_SORTED) || A->height < 2 || A->rows < 1) return 0;
+  if ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) return 0;
+  const double mu = (double)A->nnz / A->rows;
+  int L = mu <= CMRS_SORTED_MU1 ? 1 : mu <= 2 * CMRS_LANE_MAX_MU ? 2 : mu <= 4 * CMRS_LANE_MAX_MU ? 4 : 0;
+  if (L > 1 && A->height * L > 32) L = mu <= CMRS_LANE_MAX_MU ? 1 : 0;
+  return L;
+}
+
+template <int DT, int L, int kPack>
+int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, const typename Form<DT>::Stored *lo,
+                  const typename Form<DT>::Acc *x, typename Form<DT>::Acc *y, const int32_t *row_map, uint32_t *status,
+                  cudaStream_t st) {
+  typedef typename Form<DT>::Acc Acc;
+  const double mu = (double)A->nnz / A->rows;
+  const int ns = 32 / L / A->height;
+  // stage: 1.25x an average unit; list: rows of 1.25x the mean and some; at
+  // least Algorithm 1's buffer
+  const int cap = (int)std::min<long long>(CMRS_SORTED_CAP,
+                                           std::max<long long>(128, ceil_div((long long)(1.25 * mu * ns * A->height), 32) * 32));
+  const int ml = (int)(1.25 * mu) + 8;
+  const size_t list = ((size_t)ml * (32 / L + 2) * 2 + 127) & ~size_t(127);
+  const size_t warp_bytes = std::max(Stage<DT>::bytes(cap) + list, (size_t)A->height * 32 * sizeof(Acc));
+  const size_t smem = kSortedWarps * warp_bytes;
+  static Occ occ[256];  // by the warp's bytes, in units of 128: at most 19 KB
+  const int per_sm = occupancy(k_spmv_sorted<DT, L, kPack>, kSortedWarps * 32, smem,
+                               occ[std::min<size_t>(warp_bytes / 128, 255)], 128 * 1024, CMRS_SORTED_CTAS);
+  const long long need = ceil_div(ceil_div(A->strips, ns), kSortedWarps);
+  const int grid = (int)std::min<long long>(need, (long long)per_sm * sm_count());
+  k_spmv_sorted<DT, L, kPack><<<grid, kSortedWarps * 32, smem, st>>>(A->rows, A->height, A->bits, A->strips, cap, ml,
+                                                              (int)warp_bytes, A->nnz, A->strip_ptr, A->col_packed, hi,
+                                                              lo, x, y, row_map, status);
+  CMRS_LAUNCH_CHECK();
+  return CMRS_OK;
+}
+
 template <int DT>
 int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_map, int variant, char *ws,
            size_t ws_bytes, cudaStream_t st) {
@@ -1506,6 +1781,19 @@ int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_ma
     k_spmv_row<DT><<<grid, RowCfg<DT>::kThreads, smem, st>>>(A->rows, A->height, A->bits, A->nnz, A->strip_ptr,
                                                              A->col_packed, hi, lo, x, y, row_map, status);
     CMRS_LAUNCH_CHECK();
+  } else if (variant == CMRS_VARIANT_STRIP && sorted_lanes<DT>(A)) {
+    const int lanes_s = sorted_lanes<DT>(A);
+    const int h = A->height;
+    if (lanes_s == 1)
+      return h <= 4   ? launch_sorted<DT, 1, 4>(A, hi, lo, x, y, row_map, status, st)
+             : h <= 8 ? launch_sorted<DT, 1, 8>(A, hi, lo, x, y, row_map, status, st)
+                      : launch_sorted<DT, 1, 0>(A, hi, lo, x, y, row_map, status, st);
+    if (lanes_s == 2)
+      return h <= 4   ? launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st)
+             : h <= 8 ? launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st)
+                      : launch_sorted<DT, 2, 0>(A, hi, lo, x, y, row_map, status, st);
+    return h <= 4 ? launch_sorted<DT, 4, 4>(A, hi, lo, x, y, row_map, status, st)  // heights up to 8
+                  : launch_sorted<DT, 4, 8>(A, hi, lo, x, y, row_map, status, st);
   } else if (variant == CMRS_VARIANT_STRIP) {
     static Occ occ;
     const size_t smem = (size_t)kStripWarps * A->height * 32 * sizeof(Acc);
