@@ -274,8 +274,8 @@ __global__ void __launch_bounds__(RowCfg<DT>::kThreads) k_spmv_row(int rows, int
     auto bounds = [&](int b, long long &ea, long long &eb) {
       const long long r0 = (long long)b * kRowThreads;
       const long long r1 = min(r0 + kRowThreads, (long long)rows);
-      ea = sp[(int)(r0 / height)];
-      eb = sp[(int)((r1 - 1) / height) + 1];
+      ea = sp[(int)((unsigned)r0 / (unsigned)height)];  // row numbers fit 32 unsigned bits
+      eb = sp[(int)((unsigned)(r1 - 1) / (unsigned)height) + 1];
     };
     long long ea = 0, eb = 0, nea = 0, neb = 0;
     int b = blockIdx.x;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(RowCfg<DT>::kThreads) k_spmv_row(int rows, int
   if (RowCfg<DT>::kPrefetch && blockIdx.x < (unsigned)nblk) {
     const long long row0 = (long long)blockIdx.x * kRowThreads + rloc;
     if (row0 < rows) {
-      const int s0 = (int)(row0 / height);
+      const int s0 = (int)((unsigned)row0 / (unsigned)height);
       nsa = sp[s0];
       nsb = sp[s0 + 1];
     }
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(RowCfg<DT>::kThreads) k_spmv_row(int rows, int
     const int st = it % kRowStages, use = it / kRowStages;
     const long long row = (long long)b * kRowThreads + rloc;
     const bool active = row < rows;
-    const int s = active ? (int)(row / height) : 0;
+    const int s = active ? (int)((unsigned)row / (unsigned)height) : 0;
     const uint32_t r = (uint32_t)(row - (long long)s * height);
     int sa = nsa, sb = nsb;
     if (!RowCfg<DT>::kPrefetch) {
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(RowCfg<DT>::kThreads) k_spmv_row(int rows, int
     } else {
       const long long rown = row + (long long)gridDim.x * kRowThreads;
       if (rown < rows) {
-        const int sn = (int)(rown / height);
+        const int sn = (int)((unsigned)rown / (unsigned)height);
         nsa = sp[sn];
         nsb = sp[sn + 1];
       }
@@ -451,35 +451,22 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_spmv_lane(int rows, int hei
   const long long units = ((long long)rows + R - 1) / R;
   const long long nw = (long long)gridDim.x * kLaneWarps;
   uint32_t phase = 0;
-  // Strip bounds of a unit: the unit's own (its first and last strip's) and of
-  // this lane's row's strip.  Loaded a unit ahead, so that a unit starts with
-  // its copy instead of a round trip for StripPtr.
-  struct Bounds {
-    int ea, eb, sa, sb;
-  };
-  auto bounds = [&](long long u) {
-    const long long r0 = u * R, r1 = min(r0 + R, (long long)rows), row = r0 + slot;
-    const int s0 = (int)((unsigned)r0 / (unsigned)height), s1 = (int)((unsigned)(r1 - 1) / (unsigned)height) + 1;
-    Bounds B;
-    B.ea = sp[s0];
-    B.eb = sp[s1];
-    const int s = row < rows ? (int)((unsigned)row / (unsigned)height) : s0;
-    B.sa = row < rows ? sp[s] : 0;
-    B.sb = row < rows ? sp[s + 1] : 0;
-    return B;
-  };
-  long long u = (long long)blockIdx.x * kLaneWarps + w;
-  Bounds next = {0, 0, 0, 0};
-  if (u < units) next = bounds(u);
-  for (; u < units; u += nw) {
-    const Bounds B = next;
-    const bool staged = B.eb - B.ea <= cap;  // warp-uniform
-    if (staged && lane == 0) issue_stage<DT>(B.ea, B.eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
-    if (u + nw < units) next = bounds(u + nw);
-    const long long row = u * R + slot;
+  for (long long u = (long long)blockIdx.x * kLaneWarps + w; u < units; u += nw) {
+    const long long r0 = u * R;
+    const long long r1 = min(r0 + R, (long long)rows);
+    // the unit's strips (row numbers fit 32 unsigned bits: 64-bit divisions here, three a unit, cost 6% of the
+    // kernel's time on rows of 27 entries and of 5)
+    const unsigned h = (unsigned)height;
+    const int s0 = (int)((unsigned)r0 / h), s1 = (int)((unsigned)(r1 - 1) / h) + 1;
+    const int ea = sp[s0], eb = sp[s1];
+    const bool staged = eb - ea <= cap;  // warp-uniform
+    if (staged && lane == 0) issue_stage<DT>(ea, eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
+    // this lane's row and its strip's bounds, loaded while the copy is in flight
+    const long long row = r0 + slot;
     const bool active = row < rows;
-    const uint32_t rr = active ? (uint32_t)row % (uint32_t)height : 0;
-    const int sa = B.sa, sb = B.sb;
+    const int s = active ? (int)((unsigned)row / h) : s0;
+    const uint32_t rr = active ? (uint32_t)row - (uint32_t)s * h : 0;
+    const int sa = active ? sp[s] : 0, sb = active ? sp[s + 1] : 0;
     bool ok = true;
     if (staged) {
       ok = __all_sync(kAll, mbar_wait_bounded(&bars[w], phase));
