@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // this GPU an FP64 warp instruction costs its issue slot whatever its active
 // lanes do: with rows of 27 entries the reduction and the steps' partly filled
 // multiply-adds are two thirds of the FP64 pipe's time (27-point 128^3, h = 4:
-// 353 us).  Here a warp takes R = 32 / L rows, or the whole strips below that,
+// 355 us; 219 us here, bound by instructions).  Here a warp takes R = 32 / L rows, or the whole strips below that,
 // stages their entries by one bulk copy, and finds each row's entries there
 // with integer work only; L lanes then walk each row in column order, one
 // multiply-add per entry and lane, the row's sum in a register (FP32 forms: four sums, joined at the end,
@@ -617,9 +617,6 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 #endif
 #ifndef CMRS_SORTED_CAP
 #define CMRS_SORTED_CAP 1024  // most entries per warp stage
-#endif
-#ifndef CMRS_SORTED_MU1
-#define CMRS_SORTED_MU1 14.0  // mean entries per row up to which a lane takes a row alone
 #endif
 #ifndef CMRS_SORTED_CH_F64
 #define CMRS_SORTED_CH_F64 7
@@ -1679,16 +1676,31 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
 }
 
 // Lanes per row of the SORTED mapping, 0 where Algorithm 1 runs instead:
-// unsorted or padded strips, heights of 1 or too large for the lanes a row of
-// this mean length needs, arrays the bulk copies cannot read.
+// unsorted or padded strips, arrays the bulk copies cannot read, and
+//   - rows too long for their height: Algorithm 1's reduction costs a strip 31
+//     adds per row whatever the rows' length, undoing the sort costs every
+//     entry, and by votes (heights past 8) twice as much.  1M rows, Algorithm 1
+//     against this mapping, us: 7-point FP64 246 -> 33, 132 -> 33, 89 -> 48 at
+//     h = 2, 4, 16, FP32 136 -> 25, 77 -> 25, 61 -> 38; rows of 8..20 FP64 157
+//     -> 72, 104 -> 91 at h = 4, 16, FP32 83 -> 50, 68 -> 68; 27-point FP64 171
+//     -> 104, 136 -> 111, 128 -> 150 at h = 4, 8, 16, FP32 147 -> 79, 87 -> 80,
+//     79 -> 86 at h = 2, 4, 8; rows of 20..60 FP64 300 -> 210, 202 -> 202 at h
+//     = 2, 4, FP32 155 -> 133, 108 -> 126;
+//   - few units: a unit's copy, walks and gathers take 4..7 us one after
+//     another (100,000 rows: 27-point FP64 h = 4 18.5 -> 12.3 us, FP32 9.6 ->
+//     9.7; 64,000 rows of 8..20: 12.0 -> 8.8, 7.0 -> 6.5; 16,000 rows of 7:
+//     FP32 3.2 -> 3.4).
 template <int DT>
 int sorted_lanes(const cmrs_matrix *A) {
+  constexpr bool kF64 = DT == CMRS_F64;
   if (!(A->flags & CMRS_SORTED) || A->height < 2 || A->rows < 1) return 0;
   if ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) return 0;
   const double mu = (double)A->nnz / A->rows;
-  int L = mu <= CMRS_SORTED_MU1 ? 1 : mu <= 2 * CMRS_LANE_MAX_MU ? 2 : mu <= 4 * CMRS_LANE_MAX_MU ? 4 : 0;
-  if (L > 1 && A->height * L > 32) L = mu <= CMRS_LANE_MAX_MU ? 1 : 0;
-  return L;
+  const int highest = mu <= (kF64 ? 14.0 : 10.0) ? 32 : mu <= 14.0 ? 8 : mu <= 28.0 ? (kF64 ? 8 : 4) : mu <= 56.0 ? 3 : 0;
+  if (A->height > highest) return 0;
+  const int L = mu <= 14.0 ? 1 : 2;
+  const long long units = ceil_div(A->strips, 32 / L / A->height);
+  return units >= (L == 1 ? 8LL : kF64 ? 40LL : 100LL) * sm_count() ? L : 0;
 }
 
 template <int DT, int L, int kPack>
@@ -1698,11 +1710,11 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   typedef typename Form<DT>::Acc Acc;
   const double mu = (double)A->nnz / A->rows;
   const int ns = 32 / L / A->height;
-  // stage: 1.25x an average unit; list: rows of 1.25x the mean and some; at
+  // stage: 1.25x an average unit; list: rows of 1.5x the mean and 16 more; at
   // least Algorithm 1's buffer
   const int cap = (int)std::min<long long>(CMRS_SORTED_CAP,
                                            std::max<long long>(128, ceil_div((long long)(1.25 * mu * ns * A->height), 32) * 32));
-  const int ml = (int)(1.25 * mu) + 8;
+  const int ml = (int)(1.5 * mu) + 16;
   const size_t list = ((size_t)ml * (32 / L + 2) * 2 + 127) & ~size_t(127);
   const size_t warp_bytes = std::max(Stage<DT>::bytes(cap) + list, (size_t)A->height * 32 * sizeof(Acc));
   const size_t smem = kSortedWarps * warp_bytes;
@@ -1775,12 +1787,8 @@ int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_ma
       return h <= 4   ? launch_sorted<DT, 1, 4>(A, hi, lo, x, y, row_map, status, st)
              : h <= 8 ? launch_sorted<DT, 1, 8>(A, hi, lo, x, y, row_map, status, st)
                       : launch_sorted<DT, 1, 0>(A, hi, lo, x, y, row_map, status, st);
-    if (lanes_s == 2)
-      return h <= 4   ? launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st)
-             : h <= 8 ? launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st)
-                      : launch_sorted<DT, 2, 0>(A, hi, lo, x, y, row_map, status, st);
-    return h <= 4 ? launch_sorted<DT, 4, 4>(A, hi, lo, x, y, row_map, status, st)  // heights up to 8
-                  : launch_sorted<DT, 4, 8>(A, hi, lo, x, y, row_map, status, st);
+    return h <= 4 ? launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st)  // heights up to 8
+                  : launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st);
   } else if (variant == CMRS_VARIANT_STRIP) {
     static Occ occ;
     const size_t smem = (size_t)kStripWarps * A->height * 32 * sizeof(Acc);

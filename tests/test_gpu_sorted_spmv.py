@@ -1,7 +1,10 @@
 """SpMV on column-sorted strips at the sizes where its paths change: whole
-strips per warp (heights that divide 32 and heights that do not), one, two and
-four lanes per row, units longer than the stage, rows longer than the list,
-empty rows, arrays no bulk copy can read."""
+strips per warp (heights that divide 32 and heights that do not), one and two
+lanes per row, units longer than the stage, rows longer than the list, empty
+rows, arrays no bulk copy can read; matrices large enough for the mapping and
+small ones, which keep Algorithm 1."""
+import functools
+
 import numpy as np
 import pytest
 import torch
@@ -21,7 +24,11 @@ def b():
 
 
 def lengths(kind):
+    """About 1,000 rows of a kind, or (large_*) 45,000 to 230,000 of them: past the fewest units of the mapping."""
     rng = np.random.default_rng(12)
+    if kind.startswith("large_"):
+        L = lengths(kind[6:])
+        return np.tile(L, {"short": 45, "skewed": 45, "regular": 230, "two": 120}[kind[6:]])
     if kind == "short":
         return rng.integers(0, 9, 1003)
     if kind == "regular":  # mean 27: one lane per row
@@ -38,11 +45,27 @@ def lengths(kind):
     return L
 
 
-@pytest.mark.parametrize("kind", ["short", "regular", "two", "four", "long", "skewed"])
+@functools.lru_cache(maxsize=None)
+def matrix(kind):
+    L = lengths(kind)
+    if not kind.startswith("large_"):
+        return inputs.from_lengths(L, 7000, seed=3)
+    # one column drawn in each of a row's equal strata: distinct and increasing
+    row = np.repeat(np.arange(L.size), L)
+    j = np.arange(row.size) - np.repeat(np.cumsum(L) - L, L)
+    rng = np.random.default_rng(5)
+    lo, hi = j * 7000 // L[row], (j + 1) * 7000 // L[row]
+    col = (lo + rng.random(row.size) * (hi - lo)).astype(np.int32)
+    rp = np.concatenate([[0], np.cumsum(L)]).astype(np.int32)
+    return inputs.CSR(L.size, 7000, rp, col, rng.uniform(-1, 1, row.size), kind)
+
+
+@pytest.mark.parametrize("kind", ["short", "regular", "two", "four", "long", "skewed", "large_short", "large_skewed",
+                                  "large_regular", "large_two"])
 @pytest.mark.parametrize("h", [1, 2, 3, 4, 6, 8, 12, 16, 17, 32])
 @pytest.mark.parametrize("dtype", [0, 1, 2, 3])
 def test_sorted_spmv(b, kind, h, dtype):
-    a = inputs.from_lengths(lengths(kind), 7000, seed=3)
+    a = matrix(kind)
     rp, ci = torch.from_numpy(a.row_ptr).cuda(), torch.from_numpy(a.col_ind).cuda()
     M = b.cmrs_from_csr(rp, ci, torch.from_numpy(a.val).cuda(), a.cols, h, flags=b.CMRS_SORTED, dtype=dtype)
     x = inputs.uniform_vector(a.cols, 5)
