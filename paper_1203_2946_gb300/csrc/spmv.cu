@@ -30,15 +30,16 @@ constexpr int kRowCap = 32 * CMRS_ROW_ROWS;   // ROW: entries per shared-memory 
 // per SM asked of the register allocator, and the CTAs per SM the launch
 // keeps (its shared-memory carveout holds that many and no more, the rest of
 // the SM's L1/shared storage stays L1).  The x gathers miss L1 and each miss
-// in flight holds an L1 line: with two stages of 15 entries a thread at 5
-// CTAs, the FP32 tiles left 92 KB of L1 and FP64 (4 CTAs) 60 KB, and a
-// further 8 KB of shared memory per CTA, leaving 28 KB, took the power-law
-// FP32 product from 143 to 222 us.  FP32: 11 entries at 6 CTAs (80
-// registers); FP64: 9 at 5 CTAs (96 registers); both keep 92 KB of L1.
+// in flight holds an L1 line, so a CTA stages one tile, whose words and values
+// the threads move to registers before the next tile's copy starts.  FP32: 13
+// entries at 6 CTAs (80 registers), FP64: 9 at 5 CTAs (96 registers).
+// Power-law 4.2M rows, FP32 / FP64 / BF16: 131 / 168 / 130 us against 141 / 167
+// / 139 with two stages (FP32 then 11 entries); FP32 with 9, 11, 15 entries at
+// 7, 6, 5 CTAs: 141, 139, 132 us.
 // Matrices whose rows average CMRS_MERGE_LONG_MU entries or more pay for
 // MERGE's per-tile joins more than for L1 misses: they take the _LONG tiles,
-// 15 entries a thread at as many CTAs as fit (dense 10^4 x 10^4 as sparse:
-// FP64 425 us against 486 us with the short tiles, FP32 257 against 287).
+// 15 entries a thread at as many CTAs as fit (27-point 100^3, FP32 / FP64: 77 /
+// 123 us; two stages: 84 / 128).
 #ifndef CMRS_MERGE_LONG_MU
 #define CMRS_MERGE_LONG_MU 16
 #endif
@@ -64,7 +65,7 @@ constexpr int kRowCap = 32 * CMRS_ROW_ROWS;   // ROW: entries per shared-memory 
 #define CMRS_MERGE_E_F64 9
 #endif
 #ifndef CMRS_MERGE_E_F32
-#define CMRS_MERGE_E_F32 11
+#define CMRS_MERGE_E_F32 13
 #endif
 #ifndef CMRS_MERGE_MINB_F64
 #define CMRS_MERGE_MINB_F64 5
@@ -76,11 +77,6 @@ constexpr int kRowCap = 32 * CMRS_ROW_ROWS;   // ROW: entries per shared-memory 
 #define CMRS_MERGE_THREADS 128  // threads per MERGE tile (a CTA)
 #endif
 constexpr int kMergeThreads = CMRS_MERGE_THREADS;
-#ifndef CMRS_MERGE_VSMEM
-#define CMRS_MERGE_VSMEM 0
-#endif
-// MERGE: values read from the staged tile at their multiply-add instead of held in registers
-constexpr bool kMergeVSmem = CMRS_MERGE_VSMEM != 0;
 #ifndef CMRS_MERGE_CTAS_F64
 #define CMRS_MERGE_CTAS_F64 5
 #endif
@@ -112,8 +108,6 @@ constexpr bool merge_long_differs() {
 }
 constexpr int kMergeWarps = kMergeThreads / 32;
 constexpr int kStripWarps = 8;
-constexpr int kStages = 2;
-
 enum : uint8_t { F_HEAD = 1, F_TAIL = 2, F_THROUGH = 4 };
 
 // Rows crossing a MERGE tile boundary: each tile leaves the partial sum of the
@@ -943,7 +937,7 @@ __global__ void __launch_bounds__(kPadWarps * 32, CMRS_PAD_MINB) k_spmv_padded(i
 
 // ============================================================== MERGE mapping
 // Tile t = entries [T t, T t + T), T = 128 E, staged by bulk copies; thread i
-// owns the E consecutive entries from T t + E i (E = 9 for FP64, 11 for the
+// owns the E consecutive entries from T t + E i (E = 9 for FP64, 13 for the
 // other forms, 15 for both where rows average 16 entries or more).  It finds their strip by
 // a binary search of StripPtr between the strips holding the tile's first
 // and next tile's first entry (tile_strip[], one small pre-pass), then walks
@@ -978,52 +972,80 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
   typedef typename Form<DT>::Acc A;
   constexpr int kMergeE = MergeCfg<DT, kLong>::E, kMergeTile = MergeCfg<DT, kLong>::Tile;
   extern __shared__ __align__(128) char smem[];
-  __shared__ uint64_t bars[kStages];
-  __shared__ StageInfo info[kStages];
+  __shared__ uint64_t bar;
+  __shared__ StageInfo info;
   __shared__ A s_wv[kMergeWarps];         // per warp: scan value of its last lane
   __shared__ int s_wf[kMergeWarps];       // per warp: a segment starts in it
   __shared__ unsigned s_wt[kMergeWarps];  // per warp: lanes whose single run passes through
   __shared__ int s_head0, s_abort;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint32_t mask = (1u << bits) - 1;
-  const size_t stage_bytes = Stage<DT>::bytes(kMergeTile);
   if (tid == 0) {
-    for (int i = 0; i < kStages; ++i) mbar_init(&bars[i], 1);
+    mbar_init(&bar, 1);
     fence_barrier_init();
     s_abort = 0;
   }
   __syncthreads();
   uint64_t pol = 0;
   if (tid == 0) pol = policy_evict_first();
-  auto issue = [&](int t, int st) {
+  const uint32_t *cp = reinterpret_cast<const uint32_t *>(smem);
+  const S *vh = reinterpret_cast<const S *>(smem + Stage<DT>::colp_bytes(kMergeTile));
+  const S *vl = reinterpret_cast<const S *>(smem + Stage<DT>::colp_bytes(kMergeTile) + Stage<DT>::val_bytes(kMergeTile));
+  auto issue = [&](int t) {
     const long long ta = (long long)t * kMergeTile;
     const long long tb = min(ta + kMergeTile, (long long)nnz);
-    issue_stage<DT>(ta, tb, nnz, packed, hi, lo, smem + st * stage_bytes, kMergeTile, &bars[st], pol, &info[st]);
+    issue_stage<DT>(ta, tb, nnz, packed, hi, lo, smem, kMergeTile, &bar, pol, &info);
   };
   int t = blockIdx.x;
-  if (tid == 0 && t < ntiles) issue(t, 0);  // the matrix streams are inputs: no wait needed
-  pdl_wait();                                // tile_strip is k_tile_map's output
-  pdl_launch_dependents();                   // the fix-up kernel may launch and wait in turn
-  for (int it = 0; t < ntiles; ++it, t += gridDim.x) {
-    const int st = it & 1;
-    if (tid == 0) {
-      if (t + (int)gridDim.x < ntiles) issue(t + gridDim.x, st ^ 1);
-      recs[t].tail_flag = 0;
-    }
-    const bool ok = mbar_wait_bounded(&bars[st], (it >> 1) & 1);
+  if (tid == 0 && t < ntiles) issue(t);  // the matrix streams are inputs: no wait needed
+  pdl_wait();                            // tile_strip is k_tile_map's output
+  pdl_launch_dependents();               // the fix-up kernel may launch and wait in turn
+  int it = 0;
+  for (; t < ntiles; ++it, t += gridDim.x) {
+    if (tid == 0) recs[t].tail_flag = 0;
+    const bool ok = mbar_wait_bounded(&bar, it & 1);
     if (!ok) {
       s_abort = 1;
       atomicOr(status, ST_TIMEOUT);
     }
-    const char *stg = smem + st * stage_bytes;
-    const uint32_t *cp = reinterpret_cast<const uint32_t *>(stg);
-    const S *vh = reinterpret_cast<const S *>(stg + Stage<DT>::colp_bytes(kMergeTile));
-    const S *vl = reinterpret_cast<const S *>(stg + Stage<DT>::colp_bytes(kMergeTile) + Stage<DT>::val_bytes(kMergeTile));
-    const long long base = info[st].a8;
+    const long long base = info.a8;
     const long long ta = (long long)t * kMergeTile;
     const long long tb = min(ta + kMergeTile, (long long)nnz);
     const long long k0 = ta + (long long)tid * kMergeE;
     const long long k1 = min(k0 + kMergeE, tb);
+    const int n = (int)(k1 - k0);  // entries of this thread, if any: 1 .. kMergeE
+    const bool has = ok && k0 < tb;
+    // Operands first: the thread's words and values move to registers and its
+    // x gathers start, then the stage is free for the next tile's copy, which
+    // runs while this tile's gathers return and its sums are formed.  One
+    // stage instead of two leaves the other half of its shared memory to L1,
+    // which holds a line per gather in flight.
+    uint32_t c[kMergeE], rw[kMergeE];
+    A xv[kMergeE], v[kMergeE];
+    uint32_t cprev = 0, cnext = 0;  // the entries before and after the thread's own
+    // The walks over the thread's entries are compiled twice: for a thread
+    // holding all kMergeE entries (every thread but the matrix's last one
+    // with entries) the per-entry guards j < n vanish.
+    auto operands = [&](auto full) {
+#pragma unroll
+      for (int j = 0; j < kMergeE; ++j) {
+        if (decltype(full)::value || j < n) {
+          const long long i = k0 + j - base;
+          c[j] = cp[i];
+          v[j] = Form<DT>::value(vh, vl, i);
+          xv[j] = ld_x(x + (c[j] >> bits));
+        }
+      }
+    };
+    if (has) {
+      if (n == kMergeE) operands(std::true_type{});
+      else operands(std::false_type{});
+      if (k0 > 0) cprev = k0 > ta ? cp[k0 - 1 - base] : __ldg(packed + k0 - 1);
+      if (k1 < nnz) cnext = k1 < tb ? cp[k1 - base] : __ldg(packed + k1);
+    }
+    __syncthreads();  // every thread is done with the stage, and with the last tile's scan values
+    if (s_abort) break;
+    if (tid == 0 && t + (int)gridDim.x < ntiles) issue(t + gridDim.x);
     auto put = [&](uint32_t row, A val) {
       if (row < (uint32_t)rows) y[row] = val;
     };
@@ -1031,8 +1053,8 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
     A hv = A(0), tv = A(0);      // head partial (row continued from before), tail partial (row going on)
     uint32_t hrow = 0, trow = 0;
     // lanes with entries in this tile (every lane of the warp votes)
-    const unsigned part = __ballot_sync(0xffffffffu, ok && k0 < tb);
-    if (ok && k0 < tb) {
+    const unsigned part = __ballot_sync(0xffffffffu, has);
+    if (has) {
       // strip holding k0: the largest s in [s_lo, s_hi] with StripPtr[s] <= k0
       int slo = tile_strip[t];
       int shi = (t + 1 < ntiles) ? tile_strip[t + 1] : strips - 1;
@@ -1044,31 +1066,11 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
       int cur = slo;
       long long next = sp[cur + 1];
       // does the entry before k0 (previous thread, or previous tile for thread 0) lie in the same row?
-      bool cont_in = false;
-      if (k0 > sp[cur]) {
-        const uint32_t cprev = k0 > ta ? cp[k0 - 1 - base] : __ldg(packed + k0 - 1);
-        cont_in = (cprev & mask) == (cp[k0 - base] & mask);
-      }
-      const int n = (int)(k1 - k0);  // 1 .. kMergeE
-      // The walk over the thread's entries is compiled twice: for a thread
-      // holding all kMergeE entries (every thread but the matrix's last one
-      // with entries) the per-entry guards j < n vanish.
-      uint32_t c[kMergeE], rw[kMergeE];
-      A xv[kMergeE], v[kMergeE];
-      // operands first, so that the x loads of the run are in flight together;
-      // then the row of every entry: integer work only.  When all of the
-      // thread's entries lie in the strip holding k0 (the usual case) no
-      // StripPtr walk is needed; otherwise the walk may diverge.
-      auto operands_and_rows = [&](auto full) {
-#pragma unroll
-        for (int j = 0; j < kMergeE; ++j) {
-          if (decltype(full)::value || j < n) {
-            const long long i = k0 + j - base;
-            c[j] = cp[i];
-            if (!kMergeVSmem) v[j] = Form<DT>::value(vh, vl, i);
-            xv[j] = ld_x(x + (c[j] >> bits));
-          }
-        }
+      const bool cont_in = k0 > sp[cur] && (cprev & mask) == (c[0] & mask);
+      // the row of every entry: integer work only.  When all of the thread's
+      // entries lie in the strip holding k0 (the usual case) no StripPtr walk
+      // is needed; otherwise the walk may diverge.
+      auto entry_rows = [&](auto full) {
         if (k1 <= next) {
           const uint32_t r0 = (uint32_t)cur * (uint32_t)height;
 #pragma unroll
@@ -1084,8 +1086,8 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
           }
         }
       };
-      if (n == kMergeE) operands_and_rows(std::true_type{});
-      else operands_and_rows(std::false_type{});
+      if (n == kMergeE) entry_rows(std::true_type{});
+      else entry_rows(std::false_type{});
       // rows before the first entry of the matrix are empty
       if (k0 == 0)
         for (uint32_t g = 0; g < rw[0] && g < (uint32_t)rows; ++g) put(g, A(0));
@@ -1094,8 +1096,7 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
       // the warp reconverged first, so that every FMA issues for the whole
       // warp (FP64 issue is charged per warp instruction).
       __syncwarp(part);
-      auto val_of = [&](int j) -> A { return kMergeVSmem ? Form<DT>::value(vh, vl, k0 + j - base) : v[j]; };
-      A acc = fma_acc(val_of(0), xv[0], A(0));
+      A acc = fma_acc(v[0], xv[0], A(0));
       A head_sum = A(0);
       bool first = true;  // the current run is this thread's first
       uint32_t run_row = rw[0];
@@ -1109,7 +1110,7 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
             if (nw && !to_head) put(rw[j - 1], acc);
             first = first && !nw;
             acc = nw ? A(0) : acc;
-            acc = fma_acc(val_of(j), xv[j], acc);
+            acc = fma_acc(v[j], xv[j], acc);
             run_row = rw[j];
           }
         }
@@ -1131,10 +1132,9 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
       // the entry after this thread's last one: same row?
       long long next_row = rows;
       if (k1 < nnz) {
-        const uint32_t cn = (k1 < tb) ? cp[k1 - base] : __ldg(packed + k1);
         int s2 = cur;
         while (k1 >= sp[s2 + 1]) ++s2;
-        next_row = (long long)s2 * height + (cn & mask);
+        next_row = (long long)s2 * height + (cnext & mask);
       }
       const bool cont_out = next_row == (long long)run_row;
       if (first && cont_in) {
@@ -1170,7 +1170,7 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
     // per warp instead of a 127-step serial walk.
     const bool through = (flags & F_THROUGH) != 0;
     const bool start = !through || tid == 0;
-    A v = through ? hv : ((flags & F_TAIL) ? tv : A(0));
+    A sv = through ? hv : ((flags & F_TAIL) ? tv : A(0));
     bool f = start;
     unsigned z = ~__ballot_sync(0xffffffffu, start);
     int nsteps = 0;  // ceil(log2(longest run of non-start lanes + 1))
@@ -1179,30 +1179,30 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
       z &= z >> sh;
     }
     for (int st2 = 0, d = 1; st2 < nsteps; ++st2, d <<= 1) {
-      const A vo = __shfl_up_sync(0xffffffffu, v, d);
+      const A vo = __shfl_up_sync(0xffffffffu, sv, d);
       const int fo = __shfl_up_sync(0xffffffffu, (int)f, d);
       if (lane >= d) {
-        if (!f) v = vo + v;
+        if (!f) sv = vo + sv;
         f = f || fo;
       }
     }
     const unsigned tmask = __ballot_sync(0xffffffffu, through);
     const bool end = (flags & F_HEAD) && !through;
     if (lane == 31) {
-      s_wv[wid] = v;
+      s_wv[wid] = sv;
       s_wf[wid] = f;
     }
     if (lane == 0) s_wt[wid] = tmask;
     if (tid == 0) s_head0 = (flags & F_HEAD) != 0;
     __syncthreads();
-    if (!s_abort) {
+    {
       // the segment open at this warp's start, summed over the warps before it
       A carry = A(0);
       if (wid > 0 && __any_sync(0xffffffffu, !f || (end && lane == 0))) {
         for (int u = 0; u < wid; ++u) carry = s_wf[u] ? s_wv[u] : carry + s_wv[u];
-        if (!f) v = carry + v;
+        if (!f) sv = carry + sv;
       }
-      A in = __shfl_up_sync(0xffffffffu, v, 1);
+      A in = __shfl_up_sync(0xffffffffu, sv, 1);
       if (lane == 0) in = carry;
       int estar = kMergeThreads;  // first thread whose run does not pass through
       for (int u = 0; u < kMergeWarps; ++u)
@@ -1225,12 +1225,12 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
         if (head0 && estar == kMergeThreads) {
           // one row runs through the whole tile
           recs[t].head_row = (int)hrow;
-          recs[t].head_sum = (double)v;
+          recs[t].head_sum = (double)sv;
           recs[t].head_flag = 2;
           recs[t].tail_flag = 0;
         } else if (through || (flags & F_TAIL)) {
           recs[t].tail_row = (int)(through ? hrow : trow);
-          recs[t].tail_sum = (double)v;
+          recs[t].tail_sum = (double)sv;
           recs[t].tail_flag = 1;
         } else {
           recs[t].tail_flag = 0;
@@ -1238,9 +1238,8 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
       }
       if (tid == 0 && !head0) recs[t].head_flag = 0;
     }
-    __syncthreads();
-    if (s_abort) break;
   }
+  if (s_abort) mbar_wait_bounded(&bar, it & 1);  // a late copy lands before the block leaves
 }
 
 template <typename A>
@@ -1578,10 +1577,12 @@ int occupancy(K kernel, int threads, size_t smem, Occ &cache, size_t smem_cap = 
   return cache.val[dev];
 }
 
-// sized for the smaller of the form's two tiles: enough for either launch
+// sized for tiles of 1,152 (FP64) and 1,408 entries, the least either launch
+// takes (cmrs.h states cmrs_spmv_noalloc's limits in these)
 size_t merge_ws_bytes(int nnz, int dtype) {
-  const int tile = dtype == CMRS_F64 ? std::min(MergeCfg<CMRS_F64, false>::Tile, MergeCfg<CMRS_F64, true>::Tile)
-                                     : std::min(MergeCfg<CMRS_F32, false>::Tile, MergeCfg<CMRS_F32, true>::Tile);
+  const int tile = dtype == CMRS_F64 ? 1152 : 1408;
+  static_assert(MergeCfg<CMRS_F64, false>::Tile >= 1152 && MergeCfg<CMRS_F64, true>::Tile >= 1152 &&
+                MergeCfg<CMRS_F32, false>::Tile >= 1408 && MergeCfg<CMRS_F32, true>::Tile >= 1408, "MERGE workspace");
   const long long ntiles = ceil_div(nnz, tile);
   return 256 + align256((size_t)(ntiles + 1) * 4) + align256((size_t)ntiles * sizeof(TileRec));
 }
@@ -1666,7 +1667,7 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
   TileRec *recs = reinterpret_cast<TileRec *>(ws + 256 + align256((size_t)(ntiles + 1) * 4));
   k_tile_map<<<(int)ceil_div(A->strips, 256), 256, 0, st>>>(A->strips, A->strip_ptr, kMergeTile, ntiles, tile_strip);
   CMRS_LAUNCH_CHECK();
-  const size_t smem = kStages * Stage<DT>::bytes(kMergeTile);
+  const size_t smem = Stage<DT>::bytes(kMergeTile);
   const int per_sm = occupancy(k_spmv_merge<DT, kLong>, kMergeThreads, smem, occ, 0, MergeCfg<DT, kLong>::Ctas);
   const int grid = (int)std::min<long long>(ntiles, (long long)per_sm * sm_count());
   int rc = launch_pdl(k_spmv_merge<DT, kLong>, (unsigned)grid, kMergeThreads, smem, st, A->rows, A->height, A->bits,
