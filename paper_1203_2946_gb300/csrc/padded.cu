@@ -451,9 +451,8 @@ extern "C" int cmrs_pad_layout(const cmrs_matrix *A, int slots, int32_t *strip_p
   CMRS_LAUNCH_CHECK();
   rc = scan_counts(S, ws + 256, 32, strip_ptr_padded, status, st);
   if (rc) return rc;
-  uint32_t host[2] = {0, 0};
-  CMRS_CUDA_TRY(cudaMemcpyAsync(&host[0], status, 4, cudaMemcpyDeviceToHost, st));
-  CMRS_CUDA_TRY(cudaMemcpyAsync(&host[1], strip_ptr_padded + S, 4, cudaMemcpyDeviceToHost, st));
+  uint32_t host[2] = {0, 0};  // status, padded item count
+  CMRS_CUDA_TRY(cudaMemcpyAsync(host, status, 8, cudaMemcpyDeviceToHost, st));
   CMRS_CUDA_TRY(cudaStreamSynchronize(st));
   if (host[0] & ST_PAD_PLAN) return CMRS_ERR_CSR_INVALID;
   if (host[0] & ST_SCAN_OVERFLOW) return CMRS_ERR_ARG;

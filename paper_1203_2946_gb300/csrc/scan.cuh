@@ -91,6 +91,7 @@ __global__ void k_scan_finish(int n, const long long *__restrict__ incl, const l
   } else {
     out[i + 1] = (int32_t)v;
   }
+  if (i == n - 1) status[1] = (uint32_t)out[n];  // the total, beside the status: one read-back for both
 }
 
 // Workspace bytes for the scan of n counts: counts int32[n], incl int64[n], aux int64[blocks].
@@ -99,7 +100,8 @@ inline size_t scan_ws_bytes(int n) {
   return align256(m * 4) + align256(m * 8) + align256((size_t)ceil_div((long long)m, kScanThreads) * 8);
 }
 
-// Enqueues the scan of counts (already written at `ws`) into out[n + 1].
+// Enqueues the scan of counts (already written at `ws`) into out[n + 1], its
+// total also into status[1].
 inline int scan_counts(int n, char *ws, int mult, int32_t *out, uint32_t *status, cudaStream_t st) {
   const size_t m = (size_t)(n > 0 ? n : 1);
   int32_t *counts = reinterpret_cast<int32_t *>(ws);
