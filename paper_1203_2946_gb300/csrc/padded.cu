@@ -191,8 +191,49 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
       *po = cp[src];
       *ho = vh[src];
       if (kSplit) *lo = vl[src];
-    } else {
+      continue;
+    }
+    const unsigned some = __ballot_sync(kFull, left > 0);
+    const int same = __popc(some) > K ? 0 : min(D, (int)__reduce_min_sync(kFull, left > 0 ? (unsigned)left / kM : ~0u >> 1));
+    __syncwarp();
+    if (same > 1) {
+      // 32 / M rows or fewer have items left, so each takes min(left, M) of them
+      // every pass; until one holds fewer than M the passes are alike: M items
+      // of each, the same zero items.  The pass's layout once -- each position's
+      // row, and where its items lie -- then `same` passes of copies.  (A strip
+      // with one row of 2,000 items, M = 8: 250 passes of 2 us each before.)
+      const int take = left > 0 ? kM : 0;
+      const int zcap = lane < height ? kM - take : 0;
+      const int zero = max(0, min(zcap, 32 - kM * __popc(some) - warp_excl_scan(zcap, lane)));
+      const int len = take + zero, off = warp_excl_scan(len, lane);
+      const unsigned rows = __ballot_sync(kFull, len > 0);
+      const unsigned starts = __reduce_or_sync(kFull, len > 0 ? 1u << off : 0u);
+      if (len > 0) {
+        const int k = __popc(rows & lt);
+        map[k] = (uint32_t)next;
+        map[32 + k] = (uint32_t)(off | take << 8 | lane << 16);
+      }
       __syncwarp();
+      const int k = __popc(starts << (31 - lane)) - 1;  // the run of this position
+      const uint32_t in = map[32 + k];
+      const int at = lane - (int)(in & 255);
+      const bool real = at < (int)((in >> 8) & 255);
+      const int src = (int)map[k] + at;
+      const uint32_t filler = in >> 16;  // a zero item: column 0, this row
+      __syncwarp();
+#pragma unroll 4
+      for (int p = 0; p < same; ++p) {
+        po[32 * (long long)p] = real ? cp[src + kM * p] : filler;
+        ho[32 * (long long)p] = real ? vh[src + kM * p] : S(0);
+        if (kSplit) lo[32 * (long long)p] = real ? vl[src + kM * p] : S(0);
+      }
+      next += take * same;
+      left -= take * same;
+      D -= same - 1;
+      po += 32 * (long long)(same - 1);
+      ho += 32 * (long long)(same - 1);
+      lo += kSplit ? 32 * (long long)(same - 1) : 0;
+    } else {
       if (!pad_pass<S, kSplit, kM>(left, next, D + 1, height, cp, vh, vl, po - lane, ho - lane,
                                    kSplit ? lo - lane : nullptr))
         return;
