@@ -91,6 +91,13 @@ extern "C" {
  *                       stride through the strip and accumulate per-row
  *                       partial sums in a shared-memory buffer buf[row][lane],
  *                       then a lane reduction.  Works on sorted strips.
+ *                       Sorted strips of short rows, in matrices of enough
+ *                       of them, are summed by the row instead: a warp stages
+ *                       the strips of 32 or 16 rows, finds each row's entries
+ *                       among them with integer work, and one or two lanes
+ *                       per row sum them in column order in registers (needs
+ *                       col_packed and val 16-byte aligned; Algorithm 1 runs
+ *                       otherwise).
  *   CMRS_VARIANT_MERGE  equal-work tiles of nonzeros: each thread owns a run
  *                       of consecutive entries, rows that cross thread or
  *                       tile boundaries are joined afterwards in a fixed

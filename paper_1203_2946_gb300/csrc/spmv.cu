@@ -1,4 +1,5 @@
-// y = A x on the CMRS format (Section 4, Algorithm 1), three thread mappings.
+// y = A x on the CMRS format (Section 4, Algorithm 1): the ROW, STRIP, MERGE
+// and PADDED thread mappings.
 //
 // GB300 design notes.  FP64 issue rate on this part is about 1/58 of FP32
 // (measured 1.2 TFLOP/s), so at HBM speed an FP64 SpMV can afford about one
@@ -6,9 +7,10 @@
 // each row's sum in one thread's register (one FMA per nonzero, no per-lane
 // buffer, no lane reduction); the STRIP mapping is Algorithm 1 as the paper
 // states it (per-lane row buffers + reduction) and costs 31*height extra adds
-// per strip.  Nonzero streams are copied into shared memory by the bulk-copy
-// engine (cp.async.bulk, mbarrier completion, L2 evict-first) two stages
-// ahead of the threads that use them.
+// per strip, so column-sorted strips of short rows have the sort undone in
+// shared memory and are summed by the row instead (the SORTED mapping).
+// Nonzero streams are copied into shared memory by the bulk-copy engine
+// (cp.async.bulk, mbarrier completion, L2 evict-first).
 #include <algorithm>
 #include <mutex>
 

@@ -60,16 +60,19 @@ def test_row_of_each_entry(b, h, lengths):
     assert M.struct.max_strip_nnz == np.diff(ref["strip_ptr"]).max()
 
 
-def csr(lengths, cols, seed, ordered=True, repeats=False):
-    """Rows of the given lengths; columns increasing, or shuffled inside each row, or drawn with repeats."""
+def csr(lengths, cols, seed, order="ordered"):
+    """Rows of the given lengths; columns increasing, or shuffled inside each row, or drawn with repeats (equal columns
+    in one row), shuffled or ordered."""
     a = inputs.from_lengths(lengths, cols, seed=seed)
-    if ordered:
+    if order == "ordered":
         return a
     rng = np.random.default_rng(seed)
     ci = a.col_ind.copy()
     for r in range(a.rows):
         p, q = a.row_ptr[r], a.row_ptr[r + 1]
-        ci[p:q] = rng.integers(0, min(50, cols), q - p) if repeats else rng.permutation(ci[p:q])
+        ci[p:q] = rng.permutation(ci[p:q]) if order == "shuffled" else rng.integers(0, min(50, cols), q - p)
+        if order == "ordered_repeats":
+            ci[p:q].sort()
     return inputs.CSR(a.rows, a.cols, a.row_ptr, ci, a.val, a.name)
 
 
@@ -86,10 +89,10 @@ SORT_CASES = {
 
 @pytest.mark.parametrize("h", [1, 2, 3, 6, 8, 16, 32])
 @pytest.mark.parametrize("case", sorted(SORT_CASES))
-@pytest.mark.parametrize("order", ["ordered", "shuffled", "repeats"])
+@pytest.mark.parametrize("order", ["ordered", "shuffled", "repeats", "ordered_repeats"])
 def test_sorted_strips(b, case, h, order):
     make, cols = SORT_CASES[case]
-    a = csr(make(np.random.default_rng(3)), cols, 5, order == "ordered", order == "repeats")
+    a = csr(make(np.random.default_rng(3)), cols, 5, order)
     rp, ci = dev(a)
     M = b.cmrs_from_csr(rp, ci, torch.from_numpy(a.val).cuda(), a.cols, h, flags=b.CMRS_SORTED)
     ref = orc.csr_to_cmrs(a.row_ptr, a.col_ind, a.val, a.cols, h, sorted_=True)
