@@ -66,6 +66,15 @@ __device__ __forceinline__ int row_span(int sa, int sb, int height, uint32_t mas
   return lane < height ? end - start : 0;
 }
 
+// Sum of v (0..kM) over the lanes below this one.  For M = 2 by two votes,
+// which do not wait for each other as a shuffle scan's five steps do.
+template <int kM>
+__device__ __forceinline__ int small_scan(int v, int lane) {
+  if (kM > 2) return warp_excl_scan(v, lane);
+  const unsigned lt = (1u << lane) - 1;
+  return __popc(__ballot_sync(kFull, v & 1) & lt) + 2 * __popc(__ballot_sync(kFull, v & 2) & lt);
+}
+
 // One pass of the plan in its general form, for the passes k_pad_fill's short
 // form does not cover: `left` items per row, C passes left (this one
 // included).  Writes the pass at out (32 items) and takes it off left and
@@ -97,7 +106,7 @@ __device__ __forceinline__ bool pad_pass(int &left, int &next, int C, int height
       const int v = (int)__reduce_max_sync(kFull, (rem >> lane) & 1u ? (unsigned)lv : 0u);
       const unsigned g = __ballot_sync(kFull, ((rem >> lane) & 1u) && lv == v);
       const int wg = (g >> lane) & 1u ? want : 0;
-      const int below = warp_excl_scan(wg, lane);  // want of the group's lower rows
+      const int below = small_scan<kM>(wg, lane);  // want of the group's lower rows
       if ((g >> lane) & 1u) before = done + below;
       done += (int)__reduce_add_sync(kFull, (unsigned)wg);
       rem &= ~g;
@@ -108,9 +117,9 @@ __device__ __forceinline__ bool pad_pass(int &left, int &next, int C, int height
   room -= (int)__reduce_add_sync(kFull, (unsigned)extra);
   // zero items: rows 0 upwards, each topped up to M
   const int zcap = lane < height ? kM - take : 0;
-  const int zero = max(0, min(zcap, room - warp_excl_scan(zcap, lane)));
+  const int zero = max(0, min(zcap, room - small_scan<kM>(zcap, lane)));
   const int len = take + zero;
-  const int off = warp_excl_scan(len, lane);
+  const int off = small_scan<kM>(len, lane);
 #pragma unroll
   for (int j = 0; j < kM; ++j) {
     if (j < take) {
@@ -128,6 +137,14 @@ __device__ __forceinline__ bool pad_pass(int &left, int &next, int C, int height
   return true;
 }
 
+// An item read from the stage, or from global memory by a load that may pass
+// the stores before it (the compiler cannot tell that they do not alias).
+template <bool kStaged, typename T>
+__device__ __forceinline__ T item(const T *p) {
+  if constexpr (kStaged) return *p;
+  return __ldg(p);
+}
+
 // Runs the plan of one strip and writes its `limit` passes from out0 on.  The
 // strip's items are cp[next..], lane r's row starting at `next` with `left`
 // items; map: this warp's 2 x 32 words of shared memory.
@@ -141,14 +158,17 @@ __device__ __forceinline__ bool pad_pass(int &left, int &next, int C, int height
 // it goes in full whenever t lies below that, or no row is forced at all.  t
 // only falls from pass to pass, so it is found by stepping down from the last
 // pass's, a vote a step.  Lane j then reads item j % M of the (j / M)-th
-// chosen row, whose next item is passed through `map`, and the pass leaves by
-// one 32-word store per array.  On rows of 4..60 items (height 32, M = 2)
-// 94% of the passes take this form; 98 instructions a pass on average against
-// 430 when every pass ran the general form, and with the staged reads
-// k_pad_fill takes 316 us instead of 1,149 on 2,097,152 such rows (67M FP32
-// entries; reading and writing them once is 163 us).  What is left is bound
-// by the votes' latency at 20 warps per SM (the stage's shared memory).
-template <typename S, bool kSplit, int kM>
+// chosen row, whose next item is passed through `map`; the pass is read and
+// stored while the next one is planned, so that the votes do not wait for the
+// two reads (M < 8).  On rows of 4..60 items (height 32, M = 2) 94% of the
+// passes take this form.  k_pad_fill on 2,097,152 such rows (67M FP32
+// entries): 1,149 us when every pass ran the general form, 316 us with each
+// pass read as it was planned, 290 us so; reading and writing the items
+// once is 163 us.  What is left is the votes' latency at 20 warps per SM (the
+// stage's shared memory).  Forms with small stages are bound by registers
+// instead: 48 (10 CTAs per SM) against the compiler's 56 leave rows of
+// power-law lengths 10% faster, 40 spill and are 4-17% slower.
+template <typename S, bool kSplit, int kM, bool kStaged>
 __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, long long limit, uint32_t *map,
                                                const uint32_t *__restrict__ cp, const S *__restrict__ vh,
                                                const S *__restrict__ vl, long long out0,
@@ -166,7 +186,16 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
   lo += kSplit ? lane : 0;
   // passes left after this one (below 2^31 / 32).  The last pass never takes
   // the short form: every item left is forced then.
+  int src = 0;        // this position's item in the pass planned last,
+  bool held = false;  // which is copied while the next one is planned
   for (int D = (int)limit - 1; D > 0; --D, po += 32, ho += 32, lo += kSplit ? 32 : 0) {
+    uint32_t c;
+    S h, l;
+    if (held) {
+      c = cp[src];
+      h = vh[src];
+      if (kSplit) l = vl[src];
+    }
     unsigned gt = __ballot_sync(kFull, left > t), ge = __ballot_sync(kFull, left >= t);
     if (__popc(ge) < K) {
       gt = ge;
@@ -186,13 +215,28 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
         next += kM;
         left -= kM;
       }
+      if (held) {
+        po[-32] = c;
+        ho[-32] = h;
+        if (kSplit) lo[-32] = l;
+      }
       __syncwarp();
-      const int src = (int)mp[lane / kM] + (lane & (kM - 1));
-      *po = cp[src];
-      *ho = vh[src];
-      if (kSplit) *lo = vl[src];
+      src = (int)mp[lane / kM] + (lane & (kM - 1));
+      if (kM == 8) {  // four rows a pass: few passes in a row take this form, and holding one cost 5-8%
+        *po = cp[src];
+        *ho = vh[src];
+        if (kSplit) *lo = vl[src];
+        continue;
+      }
+      held = true;
       continue;
     }
+    if (held) {
+      po[-32] = c;
+      ho[-32] = h;
+      if (kSplit) lo[-32] = l;
+    }
+    held = false;
     const unsigned some = __ballot_sync(kFull, left > 0);
     const int same = __popc(some) > K ? 0 : min(D, (int)__reduce_min_sync(kFull, left > 0 ? (unsigned)left / kM : ~0u >> 1));
     __syncwarp();
@@ -204,8 +248,8 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
       // with one row of 2,000 items, M = 8: 250 passes of 2 us each before.)
       const int take = left > 0 ? kM : 0;
       const int zcap = lane < height ? kM - take : 0;
-      const int zero = max(0, min(zcap, 32 - kM * __popc(some) - warp_excl_scan(zcap, lane)));
-      const int len = take + zero, off = warp_excl_scan(len, lane);
+      const int zero = max(0, min(zcap, 32 - kM * __popc(some) - small_scan<kM>(zcap, lane)));
+      const int len = take + zero, off = small_scan<kM>(len, lane);
       const unsigned rows = __ballot_sync(kFull, len > 0);
       const unsigned starts = __reduce_or_sync(kFull, len > 0 ? 1u << off : 0u);
       if (len > 0) {
@@ -221,11 +265,11 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
       const int src = (int)map[k] + at;
       const uint32_t filler = in >> 16;  // a zero item: column 0, this row
       __syncwarp();
-#pragma unroll 4
+#pragma unroll(kStaged && kM < 8 ? 2 : 4)
       for (int p = 0; p < same; ++p) {
-        po[32 * (long long)p] = real ? cp[src + kM * p] : filler;
-        ho[32 * (long long)p] = real ? vh[src + kM * p] : S(0);
-        if (kSplit) lo[32 * (long long)p] = real ? vl[src + kM * p] : S(0);
+        po[32 * (long long)p] = real ? item<kStaged>(cp + src + kM * p) : filler;
+        ho[32 * (long long)p] = real ? item<kStaged>(vh + src + kM * p) : S(0);
+        if (kSplit) lo[32 * (long long)p] = real ? item<kStaged>(vl + src + kM * p) : S(0);
       }
       next += take * same;
       left -= take * same;
@@ -238,6 +282,11 @@ __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, l
                                    kSplit ? lo - lane : nullptr))
         return;
     }
+  }
+  if (held) {
+    po[-32] = cp[src];
+    ho[-32] = vh[src];
+    if (kSplit) lo[-32] = vl[src];
   }
   pad_pass<S, kSplit, kM>(left, next, 1, height, cp, vh, vl, po - lane, ho - lane, kSplit ? lo - lane : nullptr);
 }
@@ -265,37 +314,44 @@ __global__ void __launch_bounds__(kPadWarps * 32) k_pad_count(int strips, int he
   }
 }
 
-// M = 1 (so height 32): every row with items left takes exactly one per pass
-// (the forced takes and the free room together never turn a row away), so
-// pass p holds item p of row r at position r, or a zero item of row r once
-// the row has run out; the strip has max(row length) passes.  No plan to run:
-// each lane copies its own row, kPadFillU passes' loads in flight.
-constexpr int kPadFillU = 8;
-template <typename S, bool kSplit>
-__device__ __forceinline__ void pad_strip_fill_m1(int left, int next, long long limit,
-                                                  const uint32_t *__restrict__ cp, const S *__restrict__ vh,
-                                                  const S *__restrict__ vl, long long out0,
-                                                  uint32_t *__restrict__ pk_out, S *__restrict__ vo_h,
-                                                  S *__restrict__ vo_l) {
-  const int lane = threadIdx.x & 31;
-  for (long long p = 0; p < limit; p += kPadFillU) {
-    uint32_t c[kPadFillU];
-    S h[kPadFillU], l[kPadFillU];
+// height x M = 32 (M = 1: height 32): every row with items left takes
+// min(items left, M) per pass (together at most 32, so the free room never
+// turns one away) and zero items top it up to M, so row r has positions r M ..
+// r M + M - 1 of every pass, and the strip has max(ceil(row length / M))
+// passes.  No plan to run: lane j copies every M-th item of row j / M,
+// U passes' loads in flight.  16.8M FP32 entries in rows of 4..60 at
+// height 16, M = 2: 151 us by the plan, 62 us so; M = 1 (twice the items,
+// most of them zero) 60 us either way.
+template <typename S, bool kSplit, int kM>
+__device__ __forceinline__ void pad_strip_fill_even(int left, int next, long long limit,
+                                                    const uint32_t *__restrict__ cp, const S *__restrict__ vh,
+                                                    const S *__restrict__ vl, long long out0,
+                                                    uint32_t *__restrict__ pk_out, S *__restrict__ vo_h,
+                                                    S *__restrict__ vo_l) {
+  constexpr int U = kM == 1 ? 8 : 4;
+  const int lane = threadIdx.x & 31, row = lane / kM;
+  const int items = __shfl_sync(kFull, left, row) - (lane & (kM - 1));  // of this position's row, from its first here
+  const int first = __shfl_sync(kFull, next, row) + (lane & (kM - 1));
+  const int passes = (int)limit;  // below 2^31 / 32
+  for (int p = 0; p < passes; p += U) {
+    uint32_t c[U];
+    S h[U], l[U];
 #pragma unroll
-    for (int u = 0; u < kPadFillU; ++u) {
-      c[u] = (uint32_t)lane;  // a zero item: column 0, this row
+    for (int u = 0; u < U; ++u) {
+      c[u] = (uint32_t)row;  // a zero item: column 0, this row
       h[u] = S(0);
       l[u] = S(0);
-      if (p + u < left) {
-        c[u] = cp[next + p + u];
-        h[u] = vh[next + p + u];
-        if (kSplit) l[u] = vl[next + p + u];
+      const int k = (p + u) * kM;
+      if (k < items) {
+        c[u] = cp[first + k];
+        h[u] = vh[first + k];
+        if (kSplit) l[u] = vl[first + k];
       }
     }
 #pragma unroll
-    for (int u = 0; u < kPadFillU; ++u)
-      if (p + u < limit) {
-        const long long o = out0 + (p + u) * 32 + lane;
+    for (int u = 0; u < U; ++u)
+      if (p + u < passes) {
+        const long long o = out0 + (p + u) * 32LL + lane;
         pk_out[o] = c[u];
         vo_h[o] = h[u];
         if (kSplit) vo_l[o] = l[u];
@@ -304,7 +360,7 @@ __device__ __forceinline__ void pad_strip_fill_m1(int left, int next, long long 
 }
 
 // Strip [sa, sb) whose item k is at cp[k - base].
-template <typename S, bool kSplit, int kM>
+template <typename S, bool kSplit, int kM, bool kStaged>
 __device__ __forceinline__ void pad_strip(int sa, int sb, int base, int height, int bits, long long limit,
                                           uint32_t *map, const uint32_t *__restrict__ cp, const S *__restrict__ vh,
                                           const S *__restrict__ vl, long long out0, uint32_t *__restrict__ pk_out,
@@ -312,10 +368,18 @@ __device__ __forceinline__ void pad_strip(int sa, int sb, int base, int height, 
   int next;
   int left = row_span(sa - base, sb - base, height, (1u << bits) - 1, cp, threadIdx.x & 31, &next);
   if (left < 0) left = 0;  // a corrupt strip, which the layout pass reports
-  if constexpr (kM == 1)
-    pad_strip_fill_m1<S, kSplit>(left, next, limit, cp, vh, vl, out0, pk_out, vo_h, vo_l);
+  if (kM == 1 || height * kM == 32)
+    pad_strip_fill_even<S, kSplit, kM>(left, next, limit, cp, vh, vl, out0, pk_out, vo_h, vo_l);
   else
-    pad_strip_fill<S, kSplit, kM>(left, next, height, limit, map, cp, vh, vl, out0, pk_out, vo_h, vo_l);
+    pad_strip_fill<S, kSplit, kM, kStaged>(left, next, height, limit, map, cp, vh, vl, out0, pk_out, vo_h, vo_l);
+}
+
+// Asks for the lines of [a, b) in L2, a line per lane and step.
+template <typename T>
+__device__ __forceinline__ void prefetch_l2(const T *a, const T *b) {
+  constexpr int kLine = 128 / sizeof(T);
+  for (const T *p = a + (threadIdx.x & 31) * kLine; p < b; p += 32 * kLine)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // One strip per warp.  The strip's items are copied into the warp's own
@@ -331,8 +395,9 @@ __device__ __forceinline__ void pad_strip(int sa, int sb, int base, int height, 
 #endif
 constexpr int kFillWarps = CMRS_FILL_WARPS;
 constexpr int kFillCap = 2048;  // most items per stage
+constexpr int kFillAhead = 2048;  // most items of a longer strip asked for in L2 (24 KB a warp in FP64; 6,080 warps at most)
 template <int DT, int kM>
-__global__ void __launch_bounds__(kFillWarps * 32) k_pad_fill(int strips, int height, int bits, int cap, int nnz,
+__global__ void __launch_bounds__(kFillWarps * 32, kM == 1 ? 8 : 10) k_pad_fill(int strips, int height, int bits, int cap, int nnz,
                                                              const int32_t *__restrict__ sp,
                                                              const uint32_t *__restrict__ packed,
                                                              const typename Form<DT>::Stored *__restrict__ vh,
@@ -363,6 +428,16 @@ __global__ void __launch_bounds__(kFillWarps * 32) k_pad_fill(int strips, int he
     const int sa = sp[s], sb = sp[s + 1];
     bool staged = stages && sb > sa && sb - sa <= cap;
     if (staged && lane == 0) issue_stage<DT>(sa, sb, nnz, packed, vh, vl, stg, cap, &bars[w], pol, &info[w]);
+    if (!staged) {
+      // read from global memory below, a few passes' loads at a time: from L2,
+      // as much of it as L2 holds for every warp on the chip (power-law rows
+      // of 1M, M = 8 at height 16: 250 -> 129 us with the reads of passes
+      // alike by item<>)
+      const int to = sb - sa > kFillAhead ? sa + kFillAhead : sb;
+      prefetch_l2(packed + sa, packed + to);
+      prefetch_l2(vh + sa, vh + to);
+      if (kSplit) prefetch_l2(vl + sa, vl + to);
+    }
     const long long o0 = sp_out[s], o1 = sp_out[s + 1];
     const long long limit = o1 > o0 ? (o1 - o0) / 32 : 0;
     if (staged) {
@@ -375,11 +450,11 @@ __global__ void __launch_bounds__(kFillWarps * 32) k_pad_fill(int strips, int he
     // compiled twice, so that the staged walk's reads are shared-memory loads
     if (staged) {
       const char *sh = stg + Stage<DT>::colp_bytes(cap);
-      pad_strip<S, kSplit, kM>(sa, sb, (int)info[w].a8, height, bits, limit, maps[w],
+      pad_strip<S, kSplit, kM, true>(sa, sb, (int)info[w].a8, height, bits, limit, maps[w],
                                reinterpret_cast<const uint32_t *>(stg), reinterpret_cast<const S *>(sh),
                                reinterpret_cast<const S *>(sh + Stage<DT>::val_bytes(cap)), o0, pk_out, vo_h, vo_l);
     } else {
-      pad_strip<S, kSplit, kM>(sa, sb, 0, height, bits, limit, maps[w], packed, vh, vl, o0, pk_out, vo_h, vo_l);
+      pad_strip<S, kSplit, kM, false>(sa, sb, 0, height, bits, limit, maps[w], packed, vh, vl, o0, pk_out, vo_h, vo_l);
     }
     __syncwarp();  // every lane is done with the stage before the next copy lands in it
   }
