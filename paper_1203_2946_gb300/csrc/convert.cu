@@ -462,8 +462,17 @@ __device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bit
   return bad;
 }
 
+// Most strips of more than cap entries (cap >= 256) that do not overlap: with
+// two lists of that length, one from either end, nnz words hold both.
+__host__ __device__ __forceinline__ int list_room(int nnz, int cap) { return nnz / (cap + 1); }
+
 // Validation, StripPtr and the longest strip as in k_pack; strips of up to cap
-// entries sorted here, longer ones listed for the two kernels below.
+// entries sorted here, longer ones listed for the two kernels below: CTA strips
+// from the front of the list, radix strips from its end.  A strip is found
+// valid by its own rows alone, so a RowPtr that falls back between strips makes
+// many of them valid over the same entries; each list therefore ends after
+// `room` strips, as many as can be longer than cap without overlapping, and a
+// ticket past it is an invalid RowPtr.
 template <typename In, int DT>
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int cols, int nnz, int height, int strips,
                                                                int bits, int cap, const int32_t *__restrict__ row_ptr,
@@ -477,6 +486,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int col
   extern __shared__ __align__(16) char smem[];
   __shared__ int rs_all[kSortWarps][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int room = list_room(nnz, cap);
   char *buf = smem + (size_t)w * 16 * (cap + 1);
   uint32_t bad = 0;
   int longest = 0;
@@ -495,10 +505,11 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int col
     }
     longest = max(longest, R.len);
     if (R.len > cap) {
-      // CTA strips from the front of the list, radix strips from its end
       if (lane == 0) {
-        if (R.len <= kSortBlockCap) list[atomicAdd(&st->nblock, 1)] = s;
-        else list[nnz - 1 - atomicAdd(&st->nradix, 1)] = s;
+        const bool block = R.len <= kSortBlockCap;
+        const int i = atomicAdd(block ? &st->nblock : &st->nradix, 1);
+        if (i < room) list[block ? i : nnz - 1 - i] = s;
+        else bad |= ST_BAD_ROWPTR;
       }
     } else if (R.len > 0) {
       if (sort_strip<In, DT, 32>(R, cols, bits, cap, col_ind, val_in, buf, rs_all[w], packed, vhi, vlo))
@@ -512,7 +523,9 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int col
   }
 }
 
-// Listed strips of up to kSortBlockCap entries, a CTA each.
+// Listed strips of up to kSortBlockCap entries, a CTA each.  An invalid RowPtr
+// (the status of k_sort_warp is complete here) leaves nothing to do: its lists
+// were cut short and its strips may overlap.
 template <typename In, int DT>
 __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols, int nnz, int height, int bits,
                                                              const int32_t *__restrict__ row_ptr,
@@ -524,6 +537,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols,
                                                              const int32_t *__restrict__ list, StatusBlock *st) {
   extern __shared__ __align__(16) char smem[];
   __shared__ int rs[33];
+  if (st->status & ST_BAD_ROWPTR) return;
   const int n = st->nblock;
   bool bad = false;
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
@@ -539,6 +553,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols,
 // global ping-pong buffers, 8 bits per pass.  Each pass: digit histogram,
 // exclusive scan into bucket bases, then a stable scatter of 128-entry chunks
 // ranked per warp with match_any and across warps by a per-digit prefix.
+// Nothing is done with an invalid RowPtr: strips that overlap would share their
+// part of the buffers.
 template <typename In, int DT>
 __global__ void __launch_bounds__(kRadixThreads) k_sort_radix(int rows, int cols, int nnz, int height, int bits,
                                                               int col_bits, const int32_t *__restrict__ row_ptr,
@@ -556,6 +572,7 @@ __global__ void __launch_bounds__(kRadixThreads) k_sort_radix(int rows, int cols
   __shared__ int wcnt[kRadixWarps][257];
   __shared__ int rs[33];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  if (st->status & ST_BAD_ROWPTR) return;
   const int nlist = st->nradix;
   bool bad = false;
   for (int li = blockIdx.x; li < nlist; li += gridDim.x) {
@@ -820,7 +837,7 @@ FromCsrLayout from_csr_layout(int nnz, int dtype, uint32_t flags) {
   FromCsrLayout L;
   size_t off = align256(sizeof(StatusBlock));
   if (flags & CMRS_SORTED) {
-    L.list = off;  // strips of more than 256 entries only: fewer than nnz
+    L.list = off;  // two lists of list_room() strips
     off += align256((size_t)nnz * 4);
     L.keyA = off;
     off += align256((size_t)nnz * 4);
