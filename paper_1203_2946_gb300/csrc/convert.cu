@@ -883,14 +883,14 @@ int from_csr_impl(int rows, int cols, int nnz, int height, int bits, uint32_t fl
     k_sort_warp<In, DT><<<g, kSortWarps * 32, smem, st>>>(rows, cols, nnz, height, strips, bits, cap, row_ptr, col_ind,
                                                           val_in, strip_ptr, packed, vh, vl, list, sb);
     CMRS_LAUNCH_CHECK();
-    if (nnz > cap) {  // a strip can be longer than that
+    if (strips > 0 && nnz > cap) {  // a strip can be longer than that
       const int smem_b = 16 * (kSortBlockCap + 1);
       CMRS_CUDA_TRY(cudaFuncSetAttribute(k_sort_block<In, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_b));
       k_sort_block<In, DT><<<(int)std::min<int64_t>(strips, (int64_t)sms * 2), kSortThreads, smem_b, st>>>(
           rows, cols, nnz, height, bits, row_ptr, col_ind, val_in, packed, vh, vl, list, sb);
       CMRS_LAUNCH_CHECK();
     }
-    if (nnz > kSortBlockCap) {
+    if (strips > 0 && nnz > kSortBlockCap) {
       int col_bits = 1;
       while (col_bits < 31 && ((int64_t)1 << col_bits) < (int64_t)cols) ++col_bits;
       k_sort_radix<In, DT><<<(int)std::min<int64_t>(strips, (int64_t)sms * 4), kRadixThreads, 0, st>>>(

@@ -59,3 +59,10 @@ def test_overlapping_strips(b, nnz, height, strips):
     rp[:-1] = np.where(s % 2 == 0, 0, nnz)
     rp[-1] = nnz
     assert convert_sorted(b, rp, nnz, 5000, height) == (4, True)
+
+
+# no strip to sort: entries without rows are an invalid RowPtr, not a launch of no blocks
+@pytest.mark.parametrize("first", [0, 1])
+@pytest.mark.parametrize("nnz", [1, 300, 7000])
+def test_entries_without_rows(b, nnz, first):
+    assert convert_sorted(b, np.array([first * nnz]), nnz, 5000, 4) == (4, True)
