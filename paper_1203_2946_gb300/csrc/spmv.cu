@@ -592,12 +592,14 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // this GPU an FP64 warp instruction costs its issue slot whatever its active
 // lanes do: with rows of 27 entries the reduction and the steps' partly filled
 // multiply-adds are two thirds of the FP64 pipe's time (27-point 128^3, h = 4:
-// 355 us; 219 us here, bound by instructions).  Here a warp takes R = 32 / L rows, or the whole strips below that,
+// 355 us; 227 us here, bound by instructions).  Here a warp takes R = 32 / L rows, or the whole strips below that,
 // stages their entries by one bulk copy, and finds each row's entries there
 // with integer work only; L lanes then walk each row in column order, one
-// multiply-add per entry and lane, the row's sum in a register (FP32 forms: four sums, joined at the end,
-// so that their chains stay as short as the paper's 32 partial sums of a
-// strip keep them).  x is gathered at the same place of consecutive rows.
+// multiply-add per entry and lane into one of four sums in registers, joined
+// at the end: chains of at most seven entries, as exact as Algorithm 1's 32
+// partial sums and tree (norm of the FP64 error on rows of 27 entries: 0.95 of
+// Algorithm 1's; one chain a lane, 219 us, 1.15).  x is gathered at the same
+// place of consecutive rows.
 //   An entry's place among its row's entries is found and its index left in
 // list[place][row]; the lanes of a row take every L-th place.  Heights up to 8
 // (kPack): each strip is cut into P parts, a lane each, and every lane counts
@@ -639,7 +641,7 @@ __global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_so
   typedef typename Form<DT>::Stored S;
   typedef typename Form<DT>::Acc A;
   constexpr int CH = DT == CMRS_F64 ? CMRS_SORTED_CH_F64 : 8;
-  constexpr int kAcc = DT == CMRS_F64 ? 1 : 4;
+  constexpr int kAcc = 4;
   constexpr int RS = 32 / L + 2;  // the list's row stride: an odd number of words
   extern __shared__ __align__(128) char smem[];
   __shared__ uint64_t bars[kSortedWarps];
@@ -766,12 +768,17 @@ __global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_so
             }
         }
 #pragma unroll 1
-        for (int j = nfull; j < nmax; ++j)
+        for (int j = nfull; j < nmax; ++j) {  // the sums take turns: moved up one place an entry
+          A t = acc[0];
           if (j < n) {
             const int i = l[j * (L * RS)];
-            acc[0] = fma_acc(Form<DT>::value(vh, vl, i), ld_x(x + (cp[i] >> bits)), acc[0]);
+            t = fma_acc(Form<DT>::value(vh, vl, i), ld_x(x + (cp[i] >> bits)), t);
           }
-        if constexpr (kAcc == 4) acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+          for (int k = 1; k < kAcc; ++k) acc[k - 1] = acc[k];
+          acc[kAcc - 1] = t;
+        }
+        acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
         for (int o = L / 2; o >= 1; o >>= 1) acc[0] += __shfl_down_sync(kAll, acc[0], o);
         if (active && q == 0) {
@@ -1699,7 +1706,7 @@ int sorted_lanes(const cmrs_matrix *A) {
   if (!(A->flags & CMRS_SORTED) || A->height < 2 || A->rows < 1) return 0;
   if ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) return 0;
   const double mu = (double)A->nnz / A->rows;
-  const int highest = mu <= (kF64 ? 14.0 : 10.0) ? 32 : mu <= 14.0 ? 8 : mu <= 28.0 ? (kF64 ? 8 : 4) : mu <= 56.0 ? 3 : 0;
+  const int highest = mu <= (kF64 ? 14.0 : 10.0) ? 32 : mu <= 14.0 ? 8 : mu <= 28.0 ? (kF64 ? 8 : 4) : 0;
   if (A->height > highest) return 0;
   const int L = mu <= 14.0 ? 1 : 2;
   const long long units = ceil_div(A->strips, 32 / L / A->height);
@@ -1713,11 +1720,12 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   typedef typename Form<DT>::Acc Acc;
   const double mu = (double)A->nnz / A->rows;
   const int ns = 32 / L / A->height;
-  // stage: 1.25x an average unit; list: rows of 1.5x the mean and 16 more; at
-  // least Algorithm 1's buffer
+  // stage: 1.25x an average unit; list: rows of 1.5x the mean and 16 more, but
+  // no more than 28 entries a lane, where four sums are as exact as Algorithm
+  // 1's 32; at least Algorithm 1's buffer
   const int cap = (int)std::min<long long>(CMRS_SORTED_CAP,
                                            std::max<long long>(128, ceil_div((long long)(1.25 * mu * ns * A->height), 32) * 32));
-  const int ml = (int)(1.5 * mu) + 16;
+  const int ml = std::min((int)(1.5 * mu) + 16, 28 * L);
   const size_t list = ((size_t)ml * (32 / L + 2) * 2 + 127) & ~size_t(127);
   const size_t warp_bytes = std::max(Stage<DT>::bytes(cap) + list, (size_t)A->height * 32 * sizeof(Acc));
   const size_t smem = kSortedWarps * warp_bytes;

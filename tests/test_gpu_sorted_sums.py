@@ -1,0 +1,93 @@
+"""Which sums column-sorted strips get: the SORTED mapping's (a row by one or two lanes, four sums each) are no less
+exact than those of Algorithm 1, which the same matrix gets when its packed words lie 4 bytes off a 16-byte boundary."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def b():
+    from paper_1203_2946_gb300 import build
+    build.build()
+    from paper_1203_2946_gb300 import binding
+    return binding
+
+
+def padded_rows(rows, mean, spread, seed=4, width=256):
+    """(lengths, columns [rows][longest], mask) with distinct increasing columns near the diagonal, on the GPU."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    lo, hi = round(mean * (1 - spread)), round(mean * (1 + spread))
+    L = torch.randint(lo, hi + 1, (rows,), generator=g, device="cuda")
+    j = torch.arange(hi, device="cuda")[None, :]
+    step = width // L.clamp(min=1)[:, None]
+    at = torch.rand((rows, hi), generator=g, device="cuda")
+    col = torch.arange(rows, device="cuda")[:, None] + j * step + (at * step).long().clamp(max=step - 1)
+    return L, col, j < L[:, None]
+
+
+def exact_sums(V, X):
+    """Row sums of V * X as unevaluated pairs: products by Dekker's splitting, sums by Knuth's two-sum, all in FP64."""
+    def split(a):
+        t = a * 134217729.0
+        h = t - (t - a)
+        return h, a - h
+
+    p = V * X
+    vh, vl = split(V)
+    xh, xl = split(X)
+    e = ((vh * xh - p) + vh * xl + vl * xh) + vl * xl
+    s, c = torch.zeros_like(p[:, 0]), torch.zeros_like(p[:, 0])
+    for k in range(p.shape[1]):
+        t = s + p[:, k]
+        z = t - s
+        c += ((s - (t - z)) + (p[:, k] - z)) + e[:, k]
+        s = t
+    return s, c
+
+
+def products(b, dtype, mean, spread, height, units_per_sm):
+    """(y by the variant's own choice, y by Algorithm 1, the exact sums) on rows enough for so many units per SM."""
+    lanes = 1 if mean <= 14 else 2
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = units_per_sm * sms * (32 // lanes // height * height)
+    L, col, mask = padded_rows(rows, mean, spread)
+    cols = rows + 256
+    g = torch.Generator(device="cuda").manual_seed(9)
+    work = torch.float64 if dtype == 0 else torch.float32
+    V = (torch.rand(col.shape, generator=g, device="cuda", dtype=work) * 2 - 1) * mask
+    x = torch.rand(cols, generator=g, device="cuda", dtype=work) * 2 - 1
+    if dtype == 2:
+        V = V.bfloat16().float()
+    elif dtype == 3:
+        V = V.bfloat16().float() + (V - V.bfloat16().float()).bfloat16().float()
+    rp = torch.zeros(rows + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = L.cumsum(0)
+    M = b.cmrs_from_csr(rp, col[mask].int(), V[mask], cols, height, flags=b.CMRS_SORTED, dtype=dtype)
+    y = b.cmrs_spmv(M, x)
+    pk = torch.zeros(M.nnz + 8, dtype=torch.int32, device="cuda")[1:1 + M.nnz]
+    pk.copy_(M.col_packed[:M.nnz])
+    M.col_packed = pk
+    M.struct.col_packed = pk.data_ptr()
+    alg1 = b.cmrs_spmv(M, x)
+    return y, alg1, exact_sums(V.double(), torch.where(mask, x[col.clamp(max=cols - 1)], 0).double())
+
+
+def error(y, exact):
+    s, c = exact
+    return float(((y.double() - s) - c).norm() / s.norm())
+
+
+# one and two lanes per row, packed counts of 4 and 8 bytes and votes, rows alike and not
+SORTED = [(7, 0.5, 4), (7, 0.0, 16), (13, 0.0, 8), (13, 0.5, 2), (20, 0.5, 3), (27, 0.5, 2),
+          (27, 0.0, 4), (27, 0.0, 3)]
+
+
+@pytest.mark.parametrize("dtype", [0, 1, 2, 3])
+@pytest.mark.parametrize("mean,spread,height", SORTED)
+def test_no_less_exact_than_algorithm_1(b, dtype, mean, spread, height):
+    y, alg1, exact = products(b, dtype, mean, spread, height, 110)
+    assert not torch.equal(y, alg1)  # the SORTED mapping ran
+    # four chains a lane against 32 short partial sums and a tree: the norm of the error is 0.86 to 0.98 of Algorithm
+    # 1's in a model of both orders; 100,000 rows and more sample that to well under 1%
+    assert error(y, exact) <= 1.01 * error(alg1, exact)
