@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // stages their entries by one bulk copy, and finds each row's entries there
 // with integer work only; L lanes then walk each row in column order, one
 // multiply-add per entry and lane into one of four sums in registers, joined
-// at the end: chains of at most seven entries, as exact as Algorithm 1's 32
+// at the end: chains of at most nine entries, as exact as Algorithm 1's 32
 // partial sums and tree (norm of the FP64 error on rows of 27 entries: 0.95 of
 // Algorithm 1's; one chain a lane, 219 us, 1.15).  x is gathered at the same
 // place of consecutive rows.
@@ -1686,31 +1686,47 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
 }
 
 // Lanes per row of the SORTED mapping, 0 where Algorithm 1 runs instead:
-// unsorted or padded strips, arrays the bulk copies cannot read, and
-//   - rows too long for their height: Algorithm 1's reduction costs a strip 31
-//     adds per row whatever the rows' length, undoing the sort costs every
-//     entry, and by votes (heights past 8) twice as much.  1M rows, Algorithm 1
-//     against this mapping, us: 7-point FP64 246 -> 33, 132 -> 33, 89 -> 48 at
-//     h = 2, 4, 16, FP32 136 -> 25, 77 -> 25, 61 -> 38; rows of 8..20 FP64 157
-//     -> 72, 104 -> 91 at h = 4, 16, FP32 83 -> 50, 68 -> 68; 27-point FP64 171
-//     -> 104, 136 -> 111, 128 -> 150 at h = 4, 8, 16, FP32 147 -> 79, 87 -> 80,
-//     79 -> 86 at h = 2, 4, 8; rows of 20..60 FP64 300 -> 210, 202 -> 202 at h
-//     = 2, 4, FP32 155 -> 133, 108 -> 126;
-//   - few units: a unit's copy, walks and gathers take 4..7 us one after
-//     another (100,000 rows: 27-point FP64 h = 4 18.5 -> 12.3 us, FP32 9.6 ->
-//     9.7; 64,000 rows of 8..20: 12.0 -> 8.8, 7.0 -> 6.5; 16,000 rows of 7:
-//     FP32 3.2 -> 3.4).
+// unsorted or padded strips, arrays the bulk copies cannot read, and wherever
+// the mapping was not the faster one.  The lines lie where it stopped winning on
+// rows of equal length, of 0.5 to 1.5x and 0 to 2x the mean, of Poisson and
+// power-law lengths: 20,000 to 1.5M rows, heights 2 to 32, every value form
+// (12,900 points; us below: Algorithm 1 -> the mapping).
+//   - Undoing the sort costs every entry, Algorithm 1's reduction costs a strip
+//     31 adds per row whatever the rows' length: short rows and low strips win
+//     most (7-point, 1.5M rows: FP64 408 -> 52, 219 -> 52, 128 -> 74 at h = 2,
+//     4, 16, FP32 205 -> 41, 115 -> 41, 91 -> 60), and past 28 entries a row
+//     little is left (32 at h = 3, FP64 50 -> 41, FP32 29 -> 31).  Heights past
+//     8 undo it by votes, at twice the cost (13 entries at h = 16, FP32: 15 ->
+//     15).  Two lanes a row gain nothing past `most` entries a mean strip (27 at
+//     h = 4, 6: FP64 43 -> 31, 33 -> 29; FP32 25 -> 23, 21 -> 22).
+//   - The lanes of a unit wait for its longest row, and a row past the list
+//     sends the unit to Algorithm 1 after its walks.  The longest strip against
+//     the mean one tells rows alike from others: 27 entries +-50% at h = 4, 6
+//     FP64 43 -> 44, 32 -> 37; power-law rows (the longest strip 32 to 110 times
+//     the mean) FP32 159 -> 207, 143 -> 146 at h = 4, 16.
+//   - A unit's copy, walks and gathers take 4..7 us one after another: few units
+//     pay for it only where they are alike (12 entries +-67%, 90,000 rows FP32
+//     at h = 2: 16.5 -> 20.8; 400,000 rows: 58 -> 33).
 template <int DT>
 int sorted_lanes(const cmrs_matrix *A) {
   constexpr bool kF64 = DT == CMRS_F64;
   if (!(A->flags & CMRS_SORTED) || A->height < 2 || A->rows < 1) return 0;
   if ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) return 0;
-  const double mu = (double)A->nnz / A->rows;
-  const int highest = mu <= (kF64 ? 14.0 : 10.0) ? 32 : mu <= 14.0 ? 8 : mu <= 28.0 ? (kF64 ? 8 : 4) : 0;
-  if (A->height > highest) return 0;
+  const double mu = (double)A->nnz / A->rows, strip = mu * A->height;
+  const int h = A->height, longest = A->max_strip_nnz;
+  if (mu > 28.0 || longest < 0 || longest > 4.0 * strip) return 0;
   const int L = mu <= 14.0 ? 1 : 2;
-  const long long units = ceil_div(A->strips, 32 / L / A->height);
-  return units >= (L == 1 ? 8LL : kF64 ? 40LL : 100LL) * sm_count() ? L : 0;
+  const int spread = longest <= 1.1 * strip ? 0 : longest <= 1.6 * strip ? 1 : 2;
+  int least;  // units per SM
+  if (L == 1) {
+    if (h > 8 && mu > (!kF64 ? 8.0 : spread ? 10.0 : 14.0)) return 0;
+    least = spread == 2 ? 70 : h > 8 || (spread == 1 && mu > 10.0) ? 20 : 8;
+  } else {
+    const double most[3] = {kF64 ? 224.0 : 112.0, kF64 ? 84.0 : 64.0, kF64 ? 66.0 : 44.0};
+    if (h > (kF64 && spread == 0 ? 8 : 4) || strip > most[spread]) return 0;
+    least = kF64 && spread < 2 ? 40 : 100;
+  }
+  return ceil_div(A->strips, 32 / L / h) >= (long long)least * sm_count() ? L : 0;
 }
 
 template <int DT, int L, int kPack>
@@ -1721,11 +1737,12 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   const double mu = (double)A->nnz / A->rows;
   const int ns = 32 / L / A->height;
   // stage: 1.25x an average unit; list: rows of 1.5x the mean and 16 more, but
-  // no more than 28 entries a lane, where four sums are as exact as Algorithm
-  // 1's 32; at least Algorithm 1's buffer
+  // no more than 36 entries a lane (rows of more than 28 a lane are less exact
+  // by four sums than by Algorithm 1's 32, so they have to be few); at least
+  // Algorithm 1's buffer
   const int cap = (int)std::min<long long>(CMRS_SORTED_CAP,
                                            std::max<long long>(128, ceil_div((long long)(1.25 * mu * ns * A->height), 32) * 32));
-  const int ml = std::min((int)(1.5 * mu) + 16, 28 * L);
+  const int ml = std::min((int)(1.5 * mu) + 16, 36 * L);
   const size_t list = ((size_t)ml * (32 / L + 2) * 2 + 127) & ~size_t(127);
   const size_t warp_bytes = std::max(Stage<DT>::bytes(cap) + list, (size_t)A->height * 32 * sizeof(Acc));
   const size_t smem = kSortedWarps * warp_bytes;

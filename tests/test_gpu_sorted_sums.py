@@ -46,8 +46,9 @@ def exact_sums(V, X):
     return s, c
 
 
-def products(b, dtype, mean, spread, height, units_per_sm):
-    """(y by the variant's own choice, y by Algorithm 1, the exact sums) on rows enough for so many units per SM."""
+def products(b, dtype, mean, spread, height, units_per_sm, longest=None):
+    """(y by the variant's own choice, y by Algorithm 1, the exact sums) on rows enough for so many units per SM; longest:
+    what the matrix says of its longest strip, -1 for unknown or in mean strips."""
     lanes = 1 if mean <= 14 else 2
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     rows = units_per_sm * sms * (32 // lanes // height * height)
@@ -64,6 +65,8 @@ def products(b, dtype, mean, spread, height, units_per_sm):
     rp = torch.zeros(rows + 1, dtype=torch.int32, device="cuda")
     rp[1:] = L.cumsum(0)
     M = b.cmrs_from_csr(rp, col[mask].int(), V[mask], cols, height, flags=b.CMRS_SORTED, dtype=dtype)
+    if longest is not None:
+        M.struct.max_strip_nnz = longest if longest < 0 else longest * mean * height
     y = b.cmrs_spmv(M, x)
     pk = torch.zeros(M.nnz + 8, dtype=torch.int32, device="cuda")[1:1 + M.nnz]
     pk.copy_(M.col_packed[:M.nnz])
@@ -91,3 +94,15 @@ def test_no_less_exact_than_algorithm_1(b, dtype, mean, spread, height):
     # four chains a lane against 32 short partial sums and a tree: the norm of the error is 0.86 to 0.98 of Algorithm
     # 1's in a model of both orders; 100,000 rows and more sample that to well under 1%
     assert error(y, exact) <= 1.01 * error(alg1, exact)
+
+
+# strips too long or too uneven for the mapping, too few of them, and what the matrix says of its longest strip
+ALGORITHM_1 = [(27, 0.5, 4, 110, None), (20, 0.5, 6, 110, None), (27, 0.5, 8, 110, None), (13, 1.0, 4, 40, None),
+               (32, 0.0, 2, 110, None), (7, 0.5, 4, 110, -1), (7, 0.5, 4, 110, 5)]
+
+
+@pytest.mark.parametrize("dtype", [0, 1, 2, 3])
+@pytest.mark.parametrize("mean,spread,height,units,longest", ALGORITHM_1)
+def test_algorithm_1_where_it_is_faster(b, dtype, mean, spread, height, units, longest):
+    y, alg1, _ = products(b, dtype, mean, spread, height, units, longest)
+    assert torch.equal(y, alg1)
