@@ -463,14 +463,13 @@ __global__ void __launch_bounds__(kLaneWarps * 32) k_spmv_lane(int rows, int hei
     const int s = active ? (int)((unsigned)row / h) : s0;
     const uint32_t rr = active ? (uint32_t)row - (uint32_t)s * h : 0;
     const int sa = active ? sp[s] : 0, sb = active ? sp[s + 1] : 0;
-    bool ok = true;
     if (staged) {
-      ok = __all_sync(kAll, mbar_wait_bounded(&bars[w], phase));
+      if (!__all_sync(kAll, mbar_wait_bounded(&bars[w], phase))) {
+        if (lane == 0) atomicOr(status, ST_TIMEOUT);
+        mbar_wait_bounded(&bars[w], phase);  // the late copy lands before the warp leaves
+        break;
+      }
       phase ^= 1;
-    }
-    if (!ok) {
-      if (lane == 0) atomicOr(status, ST_TIMEOUT);
-      break;
     }
     const uint32_t *cp = staged ? reinterpret_cast<const uint32_t *>(stg) : packed;
     const S *vh = staged ? reinterpret_cast<const S *>(stg + Stage<DT>::colp_bytes(cap)) : hi;
@@ -683,6 +682,7 @@ __global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_so
       if (lane == 0) issue_stage<DT>(ea, eb, nnz, packed, hi, lo, stg, cap, &bars[w], pol, &info[w]);
       if (!__all_sync(kAll, mbar_wait_bounded(&bars[w], phase))) {
         if (lane == 0) atomicOr(status, ST_TIMEOUT);
+        mbar_wait_bounded(&bars[w], phase);  // the late copy lands before the warp leaves
         break;
       }
       phase ^= 1;
