@@ -188,10 +188,11 @@ int cmrs_from_csr(int rows, int cols, int nnz, const int32_t *row_ptr, const int
  * < r}, RowPtr[rows] = nnz; within a row, entries keep their strip order (for
  * a sorted matrix each row comes out in column order); col = packed >> bits.
  * Outputs (device): row_ptr_out[rows+1], col_ind_out[nnz], val_out in A's
- * storage form (may be NULL to skip values).  Asynchronous; an entry whose
- * RowInStrip names a row >= rows sets a status the next call does not read:
- * pass a CMRS matrix built by cmrs_from_csr or one that is valid.
- * workspace: >= cmrs_to_csr_workspace() bytes (may be 0 and NULL). */
+ * storage form (may be NULL to skip values).  Asynchronous; pass a CMRS matrix
+ * built by cmrs_from_csr or one that is valid.
+ * workspace: 0 bytes and NULL, or >= cmrs_to_csr_workspace() bytes; then an
+ * entry whose RowInStrip names a row >= rows sets bit 2 of its first word,
+ * which the call neither clears nor reads. */
 int cmrs_to_csr_workspace(const cmrs_matrix *A, size_t *bytes);
 int cmrs_to_csr(const cmrs_matrix *A, int32_t *row_ptr_out, int32_t *col_ind_out, void *val_out,
                 void *workspace, size_t workspace_bytes, void *stream);

@@ -179,7 +179,8 @@ def workspace(nbytes, device="cuda"):
 
 def _scratch(nbytes, device):
     """A device workspace for one call of an entry point that initialises its
-    own status block (the conversions, features and the selector): not zeroed."""
+    own status block (cmrs_from_csr, cmrs_pad_layout, cmrs_features,
+    cmrs_select_strip): not zeroed."""
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
@@ -428,11 +429,8 @@ def cmrs_to_csr(A: Matrix, with_values=True, stream=None):
     ci = torch.empty(max(A.nnz, 1), dtype=torch.int32, device=dev)
     vb = lib().cmrs_val_bytes(A.nnz, A.dtype)
     vo = torch.empty(max(vb, 16), dtype=torch.uint8, device=dev) if with_values else None
-    n = ctypes.c_size_t()
-    _check(lib().cmrs_to_csr_workspace(A.ref(), ctypes.byref(n)), "cmrs_to_csr_workspace")
-    ws = _scratch(n.value, dev)
-    rc = lib().cmrs_to_csr(A.ref(), _ptr(rp), _ptr(ci), _ptr(vo) if with_values else ctypes.c_void_p(0), _ptr(ws),
-                           n.value, _stream(stream))
+    # no workspace: the status word it would hold is neither cleared by the call nor read by anyone
+    rc = lib().cmrs_to_csr(A.ref(), _ptr(rp), _ptr(ci), _ptr(vo) if with_values else 0, 0, 0, _stream(stream))
     _check(rc, "cmrs_to_csr")
     return rp, ci[:A.nnz], vo
 
