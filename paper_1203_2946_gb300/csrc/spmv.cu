@@ -1818,8 +1818,10 @@ int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_ma
       return h <= 4   ? launch_sorted<DT, 1, 4>(A, hi, lo, x, y, row_map, status, st)
              : h <= 8 ? launch_sorted<DT, 1, 8>(A, hi, lo, x, y, row_map, status, st)
                       : launch_sorted<DT, 1, 0>(A, hi, lo, x, y, row_map, status, st);
-    return h <= 4 ? launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st)  // heights up to 8
-                  : launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st);
+    if constexpr (DT == CMRS_F64) {  // the other forms: heights up to 4
+      if (h > 4) return launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st);
+    }
+    return launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st);
   } else if (variant == CMRS_VARIANT_STRIP) {
     static Occ occ;
     const size_t smem = (size_t)kStripWarps * A->height * 32 * sizeof(Acc);
