@@ -80,6 +80,12 @@ enum : uint32_t {
 // ------------------------------------------------------------------ device side
 // The two halves of a programmatic dependent launch (see launch_pdl).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// A load of the earlier kernel's output that stays behind pdl_wait.
+__device__ __forceinline__ int ld_ordered(const int32_t *p) {
+  int v;
+  asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {

@@ -37,11 +37,12 @@ constexpr int kRowCap = 32 * CMRS_ROW_ROWS;   // ROW: entries per shared-memory 
 // entries at 6 CTAs (80 registers), FP64: 9 at 5 CTAs (96 registers).
 // Power-law 4.2M rows, FP32 / FP64 / BF16: 131 / 168 / 130 us against 141 / 167
 // / 139 with two stages (FP32 then 11 entries); FP32 with 9, 11, 15 entries at
-// 7, 6, 5 CTAs: 141, 139, 132 us.
+// 7, 6, 5 CTAs: 141, 139, 132 us.  Launches of one or two waves have their own
+// tiles (merge_few).
 // Matrices whose rows average CMRS_MERGE_LONG_MU entries or more pay for
 // MERGE's per-tile joins more than for L1 misses: they take the _LONG tiles,
 // 15 entries a thread at as many CTAs as fit (27-point 100^3, FP32 / FP64: 77 /
-// 123 us; two stages: 84 / 128).
+// 123 us; two stages: 84 / 128); BF16 only where they are skewed (merge_long).
 #ifndef CMRS_MERGE_LONG_MU
 #define CMRS_MERGE_LONG_MU 16
 #endif
@@ -69,6 +70,9 @@ constexpr int kRowCap = 32 * CMRS_ROW_ROWS;   // ROW: entries per shared-memory 
 #ifndef CMRS_MERGE_E_F32
 #define CMRS_MERGE_E_F32 13
 #endif
+#ifndef CMRS_MERGE_E_F32_FEW
+#define CMRS_MERGE_E_F32_FEW 11
+#endif
 #ifndef CMRS_MERGE_MINB_F64
 #define CMRS_MERGE_MINB_F64 5
 #endif
@@ -89,11 +93,13 @@ constexpr int kMergeThreads = CMRS_MERGE_THREADS;
 #ifndef CMRS_LANE_CTAS
 #define CMRS_LANE_CTAS 0
 #endif
-template <int DT, bool kLong>
+// the tiles of a launch: for short rows, for long ones, for a wave or two of either
+enum { M_SHORT, M_LONG, M_FEW };
+template <int DT, int kTiles>
 struct MergeCfg {
-  static constexpr bool F64 = DT == CMRS_F64;
+  static constexpr bool F64 = DT == CMRS_F64, kLong = kTiles == M_LONG;
   static constexpr int E = F64 ? (kLong ? CMRS_MERGE_E_F64_LONG : CMRS_MERGE_E_F64)
-                               : (kLong ? CMRS_MERGE_E_F32_LONG : CMRS_MERGE_E_F32);
+                               : (kLong ? CMRS_MERGE_E_F32_LONG : kTiles == M_FEW ? CMRS_MERGE_E_F32_FEW : CMRS_MERGE_E_F32);
   static constexpr int Tile = kMergeThreads * E;  // entries per tile, a multiple of 8
   static constexpr int MinBlocks = F64 ? (kLong ? CMRS_MERGE_MINB_F64_LONG : CMRS_MERGE_MINB_F64)
                                        : (kLong ? CMRS_MERGE_MINB_F32_LONG : CMRS_MERGE_MINB_F32);
@@ -101,13 +107,6 @@ struct MergeCfg {
                                   : (kLong ? CMRS_MERGE_CTAS_F32_LONG : CMRS_MERGE_CTAS_F32);
   static_assert(E % 2 == 1 && Tile % 8 == 0, "MERGE: odd entries per thread, 8-entry-aligned tiles");
 };
-// the long-row tiles are a second kernel only where they differ
-template <int DT>
-constexpr bool merge_long_differs() {
-  return MergeCfg<DT, true>::E != MergeCfg<DT, false>::E ||
-         MergeCfg<DT, true>::MinBlocks != MergeCfg<DT, false>::MinBlocks ||
-         MergeCfg<DT, true>::Ctas != MergeCfg<DT, false>::Ctas;
-}
 constexpr int kMergeWarps = kMergeThreads / 32;
 constexpr int kStripWarps = 8;
 enum : uint8_t { F_HEAD = 1, F_TAIL = 2, F_THROUGH = 4 };
@@ -950,10 +949,10 @@ __global__ void __launch_bounds__(kPadWarps * 32, CMRS_PAD_MINB) k_spmv_padded(i
 // ============================================================== MERGE mapping
 // Tile t = entries [T t, T t + T), T = 128 E, staged by bulk copies; thread i
 // owns the E consecutive entries from T t + E i (E = 9 for FP64, 13 for the
-// other forms, 15 for both where rows average 16 entries or more).  It finds their strip by
-// a binary search of StripPtr between the strips holding the tile's first
-// and next tile's first entry (tile_strip[], one small pre-pass), then walks
-// the entries: a row's run is summed by one FMA chain; a run that starts and
+// other forms, 11 for these in one or two waves of CTAs, 15 for all where rows
+// average 16 entries or more).  It finds their strip by a binary search of
+// StripPtr between the strips holding the tile's first and next tile's first
+// entry (tile_strip[], one small pre-pass), then walks the entries: a row's run is summed by one FMA chain; a run that starts and
 // ends inside the thread is written at once; a run cut by the thread's end is
 // joined, after a CTA barrier, by the thread where it started (walking over
 // the following threads' head partials in order); a run cut by the tile's end
@@ -969,8 +968,8 @@ __global__ void k_tile_map(int strips, const int32_t *__restrict__ sp, int tile,
   for (long long t = (a + tile - 1) / tile; t * tile < b && t < ntiles; ++t) tile_strip[t] = s;
 }
 
-template <int DT, bool kLong>
-__global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks))
+template <int DT, int kTiles>
+__global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kTiles>::MinBlocks))
     k_spmv_merge(int rows, int height, int bits, int strips, int nnz,
                                                               const int32_t *__restrict__ sp,
                                                               const uint32_t *__restrict__ packed,
@@ -982,7 +981,7 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
                                                               TileRec *__restrict__ recs, uint32_t *status) {
   typedef typename Form<DT>::Stored S;
   typedef typename Form<DT>::Acc A;
-  constexpr int kMergeE = MergeCfg<DT, kLong>::E, kMergeTile = MergeCfg<DT, kLong>::Tile;
+  constexpr int kMergeE = MergeCfg<DT, kTiles>::E, kMergeTile = MergeCfg<DT, kTiles>::Tile;
   extern __shared__ __align__(128) char smem[];
   __shared__ uint64_t bar;
   __shared__ StageInfo info;
@@ -1015,6 +1014,24 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
   int it = 0;
   for (; t < ntiles; ++it, t += gridDim.x) {
     if (tid == 0) recs[t].tail_flag = 0;
+    // a launch of a wave or two finds the strip holding k0 while the tile's
+    // copy lands, a longer one behind the gathers (its later tiles landed long ago)
+    int few_cur = 0, few_next = 0, few_begin = 0;
+    if constexpr (kTiles == M_FEW) {
+      const long long ta = (long long)t * kMergeTile;
+      const long long k0 = ta + (long long)tid * kMergeE;
+      if (k0 < min(ta + kMergeTile, (long long)nnz)) {
+        few_cur = ld_ordered(tile_strip + t);
+        int shi = (t + 1 < ntiles) ? ld_ordered(tile_strip + t + 1) : strips - 1;
+        while (few_cur < shi) {
+          const int mid = (few_cur + shi + 1) >> 1;
+          if (sp[mid] <= k0) few_cur = mid;
+          else shi = mid - 1;
+        }
+        few_next = sp[few_cur + 1];
+        few_begin = sp[few_cur];
+      }
+    }
     const bool ok = mbar_wait_bounded(&bar, it & 1);
     if (!ok) {
       s_abort = 1;
@@ -1068,17 +1085,20 @@ __global__ void __launch_bounds__(kMergeThreads, (MergeCfg<DT, kLong>::MinBlocks
     const unsigned part = __ballot_sync(0xffffffffu, has);
     if (has) {
       // strip holding k0: the largest s in [s_lo, s_hi] with StripPtr[s] <= k0
-      int slo = tile_strip[t];
-      int shi = (t + 1 < ntiles) ? tile_strip[t + 1] : strips - 1;
-      while (slo < shi) {
-        const int mid = (slo + shi + 1) >> 1;
-        if (sp[mid] <= k0) slo = mid;
-        else shi = mid - 1;
+      int slo = few_cur;
+      if constexpr (kTiles != M_FEW) {
+        slo = tile_strip[t];
+        int shi = (t + 1 < ntiles) ? tile_strip[t + 1] : strips - 1;
+        while (slo < shi) {
+          const int mid = (slo + shi + 1) >> 1;
+          if (sp[mid] <= k0) slo = mid;
+          else shi = mid - 1;
+        }
       }
       int cur = slo;
-      long long next = sp[cur + 1];
+      typename std::conditional<kTiles == M_FEW, int, long long>::type next = kTiles == M_FEW ? few_next : sp[cur + 1];
       // does the entry before k0 (previous thread, or previous tile for thread 0) lie in the same row?
-      const bool cont_in = k0 > sp[cur] && (cprev & mask) == (c[0] & mask);
+      const bool cont_in = k0 > (kTiles == M_FEW ? few_begin : sp[cur]) && (cprev & mask) == (c[0] & mask);
       // the row of every entry: integer work only.  When all of the thread's
       // entries lie in the strip holding k0 (the usual case) no StripPtr walk
       // is needed; otherwise the walk may diverge.
@@ -1593,8 +1613,9 @@ int occupancy(K kernel, int threads, size_t smem, Occ &cache, size_t smem_cap = 
 // takes (cmrs.h states cmrs_spmv_noalloc's limits in these)
 size_t merge_ws_bytes(int nnz, int dtype) {
   const int tile = dtype == CMRS_F64 ? 1152 : 1408;
-  static_assert(MergeCfg<CMRS_F64, false>::Tile >= 1152 && MergeCfg<CMRS_F64, true>::Tile >= 1152 &&
-                MergeCfg<CMRS_F32, false>::Tile >= 1408 && MergeCfg<CMRS_F32, true>::Tile >= 1408, "MERGE workspace");
+  static_assert(MergeCfg<CMRS_F64, M_SHORT>::Tile >= 1152 && MergeCfg<CMRS_F64, M_LONG>::Tile >= 1152 &&
+                MergeCfg<CMRS_F32, M_SHORT>::Tile >= 1408 && MergeCfg<CMRS_F32, M_LONG>::Tile >= 1408 &&
+                MergeCfg<CMRS_F32, M_FEW>::Tile >= 1408, "MERGE workspace");
   const long long ntiles = ceil_div(nnz, tile);
   return 256 + align256((size_t)(ntiles + 1) * 4) + align256((size_t)ntiles * sizeof(TileRec));
 }
@@ -1666,23 +1687,49 @@ int launch_padded(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   return CMRS_OK;
 }
 
+// Whether the rows count as long ones.  BF16's random gathers want the short
+// rows' tiles at every length unless the rows are skewed (40 random entries a
+// row, 40M entries: 190 us against 200; power-law rows of 16, 16M entries: 114
+// against 107).
+template <int DT>
+bool merge_long(const cmrs_matrix *A) {
+  if ((double)A->nnz < CMRS_MERGE_LONG_MU * (double)A->rows) return false;
+  if (DT != CMRS_BF16 || A->max_strip_nnz < 0) return true;
+  return (double)A->max_strip_nnz * A->rows > 8.0 * A->height * A->nnz;
+}
+
+// Whether a launch takes the tiles for a wave or two of CTAs: the strips found
+// while the tile lands, and 11 entries a thread in the FP32-accumulated forms.
+// A wave takes longer with 13 entries than with 11, so up to two waves the
+// larger tiles pay only where they save one (rows of 4, FP32, 11 and 13
+// entries: 80,000 entries 7.8, 8.3 us; 1.35M, one wave instead of two, 16.0,
+// 14.4; 2.4M 20.8, 22.2); past two they pay anyway (power-law rows, 3.1M
+// entries 33.2, 30.5; 7.9M 75.3, 66.0).  Long rows take them for one wave (40
+// entries a row, 0.8M entries FP64 10.2 us against 10.5).
+template <int DT>
+bool merge_few(int nnz, bool long_rows) {
+  const long long ctas = (long long)MergeCfg<DT, M_FEW>::Ctas * sm_count();
+  const long long waves = ceil_div(nnz, MergeCfg<DT, M_SHORT>::Tile * ctas);
+  return waves < (long_rows ? 2 : 3) && waves == ceil_div(nnz, MergeCfg<DT, M_FEW>::Tile * ctas);
+}
+
 // MERGE: tile map, the product, the fix-up of rows cut by tile boundaries
-template <int DT, bool kLong>
+template <int DT, int kTiles>
 int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, const typename Form<DT>::Stored *lo,
                  const typename Form<DT>::Acc *x, typename Form<DT>::Acc *y, uint32_t *status, char *ws,
                  cudaStream_t st) {
   typedef typename Form<DT>::Acc Acc;
   static Occ occ;
-  constexpr int kMergeTile = MergeCfg<DT, kLong>::Tile;
+  constexpr int kMergeTile = MergeCfg<DT, kTiles>::Tile;
   const int ntiles = (int)ceil_div(A->nnz, kMergeTile);
   int32_t *tile_strip = reinterpret_cast<int32_t *>(ws + 256);
   TileRec *recs = reinterpret_cast<TileRec *>(ws + 256 + align256((size_t)(ntiles + 1) * 4));
   k_tile_map<<<(int)ceil_div(A->strips, 256), 256, 0, st>>>(A->strips, A->strip_ptr, kMergeTile, ntiles, tile_strip);
   CMRS_LAUNCH_CHECK();
   const size_t smem = Stage<DT>::bytes(kMergeTile);
-  const int per_sm = occupancy(k_spmv_merge<DT, kLong>, kMergeThreads, smem, occ, 0, MergeCfg<DT, kLong>::Ctas);
+  const int per_sm = occupancy(k_spmv_merge<DT, kTiles>, kMergeThreads, smem, occ, 0, MergeCfg<DT, kTiles>::Ctas);
   const int grid = (int)std::min<long long>(ntiles, (long long)per_sm * sm_count());
-  int rc = launch_pdl(k_spmv_merge<DT, kLong>, (unsigned)grid, kMergeThreads, smem, st, A->rows, A->height, A->bits,
+  int rc = launch_pdl(k_spmv_merge<DT, kTiles>, (unsigned)grid, kMergeThreads, smem, st, A->rows, A->height, A->bits,
                       A->strips, A->nnz, A->strip_ptr, A->col_packed, hi, lo, x, y, tile_strip, ntiles, recs, status);
   if (rc) return rc;
   return launch_pdl(k_merge_fixup<Acc>, (unsigned)ceil_div(ntiles, 256), 256, 0, st, ntiles, A->rows, recs, y);
@@ -1839,11 +1886,10 @@ int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_ma
       default: return launch_padded<DT, 8>(A, hi, lo, x, y, row_map, status, ws, ws_bytes, st);
     }
   } else {
-    if constexpr (merge_long_differs<DT>()) {
-      if ((double)A->nnz >= CMRS_MERGE_LONG_MU * (double)A->rows)
-        return launch_merge<DT, true>(A, hi, lo, x, y, status, ws, st);
-    }
-    return launch_merge<DT, false>(A, hi, lo, x, y, status, ws, st);
+    const bool long_rows = merge_long<DT>(A);
+    if (merge_few<DT>(A->nnz, long_rows)) return launch_merge<DT, M_FEW>(A, hi, lo, x, y, status, ws, st);
+    if (long_rows) return launch_merge<DT, M_LONG>(A, hi, lo, x, y, status, ws, st);
+    return launch_merge<DT, M_SHORT>(A, hi, lo, x, y, status, ws, st);
   }
   return CMRS_OK;
 }
