@@ -660,21 +660,22 @@ __global__ void __launch_bounds__(kRadixThreads) k_sort_radix(int rows, int cols
 }
 
 // ---------------------------------------------------------------- CMRS -> CRS
-// Sorted strips, one warp each: a stable counting sort by RowInStrip.  The
-// strip's words are staged in shared memory and its rows counted on the way;
-// an exclusive scan over the rows gives RowPtr[s*h + r] = StripPtr[s] +
-// #(RIS < r); then each chunk of 32 entries finds its places (place_in_row)
-// and leaves its index there, so that columns and values go out coalesced, the
-// values gathered from the strip's own range.  A strip longer than the stage
-// is walked in global memory, its entries scattered to their places.  With
-// every chunk walked that way, one load round trip after another, the kernel
-// took 275 us for 20M FP64 entries in strips of 320; 104 us staged.
+// Sorted strips, one warp each: a stable counting sort by RowInStrip.  Its rows
+// are counted; an exclusive scan over the rows gives RowPtr[s*h + r] =
+// StripPtr[s] + #(RIS < r).  Staged (launch_to_csr says where): the strip's
+// words are kept in shared memory on the way, then each chunk of 32 entries
+// finds its places (place_in_row) and leaves its index there, so that columns
+// and values go out coalesced, the values gathered from the strip's own range.
+// Walked: a chunk of 32 entries after the other is read again, ranked by a
+// match of its rows, and scattered to its places, one load round trip after
+// another (20M FP64 entries in strips of 320: 275 us, staged 104 us).
 //   Unsorted strips (kSorted false) already hold their entries in CRS order:
 // the entry arrays are copied with the row bits dropped (coalesced, kPackU
 // batches in flight per lane) and RowPtr[s*h + r] is the first entry of
 // row r, found by a binary search of RowInStrip.
 constexpr int kToCsrWarps = 8, kToCsrCap = 2048;  // most entries staged per warp
-template <typename V, bool kSorted>
+enum { T_PLAIN, T_STAGED, T_WALKED };  // unsorted strips; sorted ones, from the stage or from global memory
+template <typename V, int kForm>
 __global__ void __launch_bounds__(kToCsrWarps * 32) k_to_csr(
     int rows, int nnz, int height, int bits, int strips, int cap, const int32_t *__restrict__ sp,
     const uint32_t *__restrict__ packed, const V *__restrict__ vin, const V *__restrict__ vin_lo,
@@ -685,7 +686,7 @@ __global__ void __launch_bounds__(kToCsrWarps * 32) k_to_csr(
   const unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int *cnt = cnt_all[w];
-  uint32_t *words = reinterpret_cast<uint32_t *>(smem) + (size_t)w * cap;                        // kSorted: the strip
+  uint32_t *words = reinterpret_cast<uint32_t *>(smem) + (size_t)w * cap;                        // T_STAGED: the strip
   uint16_t *from = reinterpret_cast<uint16_t *>(smem + (size_t)kToCsrWarps * cap * 4) + (size_t)w * cap;  // CRS order
   const uint32_t mask = (1u << bits) - 1;
   const int nw = gridDim.x * kToCsrWarps;
@@ -695,7 +696,7 @@ __global__ void __launch_bounds__(kToCsrWarps * 32) k_to_csr(
     const int32_t a = sp[s], b = sp[s + 1];
     const int64_t row0 = (int64_t)s * height;
     const int nrow = (int)std::min<int64_t>(height, rows - row0);
-    if (!kSorted) {
+    if (kForm == T_PLAIN) {
       int32_t start = a;
       if (lane > 0 && lane < nrow) {
         int32_t lo = a, hi = b;
@@ -738,7 +739,7 @@ __global__ void __launch_bounds__(kToCsrWarps * 32) k_to_csr(
     }
     cnt[lane] = 0;
     __syncwarp();
-    const bool staged = b - a <= cap;  // warp-uniform
+    const bool staged = kForm == T_STAGED && b - a <= cap;  // warp-uniform
     for (int32_t i0 = a; i0 < b; i0 += 32 * kPackU) {
       uint32_t p[kPackU];
 #pragma unroll
@@ -809,19 +810,31 @@ __global__ void __launch_bounds__(kToCsrWarps * 32) k_to_csr(
       __syncwarp();  // the stage is reused by the next strip
       continue;
     }
+    __syncwarp();
+    cnt[lane] = next;  // running insertion point of row `lane`
+    __syncwarp();
     for (int32_t i0 = a; i0 < b; i0 += 32) {
       const int32_t i = i0 + lane;
-      const uint32_t p = i < b ? packed[i] : 0u;
-      const int r = (int)(p & mask);
-      const bool valid = i < b && r < nrow;
-      const int dst = place_in_row<5>(r, valid, next);
-      if (valid) {
+      int r = 32;
+      uint32_t p = 0;
+      if (i < b) {
+        p = packed[i];
+        r = (int)(p & mask);
+        if (r >= nrow) r = 32;
+      }
+      const uint32_t peers = __match_any_sync(kAll, r);
+      const int rank = __popc(peers & ((1u << lane) - 1));
+      if (r < 32) {
+        const int dst = cnt[r] + rank;
         col_out[dst] = (int32_t)(p >> bits);
         if (vout) {
           vout[dst] = vin[i];
           if (vout_lo) vout_lo[dst] = vin_lo[i];
         }
       }
+      __syncwarp();
+      if (r < 32 && (__ffs(peers) - 1) == lane) cnt[r] += __popc(peers);
+      __syncwarp();
     }
     __syncwarp();
   }
@@ -998,7 +1011,7 @@ int launch_to_csr(bool sorted, cudaStream_t st, const cmrs_matrix *A, const V *v
                   int32_t *col_out, V *vout, V *vout_lo, uint32_t *status) {
   if (!sorted) {
     const int g = (int)std::min<int64_t>(ceil_div(A->strips, kToCsrWarps), (int64_t)sm_count() * 8);
-    k_to_csr<V, false><<<g, kToCsrWarps * 32, 0, st>>>(A->rows, A->nnz, A->height, A->bits, A->strips, 0, A->strip_ptr,
+    k_to_csr<V, T_PLAIN><<<g, kToCsrWarps * 32, 0, st>>>(A->rows, A->nnz, A->height, A->bits, A->strips, 0, A->strip_ptr,
                                                        A->col_packed, vin, vin_lo, row_ptr, col_out, vout, vout_lo,
                                                        status);
     return set_cuda_error(cudaGetLastError());
@@ -1007,13 +1020,30 @@ int launch_to_csr(bool sorted, cudaStream_t st, const cmrs_matrix *A, const V *v
   // memory and short ones leave room for more warps
   const int64_t avg = A->nnz / A->strips;
   const int cap = (int)std::min<int64_t>(kToCsrCap, (avg + avg / 2) / 32 * 32 + 64);
+  // The stage pays where it saves a strip several load round trips and still
+  // leaves warps to hide the rest (us walked -> staged, FP64): strips of 20, 40,
+  // 80 entries 56 -> 105, 61 -> 94, 54 -> 58; of 160, 320, 640 76 -> 49, 92 ->
+  // 46, 136 -> 67; of 2,000 and 2,500 91 -> 151, 105 -> 179.  Of few rows, long
+  // strips scatter little (1,000 entries of one row 56 -> 60; of 8 rows 114 ->
+  // 58), and 2-byte values less (160 entries of 4 rows 33 -> 38).  A strip far
+  // past the stage is walked alone anyway, faster without one.
+  const bool narrow = sizeof(V) == 2 && !vin_lo;
+  const bool staged = avg >= 100 && avg <= std::min(1800, 600 * A->height) &&
+                      (!narrow || A->height > 8 || (A->height == 8 && avg >= 200)) && A->max_strip_nnz <= 8 * cap;
+  if (!staged) {
+    const int g = (int)std::min<int64_t>(ceil_div(A->strips, kToCsrWarps), (int64_t)sm_count() * 8);
+    k_to_csr<V, T_WALKED><<<g, kToCsrWarps * 32, 0, st>>>(A->rows, A->nnz, A->height, A->bits, A->strips, 0, A->strip_ptr,
+                                                          A->col_packed, vin, vin_lo, row_ptr, col_out, vout, vout_lo,
+                                                          status);
+    return set_cuda_error(cudaGetLastError());
+  }
   const size_t smem = (size_t)kToCsrWarps * cap * 6;
-  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_to_csr<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  CMRS_CUDA_TRY(cudaFuncSetAttribute(k_to_csr<V, T_STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      kToCsrWarps * kToCsrCap * 6));
   int per_sm = 0;
-  CMRS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_to_csr<V, true>, kToCsrWarps * 32, smem));
+  CMRS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_to_csr<V, T_STAGED>, kToCsrWarps * 32, smem));
   const int g = (int)std::min<int64_t>(ceil_div(A->strips, kToCsrWarps), (int64_t)sm_count() * std::max(1, per_sm));
-  k_to_csr<V, true><<<g, kToCsrWarps * 32, smem, st>>>(A->rows, A->nnz, A->height, A->bits, A->strips, cap,
+  k_to_csr<V, T_STAGED><<<g, kToCsrWarps * 32, smem, st>>>(A->rows, A->nnz, A->height, A->bits, A->strips, cap,
                                                        A->strip_ptr, A->col_packed, vin, vin_lo, row_ptr, col_out, vout,
                                                        vout_lo, status);
   return set_cuda_error(cudaGetLastError());

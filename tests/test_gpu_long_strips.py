@@ -42,3 +42,23 @@ def test_pad(b, h, slots, dtype):
     for k in range(2 if dtype == 3 else 1):
         want = torch.where(src >= 0, v0[k * M.nnz:(k + 1) * M.nnz][src.clamp(min=0)], 0)
         assert torch.equal(v1[k * P.nnz:(k + 1) * P.nnz], want)
+
+
+# sorted strips to CRS: walked (short, long, few rows, one strip far past the stage) and staged
+TO_CSR = {"short": (lambda r: r.integers(0, 9, 700), 4), "staged": (lambda r: r.integers(20, 60, 700), 8),
+          "staged_tall": (lambda r: r.integers(4, 9, 900), 32), "long": (lambda r: r.integers(100, 300, 300), 16),
+          "one_row": (lambda r: r.integers(600, 900, 40), 1), "one_long": (lambda r: np.where(np.arange(800) == 300, 8000, 30), 8)}
+
+
+@pytest.mark.parametrize("case", sorted(TO_CSR))
+@pytest.mark.parametrize("dtype", [0, 1, 2, 3])
+def test_sorted_to_csr(b, case, dtype):
+    make, h = TO_CSR[case]
+    a = inputs.from_lengths(make(np.random.default_rng(2)), 9000, seed=3)
+    M, plain = convert(b, a, h, dtype, b.CMRS_SORTED), convert(b, a, h, dtype)
+    rp, ci, v = b.cmrs_to_csr(M)
+    assert np.array_equal(rp.cpu().numpy(), a.row_ptr) and np.array_equal(ci.cpu().numpy(), a.col_ind)
+    width = {0: 8, 1: 4, 2: 2, 3: 2}[dtype]
+    pad = b.lib().cmrs_pad8(a.nnz) * 2
+    for at in (0, pad) if dtype == 3 else (0,):  # columns were in order: the plain matrix's values, byte for byte
+        assert torch.equal(v[at:at + width * a.nnz], plain.val[at:at + width * a.nnz])
