@@ -10,11 +10,15 @@
 // min(32, next_pow2(k / 4))): a k = 32 row takes 8 lanes and a warp works
 // four rows at once.  Otherwise lane g accumulates column c0 + g (G =
 // min(32, next_pow2(k))).  Columns beyond the group are done in further
-// passes over the row; each column's sum is one FMA chain in entry order
-// either way.  Work units (matrix, row range) are fetched by warps from a
-// device queue (one atomic per unit), which balances uneven matrices.
+// passes over the row.  A column's sum is one FMA chain in entry order, or two,
+// of the even and the odd entries, joined at the end, where rows of 8 entries
+// or more have one lane of columns (k = 1, 4).  Work units (matrix, row range)
+// are fetched by warps from a device queue (one atomic per unit), which balances
+// uneven matrices.
 //
-// What bounds it is the L1 data pipe: a warp's rows lie apart in the entry
+// What bounds a large batch is the L1 data pipe (rows that are short or long for
+// a stage, and wide products whose X stays in L2, wait on round trips instead
+// and are walked without one, see below): a warp's rows lie apart in the entry
 // streams, so a column word and a value read from global memory cost a line
 // each per row and entry, as much as the gather of X itself (78% busy, three
 // lines an entry).  So a warp copies the entries of up to 32 consecutive rows
@@ -69,7 +73,7 @@ constexpr size_t kSpmmSmem = kSpmmWarps * Stage<CMRS_F32>::bytes(kSpmmCap);
 struct Desc {
   int32_t rows, height, bits, k, vec, nnz;
   int32_t stage;  // the arrays' alignment allows bulk copies
-  int32_t split;  // lanes groups sharing one row (1 or 2)
+  int32_t split;  // lane groups sharing one row (1 or 2)
   const int32_t *sp;
   const uint32_t *packed;
   const float *val;
@@ -333,6 +337,188 @@ __global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_one(Desc 
   warp_stage_end(st);
 }
 
+// ------------------------------------------------------------------ walked
+// The same sums without a stage: every lane finds its row's bounds and reads
+// column words and values from global memory (the lanes of a row share each
+// line), at 40 warps per SM instead of 28 and with no round trip before the
+// first gather.  The faster way where the stage holds too little (see
+// spmm_staged, plan_staged): rows too short or too long for it, tall strips,
+// and wide products whose X stays in L2.
+constexpr int kWalkThreads = 256;
+constexpr int kWalkD = 2;  // X gathers in flight per lane (more raise the 48 registers that 5 CTAs leave)
+
+// Rows [row0, row1) of matrix d, processed by one warp: columns g, g + G, ...
+// of a row from its entries q, q + L, ..., summed as spmm_row sums them.  Of
+// 16-byte columns the next batch's column words and values are loaded while
+// this batch's gathers are in flight.
+template <typename V, int L>
+__device__ __forceinline__ void walk_rows(const Desc &d, int row0, int row1) {
+  constexpr bool kAhead = sizeof(V) == 16;
+  const int lane = threadIdx.x & 31;
+  const int kv = kAhead ? d.k >> 2 : d.k;
+  const int G = spmm_lanes(d.k, kAhead), per = 32 / (G * L);
+  const int g = lane & (G - 1), q = (lane / G) & (L - 1), sub = lane / (G * L);
+  const uint32_t mask = (1u << d.bits) - 1;
+  const V *X = reinterpret_cast<const V *>(d.X);
+  V *Y = reinterpret_cast<V *>(d.Y);
+  for (int rb = row0; rb < row1; rb += per) {
+    const int row = rb + sub;
+    const bool active = row < row1;
+    int k0 = 0, k1 = 0;
+    if (active) {
+      const int s = row / d.height;
+      k0 = __ldg(d.sp + s);
+      k1 = __ldg(d.sp + s + 1);
+      if (d.height > 1) {
+        const uint32_t r = (uint32_t)(row - s * d.height);
+        k0 = lb_ris_g(d.packed, 0, k0, k1, r, mask);
+        k1 = lb_ris_g(d.packed, 0, k0, k1, r + 1, mask);
+      }
+      k0 += q;
+    }
+    for (int c0 = 0; c0 < kv; c0 += G) {  // warp-uniform
+      const int col = c0 + g;
+      V acc = {};
+      if (active && col < kv) {
+        uint32_t pn[kWalkD];
+        float vn[kWalkD];
+        if (kAhead) {
+#pragma unroll
+          for (int u = 0; u < kWalkD; ++u)
+            if (k0 + L * u < k1) {
+              pn[u] = __ldg(d.packed + k0 + L * u);
+              vn[u] = __ldg(d.val + k0 + L * u);
+            }
+        }
+        for (int j = k0; j < k1; j += L * kWalkD) {
+          V xv[kWalkD];
+          float vv[kWalkD];
+#pragma unroll
+          for (int u = 0; u < kWalkD; ++u) {
+            if (kAhead) {
+              vv[u] = vn[u];
+              if (j + L * u < k1) xv[u] = __ldg(X + (size_t)(pn[u] >> d.bits) * kv + col);
+            } else if (j + L * u < k1) {
+              const uint32_t p = __ldg(d.packed + j + L * u);
+              vv[u] = __ldg(d.val + j + L * u);
+              xv[u] = __ldg(X + (size_t)(p >> d.bits) * kv + col);
+            }
+          }
+          if (kAhead) {
+#pragma unroll
+            for (int u = 0; u < kWalkD; ++u)
+              if (j + L * (kWalkD + u) < k1) {
+                pn[u] = __ldg(d.packed + j + L * (kWalkD + u));
+                vn[u] = __ldg(d.val + j + L * (kWalkD + u));
+              }
+          }
+#pragma unroll
+          for (int u = 0; u < kWalkD; ++u)
+            if (j + L * u < k1) fma_to(acc, vv[u], xv[u]);
+        }
+        if (L == 1) Y[(size_t)row * kv + col] = acc;
+      }
+      if (L > 1) {
+        join(acc, G);
+        if (active && q == 0 && col < kv) Y[(size_t)row * kv + col] = acc;
+      }
+    }
+  }
+}
+// kSplit: some matrices have two lane groups per row (compiled apart: together
+// they spill)
+template <bool kSplit>
+__global__ void __launch_bounds__(kWalkThreads, 5) k_spmm_walk_queue(const Desc *__restrict__ descs,
+                                                                     const Unit *__restrict__ units, int nunits,
+                                                                     QueueHead *q) {
+  for (;;) {
+    unsigned u = 0;
+    if ((threadIdx.x & 31) == 0) u = atomicAdd(&q->taken[0], 1u);
+    u = __shfl_sync(0xffffffffu, u, 0);
+    if (u >= (unsigned)nunits) break;
+    const Unit un = units[u];
+    const Desc d = descs[un.mat];
+    if (kSplit && d.split > 1) {
+      if (d.vec) walk_rows<float4, 2>(d, un.row0, un.row1);
+      else walk_rows<float, 2>(d, un.row0, un.row1);
+    } else {
+      if (d.vec) walk_rows<float4, 1>(d, un.row0, un.row1);
+      else walk_rows<float, 1>(d, un.row0, un.row1);
+    }
+  }
+}
+
+// One matrix, no queue: warp w takes rows [w*rpw, (w+1)*rpw).
+template <typename V, int L>
+__global__ void __launch_bounds__(kWalkThreads, 5) k_spmm_walk_one(Desc d, int rows_per_warp) {
+  const long long r0 = (((long long)blockIdx.x * kWalkThreads + threadIdx.x) >> 5) * rows_per_warp;
+  if (r0 >= d.rows) return;
+  walk_rows<V, L>(d, (int)r0, (int)std::min<long long>(r0 + rows_per_warp, d.rows));
+}
+int launch_walk_one(const Desc &d, cudaStream_t st) {
+  const int per = 32 / (spmm_lanes(d.k, d.vec) * d.split);
+  const int grid = (int)ceil_div(ceil_div(d.rows, per) * 32, kWalkThreads);
+  if (d.vec && d.split == 1) k_spmm_walk_one<float4, 1><<<grid, kWalkThreads, 0, st>>>(d, per);
+  else if (d.vec) k_spmm_walk_one<float4, 2><<<grid, kWalkThreads, 0, st>>>(d, per);
+  else if (d.split == 1) k_spmm_walk_one<float, 1><<<grid, kWalkThreads, 0, st>>>(d, per);
+  else k_spmm_walk_one<float, 2><<<grid, kWalkThreads, 0, st>>>(d, per);
+  CMRS_LAUNCH_CHECK();
+  return CMRS_OK;
+}
+
+// Whether one matrix's product takes the stage: where it was the faster way on
+// 1,290 points (0.5 to 1,500 entries a row, heights 1 to 32, 1 to 64 columns; us
+// walked -> staged).  A row's words have to be many, or read by many lanes, to
+// pay for the copy's round trip (5-point rows, 1M: k = 1, 4 13 -> 23, 16 -> 27),
+// and a group of rows has to fit the stage (200 entries a row, k = 2 78 -> 129;
+// strips of 32 rows of 40, k = 8 54 -> 80); narrow products of 12 to 65 entries
+// a row do both (40, 200,000 rows: k = 1 43 -> 23, k = 5 84 -> 71).  Rows of 300
+// and more are read from global memory either way, few columns with four
+// gathers in flight (400, 15,000 rows: k = 1 89 -> 31).
+bool spmm_staged(const Desc &d) {
+  const double mu = (double)d.nnz / d.rows, strip = mu * d.height;
+  if (!d.stage) return false;
+  if (mu >= 300.0) return d.k <= 5;
+  if (strip > 600.0) return false;
+  if (d.k == 1) return mu >= 12.0 && mu <= 65.0;
+  if (d.k == 2) return mu >= 15.0 && mu <= 65.0;
+  if (!d.vec) return (d.height >= 4 || mu >= 4.0) && mu <= 130.0;
+  if (d.k == 4) return mu >= 18.0 && mu <= 55.0;
+  if (d.k == 8) return d.height >= 2 && mu <= 6.0;
+  return d.height >= 2 && mu <= 35.0 && d.rows >= 60000;
+}
+
+// Whether a batch does: by the sum of its products' times (nnz (24 + k), as
+// one-launch batches of one k take them) with what the stage gains on each, from
+// 645 batches of one matrix and 120 of many: narrow products 1.5 to 2.5 times
+// the speed; wide ones whose X outgrows L2 (the blocks of the queue keep its
+// rows in L1) 1.2, others 0.75 to 1.1 (15 matrices of 16,000 rows, k = 4, 8, 16:
+// 74 us walked, 83 staged).
+bool plan_staged(const std::vector<Desc> &descs) {
+  double wide = 0.0;  // bytes of the wide products' X and Y
+  for (const Desc &d : descs)
+    if (d.vec && d.k >= 8) wide += 8.0 * d.rows * d.k;
+  double walked = 0.0, staged = 0.0;
+  for (const Desc &d : descs) {
+    if (d.nnz == 0) continue;
+    const double mu = (double)d.nnz / d.rows, work = (double)d.nnz * (24 + d.k);
+    double gain = d.k == 1 ? 2.2 : 1.6;
+    if (d.k == 1 || (d.vec && d.k == 4)) gain = mu < 3.0 ? 0.85 : mu < 5.5 ? 0.95 : gain;
+    if (d.vec && d.k >= 8)
+      gain = mu >= 300.0                            ? 1.3
+             : wide > 128e6                         ? (mu >= 12.0 ? 1.2 : d.height > 1 ? 1.1 : 0.92)
+             : mu * d.height > 600.0                ? 0.75
+             : wide > 32e6                          ? (d.height > 1 ? 1.1 : 0.95)
+             : d.k == 8                             ? (mu >= 110.0 ? 1.2 : 0.8)
+             : d.k > 32                             ? 0.75
+             : d.height > 1                         ? (mu <= 18.0 ? 1.1 : d.k > 16 ? 1.0 : 0.88)
+                                                    : 0.86;
+    walked += work;
+    staged += work / (d.stage ? gain : 0.8);
+  }
+  return staged <= walked;
+}
+
 int spmm_smem_opt_in() {
   CMRS_CUDA_TRY(cudaFuncSetAttribute(k_spmm_queue, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpmmSmem));
   CMRS_CUDA_TRY(cudaFuncSetAttribute(k_spmm_one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpmmSmem));
@@ -396,6 +582,7 @@ struct cmrs_spmm_plan {
   QueueHead *d_q = nullptr;
   int grid = 0;
   Shares sh = {};
+  bool staged = false, split = false;  // split: a walked plan with two lane groups per row somewhere
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -414,6 +601,7 @@ extern "C" int cmrs_spmm(const cmrs_matrix *A, int k, const float *X, float *Y, 
   // rows per warp: up to 32 (one stage), fewer while the warps would not fill
   // the SMs twice, whole groups of the rows a warp works at once
   const int per = 32 / (spmm_lanes(k, d.vec) * d.split);
+  if (!spmm_staged(d)) return launch_walk_one(d, st);
   const long long resident = (long long)sm_count() * CMRS_SPMM_MINB * kSpmmWarps;
   const int rpw = (int)std::max<long long>(per, std::min<long long>(32, A->rows / (2 * resident)) / per * per);
   const long long warps = ceil_div(A->rows, rpw);
@@ -479,6 +667,16 @@ static void deal_wide(const Shares &sh, const int32_t *k, std::vector<Unit> &uni
   }
 }
 
+// The queue's reset and the persistent launch.
+static cudaError_t enqueue_plan(const cmrs_spmm_plan *p, cudaStream_t st) {
+  const cudaError_t e = cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int) * (p->staged ? p->sh.shares : 1), st);
+  if (e != cudaSuccess) return e;
+  if (p->staged) k_spmm_queue<<<p->grid, kSpmmThreads, kSpmmSmem, st>>>(p->d_desc, p->d_units, p->sh, p->d_q);
+  else if (p->split) k_spmm_walk_queue<true><<<p->grid, kWalkThreads, 0, st>>>(p->d_desc, p->d_units, p->nunits, p->d_q);
+  else k_spmm_walk_queue<false><<<p->grid, kWalkThreads, 0, st>>>(p->d_desc, p->d_units, p->nunits, p->d_q);
+  return cudaSuccess;
+}
+
 extern "C" int cmrs_spmm_plan_workspace(int batch, const cmrs_matrix *const *A, const int32_t *k, int work_target,
                                         size_t *bytes) {
   if (batch < 0 || !bytes || (batch > 0 && (!A || !k)) || work_target < 1) return CMRS_ERR_ARG;
@@ -509,15 +707,18 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
   std::vector<Unit> units;
   build_units(batch, A, k, work_target, units);
   const Shares sh = make_shares(units.size());
-  deal_wide(sh, k, units);
   std::vector<Desc> descs(batch);
   for (int b = 0; b < batch; ++b) descs[b] = make_desc(A[b], k[b], X[b], Y[b]);
+  const bool staged = plan_staged(descs);
+  if (staged) deal_wide(sh, k, units);
   cmrs_spmm_plan *p = new (std::nothrow) cmrs_spmm_plan();
   if (!p) return CMRS_ERR_ARG;
   char *ws = reinterpret_cast<char *>(workspace);
   p->batch = batch;
   p->nunits = (int)units.size();
   p->sh = sh;
+  p->staged = staged;
+  for (const Desc &d : descs) p->split |= d.split > 1;
   p->work_target = work_target;
   p->d_q = reinterpret_cast<QueueHead *>(ws);
   p->d_desc = reinterpret_cast<Desc *>(ws + align256(sizeof(QueueHead)));
@@ -538,7 +739,8 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
     return arc;
   }
   int per_sm = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmm_queue, kSpmmThreads, kSpmmSmem);
+  if (staged) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmm_queue, kSpmmThreads, kSpmmSmem);
+  else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_spmm_walk_queue<false>, kWalkThreads, 0);
   p->grid = std::max(1, per_sm) * sm_count();
   if (use_graph) {
     // the graph holds the queue reset and the persistent launch; replaying it
@@ -547,8 +749,7 @@ extern "C" int cmrs_spmm_plan_create(int batch, const cmrs_matrix *const *A, con
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-      cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int) * p->sh.shares, cap);
-      k_spmm_queue<<<p->grid, kSpmmThreads, kSpmmSmem, cap>>>(p->d_desc, p->d_units, p->sh, p->d_q);
+      enqueue_plan(p, cap);
       e = cudaStreamEndCapture(cap, &p->graph);
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&p->exec, p->graph, 0);
@@ -571,8 +772,7 @@ extern "C" int cmrs_spmm_batched(cmrs_spmm_plan *p, void *stream) {
   if (p->exec) {
     CMRS_CUDA_TRY(cudaGraphLaunch(p->exec, st));
   } else {
-    CMRS_CUDA_TRY(cudaMemsetAsync(p->d_q, 0, sizeof(unsigned int) * p->sh.shares, st));
-    k_spmm_queue<<<p->grid, kSpmmThreads, kSpmmSmem, st>>>(p->d_desc, p->d_units, p->sh, p->d_q);
+    CMRS_CUDA_TRY(enqueue_plan(p, st));
     CMRS_LAUNCH_CHECK();
   }
   return CMRS_OK;
