@@ -10,6 +10,8 @@ namespace {
 
 constexpr int kSortWarpCap = 1024;   // in-strip sort: strips up to this length (or less, see the launch) a warp each
 constexpr int kSortBlockCap = 6144;  // up to this length a CTA each, longer ones by the radix sort
+constexpr int kSortKeyedMin = 256, kSortKeyedCap = 1024;  // rows out of order: see k_sort_keyed
+static_assert(kSortWarpCap <= kSortKeyedCap, "a strip that a warp lists has to fit k_sort_keyed's buffer");
 constexpr int kSortWarps = 4;        // warps per CTA, a strip each
 constexpr int kSortThreads = 256;    // threads sharing a strip of the CTA kernel
 constexpr int kSortBatch = 4;        // independent loads each lane issues before using them
@@ -19,8 +21,8 @@ constexpr int kRadixWarps = kRadixThreads / 32;
 struct StatusBlock {
   uint32_t status;
   int32_t max_strip;
-  int32_t nblock, nradix;  // strips left to the CTA sort, to the radix sort
-  uint32_t pad[60];
+  int32_t nblock, nradix, nkeyed;  // strips left to the CTA sort, to the radix sort, to the keyed sort
+  uint32_t pad[59];
 };
 
 // ---------------------------------------------------------------- value forms
@@ -208,7 +210,11 @@ __global__ void k_pack(int rows, int cols, int nnz, int height, int strips, int 
 // 226 us, packing included, against 1,083 + 75).  Bound by instructions (178M, two
 // thirds of them the merges) and shared-memory reads.
 //   Otherwise the threads sort unique 64-bit keys (column << 32 | position in
-// strip), which makes the order stable, with a bitonic network.
+// strip), which makes the order stable, with a bitonic network: strips of up to
+// kSortKeyedMin entries where they are, longer ones up to kSortKeyedCap listed
+// for k_sort_keyed, whose warps need half the buffer, and the rest by radix.
+// (Rows shuffled, FP64: strips of 640, 1,280 and 4,800 entries took 821, 1,057
+// and 1,391 us by the network in the merge's buffers, 567, 627, 523 before.)
 template <int G>
 __device__ __forceinline__ void group_sync() {
   if constexpr (G == 32) __syncwarp();
@@ -328,16 +334,18 @@ __device__ __forceinline__ void sort_keys(const E *words, unsigned long long *ke
   }
 }
 
-// One strip of at most cap entries by G threads; buf: 16 (cap + 1) bytes, rs:
-// 33 words of shared memory.  Returns whether a column was out of range (this
-// thread's view).
+// One strip of at most cap entries by G threads; buf: 16 (cap + 1) bytes (kKeyed:
+// 8 for each of the power of two at or above cap), rs: 33 words of shared memory.
+// `bad`: a column was out of range (this thread's view).  Returns whether the
+// strip was left alone, its rows out of order and more than `most` entries.
 //   A warp merges the packed words alone: an entry's position in the strip is
 // then its row's start plus its place among the row's entries, in sorted order
 // as in CRS order, and its value waits in the other half of the buffer
 // (copied there while the words are packed and merged).  A CTA merges (word,
-// position) pairs and gathers the values from global memory.
-template <typename In, int DT, int G>
-__device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bits, int cap,
+// position) pairs and gathers the values from global memory.  kKeyed: no merge,
+// the keys at once.
+template <typename In, int DT, int G, bool kKeyed = false>
+__device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bits, int cap, int most, bool &bad,
                                            const int32_t *__restrict__ col_ind, const In *__restrict__ val_in,
                                            char *buf, int *rs, uint32_t *__restrict__ packed,
                                            typename Encode<DT>::Out *__restrict__ vhi,
@@ -347,14 +355,14 @@ __device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bit
   const int lane = threadIdx.x & 31;
   const int tid = G == 32 ? lane : (int)threadIdx.x;
   const int a = R.a, len = R.len, nrow = R.nrow;
-  bool bad = false, unordered = false;
+  bool unordered = false;
   int32_t carry = 0;
   E *src = reinterpret_cast<E *>(buf), *dst = src + cap + 1;
   In *vals = reinterpret_cast<In *>(buf + 8 * ((size_t)cap + 1));  // the warp's values, behind both word buffers
   // row starts, relative to the strip
   if (tid < nrow) rs[tid] = R.start - a;
   if (tid == 0) rs[nrow] = len;
-  if constexpr (G == 32) {
+  if constexpr (G == 32 && !kKeyed) {
     for (int i = lane; i < len; i += 32)
       asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(vals + i)), "l"(val_in + a + i),
                    "n"(sizeof(In))
@@ -404,14 +412,19 @@ __device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bit
       }
     }
   }
-  const bool keyed = group_any<G>(unordered);
+  const bool keyed = kKeyed || group_any<G>(unordered);
   group_sync<G>();
+  if (keyed && len > most) {
+    if constexpr (G == 32) asm volatile("cp.async.wait_all;" ::: "memory");
+    group_sync<G>();  // the buffer is reused by the next strip
+    return true;
+  }
   unsigned long long *keys = reinterpret_cast<unsigned long long *>(buf);
   if (keyed) {
     if constexpr (G == 32) asm volatile("cp.async.wait_all;" ::: "memory");  // the keys take the whole buffer
     group_sync<G>();
     sort_keys<G>(src, keys, len, bits);
-  } else {
+  } else if constexpr (!kKeyed) {
     src = merge_rows<G>(src, dst, rs, nrow);
   }
   const uint32_t mask = (1u << bits) - 1;
@@ -459,7 +472,7 @@ __device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bit
     }
   }
   group_sync<G>();  // the buffer is reused by the next strip
-  return bad;
+  return false;
 }
 
 // Most strips of more than cap entries (cap >= 256) that do not overlap: with
@@ -467,8 +480,10 @@ __device__ __forceinline__ bool sort_strip(const StripRows &R, int cols, int bit
 __host__ __device__ __forceinline__ int list_room(int nnz, int cap) { return nnz / (cap + 1); }
 
 // Validation, StripPtr and the longest strip as in k_pack; strips of up to cap
-// entries sorted here, longer ones listed for the two kernels below: CTA strips
-// from the front of the list, radix strips from its end.  A strip is found
+// entries sorted here (past kSortKeyedMin and out of order: listed for
+// k_sort_keyed), longer ones listed for the kernels below: CTA strips from the
+// front of the list, radix strips from its end, which the CTA sort adds its
+// strips out of order to.  A strip is found
 // valid by its own rows alone, so a RowPtr that falls back between strips makes
 // many of them valid over the same entries; each list therefore ends after
 // `room` strips, as many as can be longer than cap without overlapping, and a
@@ -482,7 +497,8 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int col
                                                                uint32_t *__restrict__ packed,
                                                                typename Encode<DT>::Out *__restrict__ vhi,
                                                                typename Encode<DT>::Out *__restrict__ vlo,
-                                                               int32_t *__restrict__ list, StatusBlock *st) {
+                                                               int32_t *__restrict__ list,
+                                                               int32_t *__restrict__ keyed_list, StatusBlock *st) {
   extern __shared__ __align__(16) char smem[];
   __shared__ int rs_all[kSortWarps][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -512,8 +528,15 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int col
         else bad |= ST_BAD_ROWPTR;
       }
     } else if (R.len > 0) {
-      if (sort_strip<In, DT, 32>(R, cols, bits, cap, col_ind, val_in, buf, rs_all[w], packed, vhi, vlo))
-        bad |= ST_BAD_COL;
+      bool bad_col = false;
+      if (sort_strip<In, DT, 32>(R, cols, bits, cap, kSortKeyedMin, bad_col, col_ind, val_in, buf, rs_all[w], packed,
+                                 vhi, vlo) &&
+          lane == 0) {
+        const int i = atomicAdd(&st->nkeyed, 1);
+        if (i < list_room(nnz, kSortKeyedMin)) keyed_list[i] = s;
+        else bad |= ST_BAD_ROWPTR;
+      }
+      if (bad_col) bad |= ST_BAD_COL;
     }
   }
   bad = __reduce_or_sync(0xffffffffu, bad);
@@ -534,7 +557,7 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols,
                                                              uint32_t *__restrict__ packed,
                                                              typename Encode<DT>::Out *__restrict__ vhi,
                                                              typename Encode<DT>::Out *__restrict__ vlo,
-                                                             const int32_t *__restrict__ list, StatusBlock *st) {
+                                                             int32_t *list, int room, StatusBlock *st) {
   extern __shared__ __align__(16) char smem[];
   __shared__ int rs[33];
   if (st->status & ST_BAD_ROWPTR) return;
@@ -542,10 +565,44 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols,
   bool bad = false;
   for (int i = blockIdx.x; i < n; i += gridDim.x) {
     StripRows R;
-    strip_rows(list[i], rows, nnz, height, row_ptr, R);  // found valid when it was listed
-    bad |= sort_strip<In, DT, kSortThreads>(R, cols, bits, kSortBlockCap, col_ind, val_in, smem, rs, packed, vhi, vlo);
+    const int s = list[i];
+    strip_rows(s, rows, nnz, height, row_ptr, R);  // found valid when it was listed
+    if (sort_strip<In, DT, kSortThreads>(R, cols, bits, kSortBlockCap, kSortKeyedCap, bad, col_ind, val_in, smem, rs,
+                                         packed, vhi, vlo) &&
+        threadIdx.x == 0) {
+      const int k = atomicAdd(&st->nradix, 1);
+      if (k < room) list[nnz - 1 - k] = s;  // always: the two lists' strips do not overlap
+    }
   }
   if (bad) atomicOr(&st->status, ST_BAD_COL);
+}
+
+// Listed strips of kSortKeyedMin to kSortKeyedCap entries with rows out of
+// order, a warp each, by keys alone: 8 bytes an entry of shared memory and none
+// set aside for the longest strip's merge, 24 warps an SM where k_sort_warp's
+// buffers of 1,024 entries leave 12.  FP64, strips of 320 and 640 entries, rows
+// shuffled: 573 and 534 us for the whole conversion (582 and 821 in k_sort_warp).
+// Shorter strips gain nothing from a second reading.
+template <typename In, int DT>
+__global__ void __launch_bounds__(kSortWarps * 32) k_sort_keyed(int rows, int cols, int nnz, int height, int bits,
+                                                                const int32_t *__restrict__ row_ptr,
+                                                                const int32_t *__restrict__ col_ind,
+                                                                const In *__restrict__ val_in,
+                                                                uint32_t *__restrict__ packed,
+                                                                typename Encode<DT>::Out *__restrict__ vhi,
+                                                                typename Encode<DT>::Out *__restrict__ vlo,
+                                                                const int32_t *__restrict__ list, const StatusBlock *st) {
+  __shared__ __align__(16) char bufs[kSortWarps][8 * kSortKeyedCap];
+  __shared__ int rs_all[kSortWarps][33];
+  if (st->status & ST_BAD_ROWPTR) return;
+  const int w = threadIdx.x >> 5, n = st->nkeyed, nw = gridDim.x * kSortWarps;
+  bool bad = false;  // columns were checked when the strip was listed
+  for (int i = blockIdx.x * kSortWarps + w; i < n; i += nw) {
+    StripRows R;
+    strip_rows(list[i], rows, nnz, height, row_ptr, R);
+    sort_strip<In, DT, 32, true>(R, cols, bits, kSortKeyedCap, kSortKeyedCap, bad, col_ind, val_in, bufs[w], rs_all[w],
+                                 packed, vhi, vlo);
+  }
 }
 
 // The longest strips: one CTA per listed strip, stable
@@ -883,6 +940,7 @@ int from_csr_impl(int rows, int cols, int nnz, int height, int bits, uint32_t fl
     CMRS_LAUNCH_CHECK();
   } else {
     int32_t *list = reinterpret_cast<int32_t *>(ws + L.list);
+    int32_t *keyed = reinterpret_cast<int32_t *>(ws + L.keyB);  // read before the radix sort writes there
     // a warp's buffers: 1.5x an average strip and some, so that few strips go
     // to the CTA kernel and short ones leave shared memory for more warps
     const int64_t avg = strips > 0 ? nnz / strips : 0;
@@ -894,16 +952,21 @@ int from_csr_impl(int rows, int cols, int nnz, int height, int bits, uint32_t fl
     CMRS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sort_warp<In, DT>, kSortWarps * 32, smem));
     int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(strips, kSortWarps), (int64_t)sms * std::max(1, per_sm)));
     k_sort_warp<In, DT><<<g, kSortWarps * 32, smem, st>>>(rows, cols, nnz, height, strips, bits, cap, row_ptr, col_ind,
-                                                          val_in, strip_ptr, packed, vh, vl, list, sb);
+                                                          val_in, strip_ptr, packed, vh, vl, list, keyed, sb);
     CMRS_LAUNCH_CHECK();
     if (strips > 0 && nnz > cap) {  // a strip can be longer than that
       const int smem_b = 16 * (kSortBlockCap + 1);
       CMRS_CUDA_TRY(cudaFuncSetAttribute(k_sort_block<In, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_b));
       k_sort_block<In, DT><<<(int)std::min<int64_t>(strips, (int64_t)sms * 2), kSortThreads, smem_b, st>>>(
-          rows, cols, nnz, height, bits, row_ptr, col_ind, val_in, packed, vh, vl, list, sb);
+          rows, cols, nnz, height, bits, row_ptr, col_ind, val_in, packed, vh, vl, list, list_room(nnz, cap), sb);
       CMRS_LAUNCH_CHECK();
     }
-    if (strips > 0 && nnz > kSortBlockCap) {
+    if (strips > 0 && nnz > kSortKeyedMin && cap > kSortKeyedMin) {
+      k_sort_keyed<In, DT><<<(int)std::min<int64_t>(ceil_div(strips, kSortWarps), (int64_t)sms * 6), kSortWarps * 32, 0, st>>>(
+          rows, cols, nnz, height, bits, row_ptr, col_ind, val_in, packed, vh, vl, keyed, sb);
+      CMRS_LAUNCH_CHECK();
+    }
+    if (strips > 0 && nnz > kSortKeyedCap) {
       int col_bits = 1;
       while (col_bits < 31 && ((int64_t)1 << col_bits) < (int64_t)cols) ++col_bits;
       k_sort_radix<In, DT><<<(int)std::min<int64_t>(strips, (int64_t)sms * 4), kRadixThreads, 0, st>>>(

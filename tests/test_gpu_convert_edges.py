@@ -137,3 +137,16 @@ def test_sorted_invalid_input_is_refused(b, what):
         b.cmrs_from_csr(torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), torch.from_numpy(a.val).cuda(), 900, 8,
                         flags=b.CMRS_SORTED)
     assert e.value.code == 4
+
+
+@pytest.mark.parametrize("length", [257, 1024, 1025, 6144, 6145])
+def test_sorted_out_of_order_strips_fill_the_lists(b, length):
+    # equal strips, every one out of order: as many listed strips as nnz has room for
+    h, n = 4, 24
+    kr = np.tile([length - 3 * (length // 4)] + 3 * [length // 4], n)
+    a = csr(kr, 9000, 7, "shuffled")
+    rp, ci = dev(a)
+    M = b.cmrs_from_csr(rp, ci, torch.from_numpy(a.val).cuda(), a.cols, h, flags=b.CMRS_SORTED)
+    ref = orc.csr_to_cmrs(a.row_ptr, a.col_ind, a.val, a.cols, h, sorted_=True)
+    assert np.array_equal(M.col_packed.cpu().numpy()[:a.nnz].view(np.uint32), ref["packed"])
+    assert np.array_equal(b.stored_values(M).cpu().numpy(), ref["val"])
