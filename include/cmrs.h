@@ -91,13 +91,15 @@ extern "C" {
  *                       stride through the strip and accumulate per-row
  *                       partial sums in a shared-memory buffer buf[row][lane],
  *                       then a lane reduction.  Works on sorted strips.
- *                       Sorted strips of short rows, in matrices of enough
- *                       of them, are summed by the row instead: a warp stages
- *                       the strips of 32 or 16 rows, finds each row's entries
+ *                       Sorted strips of short rows (a mean of at most 28,
+ *                       the longest strip, max_strip_nnz, near the mean one),
+ *                       in matrices of enough of them for the device's SMs,
+ *                       are summed by the row instead: a warp stages the
+ *                       strips of 32 or 16 rows, finds each row's entries
  *                       among them with integer work, and one or two lanes
- *                       per row sum them in column order in registers (needs
- *                       col_packed and val 16-byte aligned; Algorithm 1 runs
- *                       otherwise).
+ *                       per row sum them in column order in registers, four
+ *                       sums each (needs col_packed and val 16-byte aligned).
+ *                       Algorithm 1 runs otherwise.
  *   CMRS_VARIANT_MERGE  equal-work tiles of nonzeros: each thread owns a run
  *                       of consecutive entries, rows that cross thread or
  *                       tile boundaries are joined afterwards in a fixed
@@ -169,8 +171,9 @@ int64_t cmrs_val_bytes(int64_t nnz, int dtype);
  * nnz; packed[k] = (col << bits) | (row(k) mod height); the values converted
  * to `dtype`; with CMRS_SORTED each strip is stably sorted by column.
  * Outputs (device): strip_ptr_out[strips+1], col_packed_out[nnz],
- * val_out (cmrs_val_bytes(nnz, dtype) bytes).  If `out` is not NULL it is
- * filled with a view of the outputs (host struct).
+ * val_out (cmrs_val_bytes(nnz, dtype) bytes); they must not overlap the inputs
+ * or the workspace.  If `out` is not NULL it is filled with a view of the
+ * outputs (host struct).
  * Validation: height 1..32 (CMRS_ERR_HEIGHT), cols <= 2^(32-bits)
  * (CMRS_ERR_COL_OVERFLOW) on the host; RowPtr monotone with RowPtr[0] = 0 and
  * RowPtr[rows] = nnz and 0 <= col < cols on the device (CMRS_ERR_CSR_INVALID).
@@ -273,9 +276,12 @@ int cmrs_permute_csr(int rows, int nnz, const int32_t *row_ptr, const int32_t *c
  * includes room for per-part row sums: each strip is then split over several
  * warps and a second kernel adds each row's parts in order; with a workspace
  * of only 256 bytes the one-warp-per-strip walk runs instead.  The result
- * depends only on A, x, the variant and (padded matrices) whether the
- * workspace holds the part sums and the device's SM count: fixed summation
- * order, no atomics on values, so repeated calls give bit-identical y. */
+ * depends only on A (max_strip_nnz included: MERGE, STRIP on sorted strips), x,
+ * the variant, the device's SM count (MERGE, STRIP on sorted strips, padded
+ * matrices), whether col_packed and val are 16-byte aligned (STRIP on sorted
+ * strips) and whether the workspace holds the part sums (padded matrices):
+ * fixed summation order, no atomics on values, so repeated calls give
+ * bit-identical y. */
 int cmrs_spmv_workspace(const cmrs_matrix *A, int variant, size_t *bytes);
 
 /* The kernel variant cmrs_spmv runs for `variant` (resolves
@@ -386,8 +392,13 @@ int cmrs_spmm(const cmrs_matrix *A, int k, const float *X, float *Y, void *strea
 
 /* Batched form: many uneven matrices in one persistent launch.  A plan holds
  * the schedule -- work units (matrix, row range) of about `work_target`
- * entry-columns each, heaviest first, fetched by warps from a device queue --
+ * entry-columns each, heaviest first, fetched by warps from device queues --
  * and, with use_graph != 0, a CUDA graph of {queue reset, persistent kernel}.
+ * A batch whose products gain from staging their entries has one queue per SM,
+ * the units dealt to them in blocks of up to 64 neighbours (of wide products
+ * one by one), a warp taking from the others' once its own is empty; any other
+ * batch has one queue.  Either way each product gets the bits that cmrs_spmm
+ * gives it.
  * A[b] (host array of pointers to host structs), k[b], X[b], Y[b] (host
  * arrays of device pointers) for b < batch.  The plan's device part lives in
  * `workspace` (>= cmrs_spmm_plan_workspace() bytes, 256-byte aligned), which

@@ -164,10 +164,13 @@ __device__ __forceinline__ T item(const T *p) {
 // passes take this form.  k_pad_fill on 2,097,152 such rows (67M FP32
 // entries): 1,149 us when every pass ran the general form, 316 us with each
 // pass read as it was planned, 290 us so; reading and writing the items
-// once is 163 us.  What is left is the votes' latency at 20 warps per SM (the
-// stage's shared memory).  Forms with small stages are bound by registers
-// instead: 48 (10 CTAs per SM) against the compiler's 56 leave rows of
-// power-law lengths 10% faster, 40 spill and are 4-17% slower.
+// once is 163 us.  What is left: fixed latencies (votes, their use; a quarter
+// as many waits for shared memory) at 20 warps per SM (the stage's shared
+// memory), issue 62% of an SM's active cycles, and SMs that have run out of
+// strips while others work (524,288 such rows, 5.4 strips a warp: active 81% of
+// the elapsed cycles, issue 50%).  Forms with small stages are bound by
+// registers instead: 48 (10 CTAs per SM) against the compiler's 56 leave rows
+// of power-law lengths 10% faster, 40 spill and are 4-17% slower.
 template <typename S, bool kSplit, int kM, bool kStaged>
 __device__ __forceinline__ void pad_strip_fill(int left, int next, int height, long long limit, uint32_t *map,
                                                const uint32_t *__restrict__ cp, const S *__restrict__ vh,
@@ -390,12 +393,9 @@ __device__ __forceinline__ void prefetch_l2(const T *a, const T *b) {
 // give up, the warp reads this and its later strips from global memory, so
 // the result does not depend on it, and waits (bounded) once more before it
 // leaves.
-#ifndef CMRS_FILL_WARPS
-#define CMRS_FILL_WARPS 4
-#endif
-constexpr int kFillWarps = CMRS_FILL_WARPS;
-constexpr int kFillCap = 2048;  // most items per stage
-constexpr int kFillAhead = 2048;  // most items of a longer strip asked for in L2 (24 KB a warp in FP64; 6,080 warps at most)
+constexpr int kFillWarps = 4;
+constexpr int kFillCap = 2048;    // most items per stage
+constexpr int kFillAhead = 2048;  // most items of a longer strip asked for in L2
 template <int DT, int kM>
 __global__ void __launch_bounds__(kFillWarps * 32, kM == 1 ? 8 : 10) k_pad_fill(int strips, int height, int bits, int cap, int nnz,
                                                              const int32_t *__restrict__ sp,
@@ -430,9 +430,10 @@ __global__ void __launch_bounds__(kFillWarps * 32, kM == 1 ? 8 : 10) k_pad_fill(
     if (staged && lane == 0) issue_stage<DT>(sa, sb, nnz, packed, vh, vl, stg, cap, &bars[w], pol, &info[w]);
     if (!staged) {
       // read from global memory below, a few passes' loads at a time: from L2,
-      // as much of it as L2 holds for every warp on the chip (power-law rows
-      // of 1M, M = 8 at height 16: 250 -> 129 us with the reads of passes
-      // alike by item<>)
+      // the strip's first kFillAhead items (power-law rows of 1M, M = 8 at
+      // height 16: 250 -> 129 us with the reads of passes alike by item<>).
+      // Should every warp of the largest launch (6,080) ask for that many at
+      // once, FP64's 149 MB would pass the 129 MB of L2, FP32's 100 MB not.
       const int to = sb - sa > kFillAhead ? sa + kFillAhead : sb;
       prefetch_l2(packed + sa, packed + to);
       prefetch_l2(vh + sa, vh + to);

@@ -46,28 +46,13 @@
 namespace cmrs {
 namespace {
 
-#ifndef CMRS_SPMM_CAP
-#define CMRS_SPMM_CAP 704  // entries per warp's stage
-#endif
-#ifndef CMRS_SPMM_MINB
-#define CMRS_SPMM_MINB 7  // resident CTAs per SM asked of the register allocator (72 registers)
-#endif
-#ifndef CMRS_SPMM_D
-#define CMRS_SPMM_D 4  // X gathers in flight per lane
-#endif
-#ifndef CMRS_SPMM_BLOCK
-#define CMRS_SPMM_BLOCK 64  // neighbouring units dealt to one SM together (8: k = 4, 8 products 12% slower)
-#endif
-#ifndef CMRS_SPMM_SPLIT
-#define CMRS_SPMM_SPLIT 2  // most lane groups per row (4 with a stage of 384: no faster, k = 8 slower)
-#endif
-#ifndef CMRS_SPMM_THREADS
-#define CMRS_SPMM_THREADS 128
-#endif
-constexpr int kSpmmThreads = CMRS_SPMM_THREADS;
+constexpr int kSpmmThreads = 128;
 constexpr int kSpmmWarps = kSpmmThreads / 32;
-constexpr int kSpmmCap = CMRS_SPMM_CAP;
-constexpr int kSpmmD = CMRS_SPMM_D;
+constexpr int kSpmmCap = 704;   // entries per warp's stage
+constexpr int kSpmmMinB = 7;    // resident CTAs per SM asked of the register allocator (72 registers)
+constexpr int kSpmmD = 4;       // X gathers in flight per lane
+constexpr int kSpmmBlock = 64;  // neighbouring units dealt to one SM together (8: k = 4, 8 products 12% slower)
+constexpr int kSpmmSplit = 2;   // most lane groups per row (4 with a stage of 384: no faster, k = 8 slower)
 constexpr size_t kSpmmSmem = kSpmmWarps * Stage<CMRS_F32>::bytes(kSpmmCap);
 
 struct Desc {
@@ -282,7 +267,7 @@ __device__ __forceinline__ void warp_stage_end(WarpStage &st) {
   if (!st.ok) mbar_wait_bounded(st.bar, st.phase);
 }
 
-__global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_queue(const Desc *__restrict__ descs,
+__global__ void __launch_bounds__(kSpmmThreads, kSpmmMinB) k_spmm_queue(const Desc *__restrict__ descs,
                                                                             const Unit *__restrict__ units, Shares sh,
                                                                             QueueHead *q) {
   extern __shared__ __align__(128) char smem[];
@@ -324,7 +309,7 @@ __global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_queue(con
 }
 
 // One matrix, no queue: warp w takes rows [w*rpw, (w+1)*rpw).
-__global__ void __launch_bounds__(kSpmmThreads, CMRS_SPMM_MINB) k_spmm_one(Desc d, int rows_per_warp) {
+__global__ void __launch_bounds__(kSpmmThreads, kSpmmMinB) k_spmm_one(Desc d, int rows_per_warp) {
   extern __shared__ __align__(128) char smem[];
   __shared__ uint64_t bars[kSpmmWarps];
   __shared__ StageInfo info[kSpmmWarps];
@@ -555,7 +540,7 @@ Desc make_desc(const cmrs_matrix *A, int k, const float *X, float *Y) {
   // lanes keep fewer.
   const double mu = A->rows > 0 ? (double)A->nnz / A->rows : 0.0;
   d.split = 1;
-  while (d.split < CMRS_SPMM_SPLIT && spmm_lanes(k, d.vec) * d.split < CMRS_SPMM_SPLIT && mu >= 8.0 * d.split) d.split <<= 1;
+  while (d.split < kSpmmSplit && spmm_lanes(k, d.vec) * d.split < kSpmmSplit && mu >= 8.0 * d.split) d.split <<= 1;
   return d;
 }
 
@@ -602,7 +587,7 @@ extern "C" int cmrs_spmm(const cmrs_matrix *A, int k, const float *X, float *Y, 
   // the SMs twice, whole groups of the rows a warp works at once
   const int per = 32 / (spmm_lanes(k, d.vec) * d.split);
   if (!spmm_staged(d)) return launch_walk_one(d, st);
-  const long long resident = (long long)sm_count() * CMRS_SPMM_MINB * kSpmmWarps;
+  const long long resident = (long long)sm_count() * kSpmmMinB * kSpmmWarps;
   const int rpw = (int)std::max<long long>(per, std::min<long long>(32, A->rows / (2 * resident)) / per * per);
   const long long warps = ceil_div(A->rows, rpw);
   const int grid = (int)ceil_div(warps * 32, kSpmmThreads);
@@ -639,13 +624,13 @@ static int build_units(int batch, const cmrs_matrix *const *A, const int32_t *k,
   return CMRS_OK;
 }
 
-// Shares of a plan's units: blocks of up to CMRS_SPMM_BLOCK units, smaller ones
+// Shares of a plan's units: blocks of up to kSpmmBlock units, smaller ones
 // while a share would hold fewer than eight.
 static Shares make_shares(size_t nunits) {
   Shares sh;
   sh.nunits = (int)nunits;
   sh.shares = std::max(1, std::min(sm_count(), kMaxShares));
-  sh.block = std::max(1, std::min(CMRS_SPMM_BLOCK, sh.nunits / (8 * sh.shares)));
+  sh.block = std::max(1, std::min(kSpmmBlock, sh.nunits / (8 * sh.shares)));
   sh.len = (int)ceil_div(ceil_div(sh.nunits, sh.block), sh.shares) * sh.block;
   return sh;
 }

@@ -595,14 +595,14 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // this GPU an FP64 warp instruction costs its issue slot whatever its active
 // lanes do: with rows of 27 entries the reduction and the steps' partly filled
 // multiply-adds are two thirds of the FP64 pipe's time (27-point 128^3, h = 4:
-// 355 us; 227 us here, bound by instructions).  Here a warp takes R = 32 / L rows, or the whole strips below that,
-// stages their entries by one bulk copy, and finds each row's entries there
-// with integer work only; L lanes then walk each row in column order, one
-// multiply-add per entry and lane into one of four sums in registers, joined
-// at the end: chains of at most nine entries, as exact as Algorithm 1's 32
-// partial sums and tree (norm of the FP64 error on rows of 27 entries: 0.95 of
-// Algorithm 1's; one chain a lane, 219 us, 1.15).  x is gathered at the same
-// place of consecutive rows.
+// 355 us; 227 us here, bound by instructions).  Here a warp takes R = 32 / L
+// rows, or the whole strips below that, stages their entries by one bulk copy,
+// and finds each row's entries there with integer work only; L lanes then walk
+// each row in column order, one multiply-add per entry and lane into one of
+// four sums in registers, joined at the end: chains of at most nine entries,
+// as exact as Algorithm 1's 32 partial sums and tree (norm of the FP64 error
+// on rows of 27 entries: 0.95 of Algorithm 1's; one chain a lane, 219 us,
+// 1.15).  x is gathered at the same place of consecutive rows.
 //   An entry's place among its row's entries is found and its index left in
 // list[place][row]; the lanes of a row take every L-th place.  Heights up to 8
 // (kPack): each strip is cut into P parts, a lane each, and every lane counts
@@ -613,25 +613,12 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // heights, place_in_row) takes about 40.
 //   A unit longer than its stage, or with a row longer than the list (or a
 // packed count), runs Algorithm 1 strip by strip.
-#ifndef CMRS_SORTED_WARPS
-#define CMRS_SORTED_WARPS 4
-#endif
-#ifndef CMRS_SORTED_CAP
-#define CMRS_SORTED_CAP 1024  // most entries per warp stage
-#endif
-#ifndef CMRS_SORTED_CH_F64
-#define CMRS_SORTED_CH_F64 7
-#endif
-#ifndef CMRS_SORTED_CTAS
-#define CMRS_SORTED_CTAS 0
-#endif
-#ifndef CMRS_SORTED_MINB
-#define CMRS_SORTED_MINB 6
-#endif
-constexpr int kSortedWarps = CMRS_SORTED_WARPS;
+constexpr int kSortedWarps = 4;
+constexpr int kSortedCap = 1024;  // most entries per warp stage
+constexpr int kSortedMinB = 6;    // CTAs per SM asked of the register allocator (80 registers)
 // kPack: bytes of the packed counts, 4 (heights up to 4), 8 (up to 8), 0 (votes)
 template <int DT, int L, int kPack>
-__global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_sorted(int rows, int height, int bits, int strips, int cap,
+__global__ void __launch_bounds__(kSortedWarps * 32, kSortedMinB) k_spmv_sorted(int rows, int height, int bits, int strips, int cap,
                                                                    int ml, int warp_bytes, int nnz,
                                                                    const int32_t *__restrict__ sp,
                                                                    const uint32_t *__restrict__ packed,
@@ -643,7 +630,10 @@ __global__ void __launch_bounds__(kSortedWarps * 32, CMRS_SORTED_MINB) k_spmv_so
                                                                    uint32_t *status) {
   typedef typename Form<DT>::Stored S;
   typedef typename Form<DT>::Acc A;
-  constexpr int CH = DT == CMRS_F64 ? CMRS_SORTED_CH_F64 : 8;
+  // x gathers in flight per lane; FP64: two batches of 7 for 27 entries over two
+  // lanes, one for a row of 7 (by 8: 27-point h = 4 245 us against 226, 7-point 43
+  // against 37)
+  constexpr int CH = DT == CMRS_F64 ? 7 : 8;
   constexpr int kAcc = 4;
   constexpr int RS = 32 / L + 2;  // the list's row stride: an odd number of words
   extern __shared__ __align__(128) char smem[];
@@ -952,12 +942,13 @@ __global__ void __launch_bounds__(kPadWarps * 32, CMRS_PAD_MINB) k_spmv_padded(i
 // other forms, 11 for these in one or two waves of CTAs, 15 for all where rows
 // average 16 entries or more).  It finds their strip by a binary search of
 // StripPtr between the strips holding the tile's first and next tile's first
-// entry (tile_strip[], one small pre-pass), then walks the entries: a row's run is summed by one FMA chain; a run that starts and
-// ends inside the thread is written at once; a run cut by the thread's end is
-// joined, after a CTA barrier, by the thread where it started (walking over
-// the following threads' head partials in order); a run cut by the tile's end
-// goes to a tile record that a fix-up kernel joins in tile order.  Rows with
-// no entries are written as 0 by the thread owning the entry before the gap.
+// entry (tile_strip[], one small pre-pass), then walks the entries: a row's run
+// is summed by one FMA chain; a run that starts and ends inside the thread is
+// written at once; a run cut by the thread's end is joined, after a CTA
+// barrier, by the thread where it started (walking over the following
+// threads' head partials in order); a run cut by the tile's end goes to a tile
+// record that a fix-up kernel joins in tile order.  Rows with no entries are
+// written as 0 by the thread owning the entry before the gap.
 __global__ void k_tile_map(int strips, const int32_t *__restrict__ sp, int tile, int ntiles,
                            int32_t *__restrict__ tile_strip) {
   pdl_launch_dependents();  // the product may start staging its first tiles
@@ -1790,7 +1781,7 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   // no more than 36 entries a lane (rows of more than 28 a lane are less exact
   // by four sums than by Algorithm 1's 32, so they have to be few); at least
   // Algorithm 1's buffer
-  const int cap = (int)std::min<long long>(CMRS_SORTED_CAP,
+  const int cap = (int)std::min<long long>(kSortedCap,
                                            std::max<long long>(128, ceil_div((long long)(1.25 * mu * ns * A->height), 32) * 32));
   const int ml = std::min((int)(1.5 * mu) + 16, 36 * L);
   const size_t list = ((size_t)ml * (32 / L + 2) * 2 + 127) & ~size_t(127);
@@ -1798,7 +1789,7 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   const size_t smem = kSortedWarps * warp_bytes;
   static Occ occ[256];  // by the warp's bytes, in units of 128: at most 19 KB
   const int per_sm = occupancy(k_spmv_sorted<DT, L, kPack>, kSortedWarps * 32, smem,
-                               occ[std::min<size_t>(warp_bytes / 128, 255)], 128 * 1024, CMRS_SORTED_CTAS);
+                               occ[std::min<size_t>(warp_bytes / 128, 255)], 128 * 1024);
   const long long need = ceil_div(ceil_div(A->strips, ns), kSortedWarps);
   const int grid = (int)std::min<long long>(need, (long long)per_sm * sm_count());
   k_spmv_sorted<DT, L, kPack><<<grid, kSortedWarps * 32, smem, st>>>(A->rows, A->height, A->bits, A->strips, cap, ml,
