@@ -204,17 +204,17 @@ __global__ void k_pack(int rows, int cols, int nnz, int height, int strips, int 
 // RowInStrip, which is CRS order -- and a merge tree over the rows sorts it:
 // log2(height) rounds, each pair of runs shared by G / pairs threads, which
 // split its output evenly (each finds its part by one binary search along the
-// merge path) and merge it serially, without a branch.  A round costs about 15 instructions per
-// entry of a thread's share; the bitonic network below needs log2(n)^2 / 2
-// compare-exchanges per entry (20M entries, strips of 320 at height 16:
-// 226 us, packing included, against 1,083 + 75).  Bound by instructions (178M, two
-// thirds of them the merges) and shared-memory reads.
+// merge path) and merge it serially, without a branch.  A round costs about 15
+// instructions per entry of a thread's share; the bitonic network below needs
+// log2(n)^2 / 2 compare-exchanges per entry (20M entries, strips of 320 at
+// height 16: 226 us, packing included, against 1,083 + 75).  Bound by
+// instructions (178M, two thirds of them the merges) and shared-memory reads.
 //   Otherwise the threads sort unique 64-bit keys (column << 32 | position in
 // strip), which makes the order stable, with a bitonic network: strips of up to
 // kSortKeyedMin entries where they are, longer ones up to kSortKeyedCap listed
 // for k_sort_keyed, whose warps need half the buffer, and the rest by radix.
-// (Rows shuffled, FP64: strips of 640, 1,280 and 4,800 entries took 821, 1,057
-// and 1,391 us by the network in the merge's buffers, 567, 627, 523 before.)
+// (6M FP64 entries, rows shuffled: strips of 640, 1,280 and 4,800 entries 534,
+// 617 and 454 us so, 821, 1,057 and 1,391 by the network in the merge's buffers.)
 template <int G>
 __device__ __forceinline__ void group_sync() {
   if constexpr (G == 32) __syncwarp();
@@ -483,11 +483,10 @@ __host__ __device__ __forceinline__ int list_room(int nnz, int cap) { return nnz
 // entries sorted here (past kSortKeyedMin and out of order: listed for
 // k_sort_keyed), longer ones listed for the kernels below: CTA strips from the
 // front of the list, radix strips from its end, which the CTA sort adds its
-// strips out of order to.  A strip is found
-// valid by its own rows alone, so a RowPtr that falls back between strips makes
-// many of them valid over the same entries; each list therefore ends after
-// `room` strips, as many as can be longer than cap without overlapping, and a
-// ticket past it is an invalid RowPtr.
+// strips out of order to.  A strip is found valid by its own rows alone, so a
+// RowPtr that falls back between strips makes many of them valid over the same
+// entries; each list therefore ends after as many strips as can be that long
+// without overlapping, and a ticket past it is an invalid RowPtr.
 template <typename In, int DT>
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort_warp(int rows, int cols, int nnz, int height, int strips,
                                                                int bits, int cap, const int32_t *__restrict__ row_ptr,
@@ -580,9 +579,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_block(int rows, int cols,
 // Listed strips of kSortKeyedMin to kSortKeyedCap entries with rows out of
 // order, a warp each, by keys alone: 8 bytes an entry of shared memory and none
 // set aside for the longest strip's merge, 24 warps an SM where k_sort_warp's
-// buffers of 1,024 entries leave 12.  FP64, strips of 320 and 640 entries, rows
-// shuffled: 573 and 534 us for the whole conversion (582 and 821 in k_sort_warp).
-// Shorter strips gain nothing from a second reading.
+// buffers of 1,024 entries leave 12.  6M FP64 entries in strips of 640,
+// rows shuffled: 534 us for the whole conversion (821 in k_sort_warp).
 template <typename In, int DT>
 __global__ void __launch_bounds__(kSortWarps * 32) k_sort_keyed(int rows, int cols, int nnz, int height, int bits,
                                                                 const int32_t *__restrict__ row_ptr,
