@@ -12,6 +12,7 @@
 // Nonzero streams are copied into shared memory by the bulk-copy engine
 // (cp.async.bulk, mbarrier completion, L2 evict-first).
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include <type_traits>
@@ -1729,25 +1730,33 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
 // Lanes per row of the SORTED mapping, 0 where Algorithm 1 runs instead:
 // unsorted or padded strips, arrays the bulk copies cannot read, and wherever
 // the mapping was not the faster one.  The lines lie where it stopped winning on
-// rows of equal length, of 0.5 to 1.5x and 0 to 2x the mean, of Poisson and
-// power-law lengths: 20,000 to 1.5M rows, heights 2 to 32, every value form
-// (12,900 points; us below: Algorithm 1 -> the mapping).
+// rows of equal length, of 0.2 to 1.8x and 0 to 2x the mean, of Poisson and
+// power-law lengths: 14,000 to 1.5M rows, heights 2 to 32, every value form,
+// launches queued behind one another (22,000 points; us below: Algorithm 1 ->
+// the mapping).
 //   - Undoing the sort costs every entry, Algorithm 1's reduction costs a strip
 //     31 adds per row whatever the rows' length: short rows and low strips win
-//     most (7-point, 1.5M rows: FP64 408 -> 52, 219 -> 52, 128 -> 74 at h = 2,
-//     4, 16, FP32 205 -> 41, 115 -> 41, 91 -> 60), and past 28 entries a row
-//     little is left (32 at h = 3, FP64 50 -> 41, FP32 29 -> 31).  Heights past
-//     8 undo it by votes, at twice the cost (13 entries at h = 16, FP32: 15 ->
-//     15).  Two lanes a row gain nothing past `most` entries a mean strip (27 at
-//     h = 4, 6: FP64 43 -> 31, 33 -> 29; FP32 25 -> 23, 21 -> 22).
-//   - The lanes of a unit wait for its longest row, and a row past the list
-//     sends the unit to Algorithm 1 after its walks.  The longest strip against
-//     the mean one tells rows alike from others: 27 entries +-50% at h = 4, 6
-//     FP64 43 -> 44, 32 -> 37; power-law rows (the longest strip 32 to 110 times
-//     the mean) FP32 159 -> 207, 143 -> 146 at h = 4, 16.
-//   - A unit's copy, walks and gathers take 4..7 us one after another: few units
-//     pay for it only where they are alike (12 entries +-67%, 90,000 rows FP32
-//     at h = 2: 16.5 -> 20.8; 400,000 rows: 58 -> 33).
+//     most (7-point, 1M rows: FP64 254 -> 38, 139 -> 37, 90 -> 51 at h = 2, 4,
+//     16, FP32 138 -> 29, 80 -> 29, 63 -> 41), and past 28 entries a row little
+//     is left (32 at h = 3, FP64 50 -> 41, FP32 29 -> 31).  Heights past 8 undo
+//     it by votes, at twice the cost (13 entries at h = 16, FP32: 15 -> 15).
+//     Two lanes a row gain nothing past `most` entries a mean strip (27 at h =
+//     4, 6: FP64 43 -> 31, 33 -> 29; FP32 25 -> 23, 21 -> 22).
+//   - A unit's copy, walks and gathers take 4..7 us one after another: `least`
+//     units per SM pay for it (rows of 6, FP32, h = 4: 3 units 4.2 -> 6.2, 9 units
+//     6.3 -> 6.2, 18 units 10.3 -> 6.2).
+//   - The lanes of a unit wait for its longest row.  How far the longest strip
+//     passes the mean one tells how far the longest row does: the excess falls
+//     with sqrt(height), and `wait` is it in entries (Poisson rows of 13, FP64:
+//     h = 4, 25 units 20.5 -> 23.2, 49 units 36.9 -> 36.9; h = 8, where
+//     Algorithm 1 costs less, 32.7 -> 36.4).
+//   - A unit past its stage, or with a row past the list, runs Algorithm 1 after
+//     its walks, one warp while the others are done: rows uneven past 1.4 at
+//     means past 3 have such units, and few units have few warps to hide them
+//     (Poisson rows of 4, FP32, h = 4: 18 units 10.3 -> 12.4, 72 units 30.8 -> 20.5).
+//     Power-law rows have them throughout: only a mean of 2.5 or less and the
+//     higher strips gain (700,000 rows of 1.9, FP32, h = 32: 52 -> 30; rows of
+//     4, h = 4: 159 -> 207).
 template <int DT>
 int sorted_lanes(const cmrs_matrix *A) {
   constexpr bool kF64 = DT == CMRS_F64;
@@ -1755,15 +1764,24 @@ int sorted_lanes(const cmrs_matrix *A) {
   if ((reinterpret_cast<uintptr_t>(A->col_packed) | reinterpret_cast<uintptr_t>(A->val)) & 15) return 0;
   const double mu = (double)A->nnz / A->rows, strip = mu * A->height;
   const int h = A->height, longest = A->max_strip_nnz;
-  if (mu > 28.0 || longest < 0 || longest > 4.0 * strip) return 0;
+  if (mu > 28.0 || longest < 0 || (mu > 2.5 && longest > 4.0 * strip)) return 0;
+  const double uneven = (longest / strip - 1.0) * std::sqrt((double)h), wait = uneven * mu;
   const int L = mu <= 14.0 ? 1 : 2;
-  const int spread = longest <= 1.1 * strip ? 0 : longest <= 1.6 * strip ? 1 : 2;
   int least;  // units per SM
-  if (L == 1) {
-    if (h > 8 && mu > (!kF64 ? 8.0 : spread ? 10.0 : 14.0)) return 0;
-    least = spread == 2 ? 70 : h > 8 || (spread == 1 && mu > 10.0) ? 20 : 8;
+  if (L == 1 && longest > 8.0 * strip) {
+    if (!kF64 && h <= 4) return 0;
+    least = h > 8 ? 14 : kF64 && h > 4 ? 24 : 100;
+  } else if (L == 1) {
+    if (h > 8 && mu > (kF64 ? 14.0 : 10.0)) return 0;
+    if (kF64 && h > 4 && h <= 8 && mu > 12.5 && wait > 13.0) return 0;
+    if (mu > 10.0 && uneven > 1.6) least = 70;
+    else if (h <= 8 && mu > 3.0 && uneven > 1.4) least = kF64 ? 18 : h > 4 ? 24 : 28;
+    else if (wait > 13.0) least = h <= 4 ? 36 : kF64 ? 16 : h > 8 ? 48 : 24;
+    else if (wait > 9.0) least = h > 4 ? 14 : 20;
+    else least = !kF64 && h > 4 && mu > 7.0 ? 14 : 8;
   } else {
-    const double most[3] = {kF64 ? 224.0 : 112.0, kF64 ? 84.0 : 64.0, kF64 ? 66.0 : 44.0};
+    const int spread = uneven <= 0.45 ? 0 : longest <= 1.6 * strip ? 1 : 2;
+    const double most[3] = {kF64 ? 224.0 : 112.0, kF64 ? 84.0 : 64.0, kF64 ? 66.0 : 56.0};
     if (h > (kF64 && spread == 0 ? 8 : 4) || strip > most[spread]) return 0;
     least = kF64 && spread < 2 ? 40 : 100;
   }

@@ -106,3 +106,15 @@ ALGORITHM_1 = [(27, 0.5, 4, 110, None), (20, 0.5, 6, 110, None), (27, 0.5, 8, 11
 def test_algorithm_1_where_it_is_faster(b, dtype, mean, spread, height, units, longest):
     y, alg1, _ = products(b, dtype, mean, spread, height, units, longest)
     assert torch.equal(y, alg1)
+
+
+# units per SM on either side of where the mapping starts to pay: rows alike, uneven ones that the lanes wait for
+@pytest.mark.parametrize("dtype", [0, 1, 2, 3])
+@pytest.mark.parametrize("mean,spread,height,few,enough", [(7, 0.0, 4, 7, 9), (7, 0.0, 16, 7, 9), (6, 0.67, 4, 7, 22),
+                                                           (12, 0.67, 4, 17, 40)])
+def test_units_that_pay_for_the_mapping(b, dtype, mean, spread, height, few, enough):
+    y, alg1, _ = products(b, dtype, mean, spread, height, few)
+    assert torch.equal(y, alg1)
+    y, alg1, exact = products(b, dtype, mean, spread, height, enough)
+    assert not torch.equal(y, alg1)
+    assert error(y, exact) <= 1.03 * error(alg1, exact)  # as above, from fewer rows
