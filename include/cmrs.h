@@ -97,8 +97,8 @@ extern "C" {
  *                       are summed by the row instead: a warp stages the
  *                       strips of 32 or 16 rows, finds each row's entries
  *                       among them with integer work, and one or two lanes
- *                       per row sum them in column order in registers, four
- *                       sums each (needs col_packed and val 16-byte aligned).
+ *                       per row sum them in column order in registers, two
+ *                       or four sums each (needs col_packed and val 16-byte aligned).
  *                       Algorithm 1 runs otherwise.
  *   CMRS_VARIANT_MERGE  equal-work tiles of nonzeros: each thread owns a run
  *                       of consecutive entries, rows that cross thread or

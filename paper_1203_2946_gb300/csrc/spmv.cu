@@ -600,10 +600,13 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // rows, or the whole strips below that, stages their entries by one bulk copy,
 // and finds each row's entries there with integer work only; L lanes then walk
 // each row in column order, one multiply-add per entry and lane into one of
-// four sums in registers, joined at the end: chains of at most nine entries,
-// as exact as Algorithm 1's 32 partial sums and tree (norm of the FP64 error
-// on rows of 27 entries: 0.95 of Algorithm 1's; one chain a lane, 219 us,
-// 1.15).  x is gathered at the same place of consecutive rows.
+// kAcc sums in registers, joined at the end.  Four: chains of at most nine
+// entries, as exact as Algorithm 1's 32 partial sums and tree (norm of the
+// FP64 error on rows of 27 entries: 0.95 of Algorithm 1's; one chain a lane,
+// 219 us, 1.15).  FP64 rows averaging kSortedTwoMu or fewer take two: 0.88 to
+// 0.99 of it, rows of 0 to twice the mean included (means of 12 and 14: 1.02
+// and 1.06), at fewer instructions (300,000 7-point rows, h = 4: 14.4 us, 16.0
+// with four).  x is gathered at the same place of consecutive rows.
 //   An entry's place among its row's entries is found and its index left in
 // list[place][row]; the lanes of a row take every L-th place.  Heights up to 8
 // (kPack): each strip is cut into P parts, a lane each, and every lane counts
@@ -616,9 +619,10 @@ __global__ void __launch_bounds__(kStripWarps * 32) k_spmv_strip(int rows, int h
 // packed count), runs Algorithm 1 strip by strip.
 constexpr int kSortedWarps = 4;
 constexpr int kSortedCap = 1024;  // most entries per warp stage
+constexpr double kSortedTwoMu = 10.0;  // FP64: two sums a lane up to this mean
 constexpr int kSortedMinB = 6;    // CTAs per SM asked of the register allocator (80 registers)
 // kPack: bytes of the packed counts, 4 (heights up to 4), 8 (up to 8), 0 (votes)
-template <int DT, int L, int kPack>
+template <int DT, int L, int kPack, int kAcc>
 __global__ void __launch_bounds__(kSortedWarps * 32, kSortedMinB) k_spmv_sorted(int rows, int height, int bits, int strips, int cap,
                                                                    int ml, int warp_bytes, int nnz,
                                                                    const int32_t *__restrict__ sp,
@@ -635,7 +639,6 @@ __global__ void __launch_bounds__(kSortedWarps * 32, kSortedMinB) k_spmv_sorted(
   // lanes, one for a row of 7 (by 8: 27-point h = 4 245 us against 226, 7-point 43
   // against 37)
   constexpr int CH = DT == CMRS_F64 ? 7 : 8;
-  constexpr int kAcc = 4;
   constexpr int RS = 32 / L + 2;  // the list's row stride: an odd number of words
   extern __shared__ __align__(128) char smem[];
   __shared__ uint64_t bars[kSortedWarps];
@@ -773,7 +776,8 @@ __global__ void __launch_bounds__(kSortedWarps * 32, kSortedMinB) k_spmv_sorted(
           for (int k = 1; k < kAcc; ++k) acc[k - 1] = acc[k];
           acc[kAcc - 1] = t;
         }
-        acc[0] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+        acc[0] += acc[1];
+        if constexpr (kAcc == 4) acc[0] += acc[2] + acc[3];
 #pragma unroll
         for (int o = L / 2; o >= 1; o >>= 1) acc[0] += __shfl_down_sync(kAll, acc[0], o);
         if (active && q == 0) {
@@ -1736,8 +1740,8 @@ int launch_merge(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, cons
 // the mapping).
 //   - Undoing the sort costs every entry, Algorithm 1's reduction costs a strip
 //     31 adds per row whatever the rows' length: short rows and low strips win
-//     most (7-point, 1M rows: FP64 254 -> 38, 139 -> 37, 90 -> 51 at h = 2, 4,
-//     16, FP32 138 -> 29, 80 -> 29, 63 -> 41), and past 28 entries a row little
+//     most (7-point at h = 2, 4, 16: 300,000 rows FP64 66 -> 14, 39 -> 14, 33 ->
+//     18; 1M rows FP32 138 -> 29, 80 -> 29, 63 -> 41), past 28 entries a row little
 //     is left (32 at h = 3, FP64 50 -> 41, FP32 29 -> 31).  Heights past 8 undo
 //     it by votes, at twice the cost (13 entries at h = 16, FP32: 15 -> 15).
 //     Two lanes a row gain nothing past `most` entries a mean strip (27 at h =
@@ -1788,7 +1792,7 @@ int sorted_lanes(const cmrs_matrix *A) {
   return ceil_div(A->strips, 32 / L / h) >= (long long)least * sm_count() ? L : 0;
 }
 
-template <int DT, int L, int kPack>
+template <int DT, int L, int kPack, int kAcc>
 int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, const typename Form<DT>::Stored *lo,
                   const typename Form<DT>::Acc *x, typename Form<DT>::Acc *y, const int32_t *row_map, uint32_t *status,
                   cudaStream_t st) {
@@ -1806,11 +1810,11 @@ int launch_sorted(const cmrs_matrix *A, const typename Form<DT>::Stored *hi, con
   const size_t warp_bytes = std::max(Stage<DT>::bytes(cap) + list, (size_t)A->height * 32 * sizeof(Acc));
   const size_t smem = kSortedWarps * warp_bytes;
   static Occ occ[256];  // by the warp's bytes, in units of 128: at most 19 KB
-  const int per_sm = occupancy(k_spmv_sorted<DT, L, kPack>, kSortedWarps * 32, smem,
+  const int per_sm = occupancy(k_spmv_sorted<DT, L, kPack, kAcc>, kSortedWarps * 32, smem,
                                occ[std::min<size_t>(warp_bytes / 128, 255)], 128 * 1024);
   const long long need = ceil_div(ceil_div(A->strips, ns), kSortedWarps);
   const int grid = (int)std::min<long long>(need, (long long)per_sm * sm_count());
-  k_spmv_sorted<DT, L, kPack><<<grid, kSortedWarps * 32, smem, st>>>(A->rows, A->height, A->bits, A->strips, cap, ml,
+  k_spmv_sorted<DT, L, kPack, kAcc><<<grid, kSortedWarps * 32, smem, st>>>(A->rows, A->height, A->bits, A->strips, cap, ml,
                                                               (int)warp_bytes, A->nnz, A->strip_ptr, A->col_packed, hi,
                                                               lo, x, y, row_map, status);
   CMRS_LAUNCH_CHECK();
@@ -1870,14 +1874,20 @@ int launch(const cmrs_matrix *A, const void *xv, void *yv, const int32_t *row_ma
   } else if (variant == CMRS_VARIANT_STRIP && sorted_lanes<DT>(A)) {
     const int lanes_s = sorted_lanes<DT>(A);
     const int h = A->height;
-    if (lanes_s == 1)
-      return h <= 4   ? launch_sorted<DT, 1, 4>(A, hi, lo, x, y, row_map, status, st)
-             : h <= 8 ? launch_sorted<DT, 1, 8>(A, hi, lo, x, y, row_map, status, st)
-                      : launch_sorted<DT, 1, 0>(A, hi, lo, x, y, row_map, status, st);
-    if constexpr (DT == CMRS_F64) {  // the other forms: heights up to 4
-      if (h > 4) return launch_sorted<DT, 2, 8>(A, hi, lo, x, y, row_map, status, st);
+    if constexpr (DT == CMRS_F64) {
+      if ((double)A->nnz <= kSortedTwoMu * A->rows)
+        return h <= 4   ? launch_sorted<DT, 1, 4, 2>(A, hi, lo, x, y, row_map, status, st)
+               : h <= 8 ? launch_sorted<DT, 1, 8, 2>(A, hi, lo, x, y, row_map, status, st)
+                        : launch_sorted<DT, 1, 0, 2>(A, hi, lo, x, y, row_map, status, st);
     }
-    return launch_sorted<DT, 2, 4>(A, hi, lo, x, y, row_map, status, st);
+    if (lanes_s == 1)
+      return h <= 4   ? launch_sorted<DT, 1, 4, 4>(A, hi, lo, x, y, row_map, status, st)
+             : h <= 8 ? launch_sorted<DT, 1, 8, 4>(A, hi, lo, x, y, row_map, status, st)
+                      : launch_sorted<DT, 1, 0, 4>(A, hi, lo, x, y, row_map, status, st);
+    if constexpr (DT == CMRS_F64) {  // the other forms: heights up to 4
+      if (h > 4) return launch_sorted<DT, 2, 8, 4>(A, hi, lo, x, y, row_map, status, st);
+    }
+    return launch_sorted<DT, 2, 4, 4>(A, hi, lo, x, y, row_map, status, st);
   } else if (variant == CMRS_VARIANT_STRIP) {
     static Occ occ;
     const size_t smem = (size_t)kStripWarps * A->height * 32 * sizeof(Acc);

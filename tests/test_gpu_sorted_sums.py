@@ -118,3 +118,11 @@ def test_units_that_pay_for_the_mapping(b, dtype, mean, spread, height, few, eno
     y, alg1, exact = products(b, dtype, mean, spread, height, enough)
     assert not torch.equal(y, alg1)
     assert error(y, exact) <= 1.03 * error(alg1, exact)  # as above, from fewer rows
+
+
+# FP64 rows of up to 10 on average take two sums a lane, longer ones four; rows of 0 to twice the mean are the worst
+@pytest.mark.parametrize("mean,spread,height", [(3, 0.0, 4), (10, 0.0, 16), (10, 1.0, 2), (10, 1.0, 8), (11, 0.0, 4)])
+def test_no_less_exact_either_side_of_two_sums(b, mean, spread, height):
+    y, alg1, exact = products(b, 0, mean, spread, height, 110)
+    assert not torch.equal(y, alg1)
+    assert error(y, exact) <= 1.01 * error(alg1, exact)
